@@ -19,7 +19,7 @@ HOST_LIB = os.path.join(HERE, "librox_fadd_host.so")
 SOURCES = ["rox_api.cu", "rox_params.cu", "rox_geometry.cu", "rox_voigt.cu", "rox_static.cu", "rox_cia.cu", "rox_probe.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
+FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + BUILD]
 
 
 def check_tables():
@@ -28,6 +28,12 @@ def check_tables():
     with open(os.path.join(CSRC, "rox_faddeeva_tables.h")) as f:
         if f.read().strip() != gen.strip():
             raise RuntimeError("rox_faddeeva_tables.h is stale: rerun gen_faddeeva_tables.py")
+
+
+def make_interp_table():
+    """The span interpolation table (rox_interp_table.h), into the build folder."""
+    with open(os.path.join(BUILD, "rox_interp_table.h"), "w") as f:
+        subprocess.run([sys.executable, os.path.join(CSRC, "gen_interp_table.py")], check=True, stdout=f)
 
 
 def _run(cmd):
@@ -47,6 +53,7 @@ def build_host_lib():
 def build(verbose=False):
     check_tables()
     os.makedirs(BUILD, exist_ok=True)
+    make_interp_table()
     objs = []
     cmds = []
     for src in SOURCES:

@@ -1,6 +1,7 @@
 // C ABI of librox (include/rox.h): argument checks, workspace layout, launch order.
 // Everything after the checks is enqueued on the caller's stream; nothing here
 // allocates device memory or synchronises, except rox_ws_status.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -34,6 +35,7 @@ size_t rox_sort_ws_bytes(long long n);
 cudaError_t rox_launch_sort(const rox_lines* in, const rox_lines_buf* out, int64_t* perm_out, void* ws,
                             cudaStream_t s);
 cudaError_t rox_launch_voigt(const RoxVoigtArgs& A, int n_blocks, bool nodes, int extras, int warps, cudaStream_t s);
+cudaError_t rox_launch_moments(const RoxVoigtArgs& A, int extras, cudaStream_t s);
 cudaError_t rox_launch_node_windows(const double* nu0, long long n_lines, const double* nodes, long long n,
                                     double cutoff, int32_t* jlo, int32_t* jhi, float4* geo,
                                     unsigned long long* evals, int32_t* unsorted, int32_t unsorted_value,
@@ -133,7 +135,24 @@ int check_cutoff(double cutoff, const rox_grid* g) {
   return ROX_OK;
 }
 
+// grid steps that every line's window surely reaches on each side of its centre
+int32_t cutoff_steps(double cutoff, double dnu) { return (int32_t)std::floor(cutoff / dnu) - 2; }
+
 long long n_tiles_of(long long n_grid) { return (n_grid + ROX_TILE - 1) / ROX_TILE; }
+
+// moment scratch: slots of 16 floats, and the cells' first lines
+struct RoxMoments {
+  float4* mom = nullptr;
+  int32_t* cstart = nullptr;
+  long long cap = 0;
+};
+RoxMoments moments_at(char* p, long long slots) {
+  RoxMoments m;
+  m.mom = (float4*)p;
+  m.cstart = (int32_t*)(p + rox_align256((size_t)slots * 64));
+  m.cap = slots;
+  return m;
+}
 
 struct WsLayout {
   RoxWsHeader* hdr;
@@ -159,6 +178,7 @@ struct WsLayout {
   size_t compact_tmp_bytes;
   float* broad_G;      // broadening descriptions only: [n_temps][n_lines] broadeners' sums, [n_lines]
   float* broad_N;      //   natural widths
+  RoxMoments mom;      // uniform grids: moments of ROX_MOM_JOBS jobs' cells
   float4* rec;         // one temperature on a uniform grid: per line 3 float4 of per-line constants
   size_t bytes;
 };
@@ -184,7 +204,7 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
   off += rox_align256((size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 4);
   w.tail_cap = nt < tail_max ? nt : tail_max;
   w.tail_part = (float*)(base + off);
-  w.tail_cnt = (int32_t*)(base + off + rox_align256((size_t)w.tail_cap * ROX_PARTS * ROX_SPAN * sizeof(float)));
+  w.tail_cnt = (int32_t*)(base + off + rox_tail_part_bytes(w.tail_cap));
   off += rox_tail_bytes(w.tail_cap);
   w.node_d = nullptr;
   w.span_base = nullptr;
@@ -234,6 +254,11 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
     off += rox_align256((size_t)n_temps * nl * 4);
     w.broad_N = (float*)(base + off);
     off += rox_align256(nl * 4);
+  }
+  if (!nodes) {
+    const long long slots = (pre ? ROX_MOM_JOBS : 1) * rox_job_slots(nt);
+    w.mom = moments_at(base + off, slots);
+    off += rox_mom_bytes(slots);
   }
   w.rec = nullptr;
   if (pre && n_temps == 1 && !nodes && n_bins == 0 && !broad) {
@@ -334,25 +359,47 @@ int voigt_grid(int* out, const rox_launch_config& cfg, bool nodes = false, bool 
   return ROX_OK;
 }
 
+// Moment cells of a job: every cell that can hold a line reaching one of its spans, at most
+// ROX_CELL_EXT beyond them on each side. Cutoffs of fewer than two spans leave no cell far
+// enough from a span to be taken whole. Returns the job's slots (a multiple of 4), which depend on the
+// job alone, so that its result does not depend on what it is launched with.
+long long job_cells(RoxJobDev* J, int32_t c_steps) {
+  J->n_cells = 0;
+  if (c_steps < 2 * ROX_SPAN) return 0;
+  const long long ext = std::min<long long>((c_steps + 4) / ROX_CELL + 1, ROX_CELL_EXT);
+  J->c_first = J->span_first * ROX_CELLS_PER_SPAN - (int32_t)ext;
+  J->n_cells = J->n_spans * ROX_CELLS_PER_SPAN + 2 * (int32_t)ext;
+  return ((long long)J->n_cells + 1 + 3) & ~3LL;
+}
+
 // Voigt launches over the jobs, at most ROX_MAX_JOBS per launch; the work counter is reset
 // before each launch (the evaluation count keeps adding up). The last items of each launch,
 // up to tail_cap and half a round of the launch's warps, are split into their parts.
 int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* jobs, int n_jobs, RoxWsHeader* hdr,
-                      float* tail_part, int32_t* tail_cnt, long long tail_cap, int nblocks, cudaStream_t s,
-                      const rox_launch_config& cfg, bool nodes = false, int extras = 0) {
+                      float* tail_part, int32_t* tail_cnt, long long tail_cap, const RoxMoments& mom, int nblocks,
+                      cudaStream_t s, const rox_launch_config& cfg, bool nodes = false, int extras = 0) {
   static thread_local RoxVoigtArgs A;   // ~30 KB of per-job parameters, passed by value
   A.hdr = hdr;
   A.tail_part = tail_part;
   A.tail_cnt = tail_cnt;
   for (int l = 0; l < n_lists; l++) A.list[l] = lists[l];
-  for (int j0 = 0; j0 < n_jobs; j0 += ROX_MAX_JOBS) {
-    const int nj = (n_jobs - j0) < ROX_MAX_JOBS ? (n_jobs - j0) : ROX_MAX_JOBS;
+  A.mom = mom.mom;
+  A.cstart = mom.cstart;
+  for (int j0 = 0, nj = 0; j0 < n_jobs; j0 += nj) {
     int items = 0;
-    for (int k = 0; k < nj; k++) {
-      A.job[k] = jobs[j0 + k];
-      items += A.job[k].n_spans;
-      A.item_end[k] = items;
+    long long slots = 0;
+    for (nj = 0; nj < ROX_MAX_JOBS && j0 + nj < n_jobs; nj++) {
+      RoxJobDev J = jobs[j0 + nj];
+      const long long need = mom.cap ? job_cells(&J, lists[J.list].c_steps) : 0;
+      if (nj > 0 && slots + need > mom.cap) break;
+      if (need > mom.cap) J.n_cells = 0;      // (no caller gives a job less than its slots)
+      J.mom_off = (int32_t)slots;
+      if (J.n_cells > 0) slots += need;
+      A.job[nj] = J;
+      items += J.n_spans;
+      A.item_end[nj] = items;
     }
+    A.n_slots = (int32_t)slots;
     const int blocks = items < nblocks ? items : nblocks;
     // whole items in complete rounds of the launch's warps, then at least one round of items in
     // parts, so the launch ends in pieces of 1/ROX_PARTS of an item
@@ -369,6 +416,7 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
     if (split > 0 && (rc = cuda_check(cudaMemsetAsync(tail_cnt, 0, (size_t)split * 4, s), "memset"))) return rc;
     if (j0 == 0 && g_prof_start && (rc = cuda_check(cudaEventRecord(g_prof_start, s), "cudaEventRecord"))) return rc;
     if (items == 0) continue;
+    if ((rc = cuda_check(rox_launch_moments(A, extras, s), "moments kernel"))) return rc;
     if ((rc = cuda_check(rox_launch_voigt(A, blocks, nodes, extras, cfg.warps_per_cta, s), "voigt kernel"))) return rc;
   }
   if (g_prof_stop) return cuda_check(cudaEventRecord(g_prof_stop, s), "cudaEventRecord");
@@ -591,6 +639,7 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
   L0.idx = nullptr;
   L0.inv_dnu_f = on_nodes ? 0.0f : (float)(1.0 / grid->dnu);
   L0.rec = pre ? w.rec : nullptr;
+  L0.c_steps = on_nodes ? 0 : cutoff_steps(cutoff, grid->dnu);
   std::vector<RoxJobDev> jobs(n_pt);
   for (int k = 0; k < n_pt; k++) {
     RoxJobDev& J = jobs[k];
@@ -628,14 +677,14 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
           jg.back().list = tidx[k] - g0;
         }
       if ((rc = launch_voigt_jobs(Ls, ng, jg.data(), (int)jg.size(), w.hdr, w.tail_part, w.tail_cnt, w.tail_cap,
-                                  nblocks, s, cfg, false, ROX_VX_INDEX)))
+                                  w.mom, nblocks, s, cfg, false, ROX_VX_INDEX)))
         return rc;
     }
     return ok();
   }
   if (pre && (rc = cuda_check(rox_launch_line_params(L0, jobs[0], w.rec, s), "line parameter kernel"))) return rc;
   const int extras = br ? ROX_VX_BROAD : (pre ? ROX_VX_PRE : 0);
-  if ((rc = launch_voigt_jobs(&L0, 1, jobs.data(), n_pt, w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, nblocks, s,
+  if ((rc = launch_voigt_jobs(&L0, 1, jobs.data(), n_pt, w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, w.mom, nblocks, s,
                               cfg, on_nodes, extras)))
     return rc;
   return ok();
@@ -864,26 +913,32 @@ struct JobsTail {
   float* part;
   int32_t* cnt;
   long long cap;
+  RoxMoments mom;
 };
 size_t jobs_layout(const rox_job* jobs, int n_jobs, void* ws, double** S64, float** S32, JobsTail* tail) {
   size_t off = ROX_WS_HEADER_BYTES;
-  long long spans = 0;
+  long long spans = 0, slots = 0;
   for (int k = 0; k < n_jobs; k++) {
     const size_t c = (size_t)(jobs[k].line_count > 0 ? jobs[k].line_count : 1);
     if (S64) S64[k] = (double*)((char*)ws + off);
     off += rox_align256(c * 8);
     if (S32) S32[k] = (float*)((char*)ws + off);
     off += rox_align256(c * 4);
-    if (jobs[k].n > 0 && jobs[k].first >= 0)
-      spans += (jobs[k].first + jobs[k].n - 1) / ROX_SPAN - jobs[k].first / ROX_SPAN + 1;
+    if (jobs[k].n > 0 && jobs[k].first >= 0) {
+      const long long ns = (jobs[k].first + jobs[k].n - 1) / ROX_SPAN - jobs[k].first / ROX_SPAN + 1;
+      spans += ns;
+      slots += rox_job_slots(ns);
+    }
   }
   const long long cap = spans < ROX_TAIL_ITEMS_MAX ? spans : ROX_TAIL_ITEMS_MAX;
   if (tail) {
     tail->cap = cap;
     tail->part = (float*)((char*)ws + off);
-    tail->cnt = (int32_t*)((char*)ws + off + rox_align256((size_t)cap * ROX_PARTS * ROX_SPAN * sizeof(float)));
+    tail->cnt = (int32_t*)((char*)ws + off + rox_tail_part_bytes(cap));
   }
   off += rox_tail_bytes(cap);
+  if (tail) tail->mom = moments_at((char*)ws + off, slots);
+  off += rox_mom_bytes(slots);
   return off;
 }
 }  // namespace
@@ -983,6 +1038,7 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     L[l].width_f16 = P.lines.width_dtype == ROX_WIDTH_F16;
     L[l].inv_dnu_f = (float)(1.0 / P.lattice.dnu);
     L[l].rec = nullptr;
+    L[l].c_steps = cutoff_steps(P.cutoff, P.lattice.dnu);
   }
   std::vector<RoxJobDev> J(n_jobs);
   for (int k = 0; k < n_jobs; k++) {
@@ -1004,7 +1060,8 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     d.flags = j.flags;
     d.t_row = 0;
   }
-  if ((rc = launch_voigt_jobs(L, n_lists, J.data(), n_jobs, hdr, tail.part, tail.cnt, tail.cap, nblocks, s, cfg)))
+  if ((rc = launch_voigt_jobs(L, n_lists, J.data(), n_jobs, hdr, tail.part, tail.cnt, tail.cap, tail.mom, nblocks, s,
+                              cfg)))
     return rc;
   return ok();
 }

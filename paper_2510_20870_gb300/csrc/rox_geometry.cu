@@ -57,13 +57,18 @@ __global__ void k_windows(const double* __restrict__ nu0s, long long n_lines, do
     double k0 = floor(u);
     double f = u - k0;
     if (f >= 1.0) { k0 += 1.0; f -= 1.0; }
-    if (jh < jl) { k0 = 0.0; f = 0.0; }       // touches no grid point: never evaluated
+    // the geometry record's centre never decreases along the list: a line beyond reach of the grid
+    // (never evaluated) is put just beyond the centres that reach it
+    const double far = c_idx + 8.0;
+    const double kg = fmin(fmax(k0, -far), (double)n_grid + far);
+    const double fg = kg == k0 ? f : 0.0;
+    if (jh < jl) { k0 = 0.0; f = 0.0; }       // touches no grid point
     if (jlo_out) jlo_out[i] = (int32_t)jl;
     if (jhi_out) jhi_out[i] = (int32_t)jh;
     if (k0_out) k0_out[i] = (int32_t)k0;
     if (f_out) f_out[i] = (float)f;
     if (geo_out)
-      geo_out[i] = make_float4((float)k0, (float)(f * dnu), __int_as_float((int)jl), __int_as_float((int)jh));
+      geo_out[i] = make_float4((float)rint(kg), (float)(fg * dnu), __int_as_float((int)jl), __int_as_float((int)jh));
   }
   if (evals_out) {
 #pragma unroll

@@ -44,7 +44,7 @@ struct RoxWsHeader {
 
 // Voigt launch: up to ROX_MAX_LISTS prepared line lists and ROX_MAX_JOBS jobs, each job one
 // output window on its list's lattice at one (P,T) point; work items are (job, span) pairs.
-#define ROX_MAX_JOBS 320
+#define ROX_MAX_JOBS 256
 #define ROX_MAX_LISTS 8
 
 struct RoxListDev {
@@ -77,7 +77,20 @@ struct RoxListDev {
   float nu_min_f;
   int32_t width_f16;
   float inv_dnu_f;            // 1/dnu (uniform grid; 0 on nodes)
+  int32_t c_steps;            // floor(cutoff / dnu) - 2: points every line's window surely reaches on each side
 };
+
+// Multipole cells (uniform grids): ROX_CELL grid steps of line centres, lines with k0 in
+// [ROX_CELL c, ROX_CELL (c + 1)). Per job and cell 16 floats: ROX_MOMENTS coefficients of the sum
+// of the cell's far forms in powers of 1/(offset from the cell's centre) (rox_voigt.cu, k_moments),
+// the largest modulus of a pole and the largest slow-zone half-width of its lines (cm^-1).
+#define ROX_CELL_LOG2 6
+#define ROX_CELL (1 << ROX_CELL_LOG2)
+#define ROX_MOMENTS 14
+#define ROX_CELL_EXT 512           // cells kept on each side of a job's spans (further lines: one by one)
+#define ROX_MOM_JOBS 16            // jobs whose cells the workspace of a cross-section call holds at a time
+#define ROX_CELL_BYTES 68          // 16 floats and the cell's first line (int32)
+#define ROX_CELLS_PER_SPAN (ROX_SPAN / ROX_CELL)
 
 // Lorentz-width description of rox_broadening in kernel parameter form
 struct RoxBroadDev {
@@ -115,6 +128,9 @@ struct RoxJobDev {
   float l2_ratio;   // log2(T_ref / T)           -> (T_ref/T)^n_T = exp2(n_T * l2_ratio)
   uint32_t flags;   // ROX_ACCUMULATE, ROX_KAHAN
   int32_t t_row;    // broadened lists: the job's temperature row of the list's gLT
+  int32_t mom_off;  // the job's first slot in RoxVoigtArgs::mom and cstart (a multiple of 4)
+  int32_t c_first;  // the cell of that slot
+  int32_t n_cells;  // cells with moments (slot n_cells holds only the first line beyond them); 0: none
 };
 
 // Every span's lines are summed as ROX_PARTS consecutive parts (batch-aligned), each from
@@ -127,12 +143,19 @@ struct RoxJobDev {
 // (at most ROX_TAIL_ITEMS_MAX items, the size of the workspace's tail scratch).
 #define ROX_PARTS 16
 #define ROX_TAIL_ITEMS_MAX 8192
+// A part's sum: its ROX_SPAN points, then its values at the span's ROX_NODES Chebyshev points
+// (the lines that are smooth on the span, rox_voigt.cu)
+#define ROX_NODES 32
+#define ROX_PART_FLOATS (ROX_SPAN + ROX_NODES)
 
 struct RoxVoigtArgs {
   RoxWsHeader* hdr;
-  float* tail_part;                 // [n_items - n_whole][ROX_PARTS][ROX_SPAN] part sums
+  float* tail_part;                 // [n_items - n_whole][ROX_PARTS][ROX_PART_FLOATS] part sums
   int32_t* tail_cnt;                // [n_items - n_whole] parts finished (zeroed per launch)
+  float4* mom;                      // [slots][4] moments of the jobs' cells
+  int32_t* cstart;                  // [slots] first line (position) of each cell
   int32_t n_jobs;
+  int32_t n_slots;                  // slots over all jobs (0: no moments in this launch)
   int32_t n_items;                  // items (spans over all jobs); the last n_items - n_whole split
   int32_t n_whole;
   int32_t n_queue;                  // queue entries: n_whole + (n_items - n_whole) * ROX_PARTS
@@ -169,7 +192,15 @@ struct RoxStrengthJobs {
 static_assert(sizeof(RoxStrengthJobs) < 32000, "kernel parameter space");
 
 static inline size_t rox_align256(size_t b) { return (b + 255) & ~(size_t)255; }
-// tail scratch of a workspace: `cap` items x ROX_PARTS x ROX_SPAN floats, then cap counters
-static inline size_t rox_tail_bytes(long long cap) {
-  return rox_align256((size_t)cap * ROX_PARTS * ROX_SPAN * sizeof(float)) + rox_align256((size_t)cap * 4);
+// moment slots of a job over n_spans spans, and the bytes of a number of slots
+static inline long long rox_job_slots(long long n_spans) {
+  return n_spans * ROX_CELLS_PER_SPAN + 2 * ROX_CELL_EXT + 4;
 }
+static inline size_t rox_mom_bytes(long long slots) {
+  return rox_align256((size_t)slots * 64) + rox_align256((size_t)slots * 4);
+}
+// tail scratch of a workspace: `cap` items x ROX_PARTS x ROX_PART_FLOATS floats, then cap counters
+static inline size_t rox_tail_part_bytes(long long cap) {
+  return rox_align256((size_t)cap * ROX_PARTS * ROX_PART_FLOATS * sizeof(float));
+}
+static inline size_t rox_tail_bytes(long long cap) { return rox_tail_part_bytes(cap) + rox_align256((size_t)cap * 4); }

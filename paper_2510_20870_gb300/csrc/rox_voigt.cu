@@ -31,6 +31,7 @@
 #include <cuda_fp16.h>
 #include "rox_internal.cuh"
 #include "rox_faddeeva.cuh"
+#include "rox_interp_table.h"   // generated by gen_interp_table.py
 
 namespace {
 
@@ -201,6 +202,70 @@ __device__ __forceinline__ void cover_pair(const PairTab& P, int k, float lanef,
   for (int m = 0; m < ROX_K; m++)
     acc[m] = pair_add<CLAMP, false>(pos<NU>(m, X0, c.e0, c.f0, D, dnu_f), pos<NU>(m, X1, c.e1, c.f1, D, dnu_f), c,
                                     true, true, acc[m]);
+}
+
+// Pass 1 for pair k of lines that are smooth on the span: their sum at this lane's Chebyshev
+// point of the span (tau: its position in grid steps, or on nodes in cm^-1, from the span's first
+// point). One step in place of ROX_K.
+template <bool NU>
+__device__ __forceinline__ float smooth_pair(const PairTab& P, int k, float tau, float dnu_f, float nacc) {
+  const PairC c = pair_consts<false>(P, k);
+  float x0, x1;
+  if constexpr (NU) {
+    x0 = (tau - c.e0) - c.f0;
+    x1 = (tau - c.e1) - c.f1;
+  } else {
+    pair_x0<NU>(c, tau, dnu_f, x0, x1);
+  }
+  return pair_add<false, false>(x0, x1, c, true, true, nacc);
+}
+
+// Whether a line whose window covers the span and whose slow zone misses it is smooth there: its
+// far form at the span's 32 Chebyshev points then gives it at every point of the span by
+// polynomial interpolation. D: |offset| of the span's centre from the line, h: the span's
+// half-width. The far form's poles X^2 = -A +- sqrt(-B) have real parts of at most
+// Rp = sqrt(max(0, -A) + sqrt|B|); with none within 1.25 h of the centre the error of degree 31 is
+// below 1e-7 (a Bernstein ellipse of parameter 2: 2^-32 times 128 / (1.25^2 - 1)).
+#define ROX_SMOOTH_R 1.25f
+__device__ __forceinline__ float smooth_dmin(float A, float B, float h) {
+  const float b = fabsf(B) + 1e-30f;
+  const float rp2 = fmaxf(0.0f, -A) + b * rox_rsqrt(b) + 1e-30f;
+  return fmaf(ROX_SMOOTH_R, h, rp2 * rox_rsqrt(rp2));
+}
+
+// Adds to stot (the span's points) the polynomial through the values v at the span's 32 Chebyshev
+// points (lane k holds point k). Uniform grid: the cardinal functions are a table; nodes: the
+// barycentric quotient, evaluated at each node's position.
+template <bool NU>
+__device__ __forceinline__ void interp_span(float v, int lane, const float2* D, float half, float* stot) {
+  if constexpr (NU) {
+    const float inv = half > 0.f ? 1.0f / half : 0.f;
+    for (int m = 0; m < ROX_K; m++) {
+      const float x = fmaf(D[32 * m].x, inv, -1.0f);
+      float num = 0.f, den = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < ROX_NODES; k++) {
+        float d = x - rox_cheb_x[k];
+        d = d == 0.f ? 1e-20f : d;
+        const float q = rox_cheb_w[k] * rox_rcp(d);
+        num = fmaf(q, __shfl_sync(0xffffffffu, v, k), num);
+        den += q;
+      }
+      stot[32 * m + lane] += num / den;
+    }
+  } else {
+    float r[ROX_K];
+#pragma unroll
+    for (int m = 0; m < ROX_K; m++) r[m] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < ROX_NODES; k++) {
+      const float vk = __shfl_sync(0xffffffffu, v, k);
+#pragma unroll
+      for (int m = 0; m < ROX_K; m++) r[m] = fmaf(__ldg(&rox_interp[m][k][lane]), vk, r[m]);
+    }
+#pragma unroll
+    for (int m = 0; m < ROX_K; m++) stot[32 * m + lane] += r[m];
+  }
 }
 
 // Pass 1 for pair k of which at least one line is cut by a window edge: the sub-spans outside
@@ -395,7 +460,141 @@ __global__ void k_line_params(const RoxListDev L, const RoxJobDev J, float4* rec
     zone_bounds(g, k.hz, L.inv_dnu_f, zlo, zhi);
     rec[3 * i] = make_float4(k.A, k.B, k.P, k.Q);
     rec[3 * i + 1] = make_float4(k.tz, k.iGs, k.y, k.pc);
-    rec[3 * i + 2] = make_float4(k.cf, __int_as_float(zlo), __int_as_float(zhi), 0.0f);
+    rec[3 * i + 2] = make_float4(k.cf, __int_as_float(zlo), __int_as_float(zhi),
+                                 smooth_dmin(k.A, k.B, 0.5f * (ROX_SPAN - 1) * L.dnu_f));
+  }
+}
+
+// k_moments: the far forms of a cell's lines summed into one multipole expansion. With the cell's
+// centre as origin and its half-width as unit, a line at d has f(Y) = (P t + Q)/(t^2 + B),
+// t = (Y - d)^2 + A, a rational function whose expansion f = sum_l m_l / Y^(l+2) follows from
+// f (Y^4 + d3 Y^3 + d2 Y^2 + d1 Y + d0) = P Y^2 - 2 P d Y + P (d^2 + A) + Q by a four-term
+// recurrence, exact for every order. One warp takes four consecutive cells of one job, finds the
+// first by a 32-way search of the sorted centres and walks its lines 32 at a time; lanes' sums
+// are added by a fixed tree. Truncated after ROX_MOMENTS terms the expansion errs by
+// (r^14)(15 - 14 r) of a line's value, r = (half-width + pole modulus)/|Y|: k_voigt takes a cell only
+// where r <= 1/4 (5e-8).
+__device__ __forceinline__ float cell_k0(const RoxListDev& L, long long pos) {
+  return L.geo[L.idx ? (long long)L.idx[pos] : pos].x;
+}
+template <int X>
+__global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoigtArgs A) {
+  constexpr bool IDX = (X & ROX_VX_INDEX) != 0;
+  constexpr bool BRD = (X & ROX_VX_BROAD) != 0;
+  constexpr bool PRE = (X & ROX_VX_PRE) != 0;
+  if (*(volatile int32_t*)&A.hdr->status != ROX_OK) return;
+  const int lane = threadIdx.x & 31;
+  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+  for (int task = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); 4 * task < A.n_slots; task += nw) {
+    int k = 0, k_hi = A.n_jobs - 1;            // last job with mom_off <= 4 task
+    while (k < k_hi) {
+      const int mid = (k + k_hi + 1) >> 1;
+      if (A.job[mid].mom_off <= 4 * task) k = mid; else k_hi = mid - 1;
+    }
+    const RoxJobDev& J = A.job[k];
+    const RoxListDev& L = A.list[J.list];
+    if (J.n_cells <= 0 || *L.status != ROX_OK) continue;
+    const int s0 = 4 * task - J.mom_off;
+    const long long p0 = max(L.span_lo[J.span_first], J.l0);
+    const long long p1 = min(L.span_hi[J.span_first + J.n_spans - 1], J.l1);
+    const float dnu_f = L.dnu_f, margin_cm = fast_margin(dnu_f);
+    const float half = 0.5f * ROX_CELL * dnu_f, ih = 1.0f / half, ih2 = ih * ih;
+    const float* S_row = J.S32 - J.l0;
+    // first line of cell s0: p0 plus the lines before it
+    long long lo = p0, len = max(0LL, p1 - p0);
+    const float first = (float)(ROX_CELL * (J.c_first + s0));
+    while (len > 0) {
+      const long long step = (len + 31) >> 5, off = (long long)lane * step;
+      const bool less = off < len && cell_k0(L, lo + off) < first;
+      const int c = __popc(__ballot_sync(0xffffffffu, less));
+      if (c == 0) break;
+      const long long nlo = lo + (c - 1) * step + 1;
+      len = min(step - 1, lo + len - nlo);
+      lo = nlo;
+    }
+    for (int s = s0; s < s0 + 4 && s <= J.n_cells; s++) {
+      const int cell = J.c_first + s;
+      const float centre = (float)(ROX_CELL * cell) + 0.5f * ROX_CELL, end = (float)(ROX_CELL * (cell + 1));
+      if (lane == 0) A.cstart[J.mom_off + s] = (int32_t)lo;
+      if (s == J.n_cells) break;               // the end of the last cell
+      float M[ROX_MOMENTS], pm = 0.f, zm = 0.f;
+#pragma unroll
+      for (int l = 0; l < ROX_MOMENTS; l++) M[l] = 0.f;
+      for (;;) {
+        const long long pos = lo + lane;
+        bool in = pos < p1;
+        long long li = 0;
+        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in) {
+          li = IDX ? (long long)L.idx[pos] : pos;
+          g = L.geo[li];
+          in = g.x < end;
+        }
+        const int nb = __popc(__ballot_sync(0xffffffffu, in));
+        if (in) {
+          float a, b, p, q, hz;
+          if constexpr (PRE) {
+            const float4 r0 = L.rec[3 * li];
+            a = r0.x;
+            b = r0.y;
+            p = r0.z;
+            q = r0.w;
+            const float z2 = fmaxf(L.rec[3 * li + 1].x - a, 0.f) + 1e-30f;   // t_z = hz^2 + A
+            hz = z2 * rox_rsqrt(z2) * 1.001f;
+          } else {
+            float gref, nt;
+            load_widths<BRD>(J, L, L.width_f16, li, gref, nt);
+            const LineK kc = line_consts<BRD>(L.nu_min_f + fmaf(g.x, dnu_f, g.y), S_row[li], gref, nt, J, margin_cm, false);
+            a = kc.A;
+            b = kc.B;
+            p = kc.P;
+            q = kc.Q;
+            hz = kc.hz * 1.001f;
+          }
+          const float bm = fabsf(b) + 1e-30f;
+          const float r2 = fabsf(a) + bm * rox_rsqrt(bm) + 1e-30f;      // |pole|^2 at most
+          pm = fmaxf(pm, r2 * rox_rsqrt(r2) * 1.001f);
+          zm = fmaxf(zm, hz);
+          const float d = fmaf(g.y, ih, (g.x - centre) * (2.0f / ROX_CELL));
+          const float pu = p * ih2, qu = q * (ih2 * ih2), bu = b * (ih2 * ih2);
+          const float e = fmaf(d, d, a * ih2);
+          const float d3 = 4.0f * d, d2 = -fmaf(d3, d, 2.0f * e), d1 = d3 * e, d0 = -fmaf(e, e, bu);
+          float m0 = pu, m1 = 2.0f * pu * d;
+          float m2 = fmaf(d3, m1, fmaf(d2, m0, fmaf(pu, e, qu)));
+          float m3 = fmaf(d3, m2, fmaf(d2, m1, d1 * m0));
+          M[0] += m0;
+          M[1] += m1;
+          M[2] += m2;
+          M[3] += m3;
+#pragma unroll
+          for (int l = 4; l < ROX_MOMENTS; l++) {
+            const float m = fmaf(d3, m3, fmaf(d2, m2, fmaf(d1, m1, d0 * m0)));
+            M[l] += m;
+            m0 = m1;
+            m1 = m2;
+            m2 = m3;
+            m3 = m;
+          }
+        }
+        lo += nb;
+        if (nb < 32) break;
+      }
+      float v = 0.f;
+#pragma unroll
+      for (int l = 0; l < ROX_MOMENTS; l++) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) M[l] += __shfl_xor_sync(0xffffffffu, M[l], o);
+        v = lane == l ? M[l] : v;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
+      }
+      if (!(pm <= 64.0f * half)) pm = 1e30f;   // powers of the poles beyond FP32's range: not to be used
+      v = lane == ROX_MOMENTS ? pm : (lane == ROX_MOMENTS + 1 ? zm : v);
+      if (lane < 16) reinterpret_cast<float*>(A.mom + 4 * (size_t)(J.mom_off + s))[lane] = v;
+    }
   }
 }
 
@@ -432,6 +631,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
   PairTab& PT = s_pairs[w];
   LineTab& LT = s_lines[w];
   const float lanef = (float)lane;
+  const float cheb = rox_cheb_x[lane];
   float* zacc = s_zacc[w];
   float* stot = s_tot[w];
   float2* Drow = NU ? s_nodes + w * ROX_SPAN : nullptr;   // this span's node offsets
@@ -471,6 +671,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
     const float margin_cm = NU ? 0.0f : fast_margin(dnu_f);
     const int Aw = span * ROX_SPAN;
     const int Bw = Aw + ROX_SPAN - 1;
+    const int Bg = (int)min((long long)Bw, Lst.n_lattice - 1);   // the span's last point on the grid
     if (*Lst.status != ROX_OK) continue;           // list not prepared from sorted lines
     float bh = 0.f, bl = 0.f, Ws = 0.f;             // span's first node; offset of its last node
     if constexpr (NU) {
@@ -482,62 +683,109 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
       __syncwarp();
       Ws = Drow[ROX_SPAN - 1].x;
     }
-    const long long lo = max(Lst.span_lo[span], J.l0), hi = min(Lst.span_hi[span], J.l1);
-    const long long wlo = J.first > Aw ? J.first : Aw;             // evaluated points of this span
-    const long long whi = (J.first + J.n - 1) < Bw ? (J.first + J.n - 1) : Bw;
+    const float half = NU ? 0.5f * Ws : 0.5f * (ROX_SPAN - 1) * dnu_f;
+    const float tau = NU ? fmaf(cheb, half, half) : fmaf(cheb, 0.5f * (ROX_SPAN - 1), 0.5f * (ROX_SPAN - 1));
+    float ntot = 0.f;   // whole items: this lane's Chebyshev point, over the parts
+    const int lo = (int)max(Lst.span_lo[span], J.l0), hi = (int)min(Lst.span_hi[span], J.l1);   // at most 2e9 lines
+    const int wlo = (int)max(J.first, (long long)Aw);              // evaluated points of this span
+    const int whi = (int)min(J.first + J.n - 1, (long long)Bw);
     const double smax = __longlong_as_double((long long)*J.smax_bits);
     const int e = smax > 0.0 ? ilogb(smax) : 0;     // S32 holds S * 2^-e (FP32)
     const float* S_row = J.S32 - J.l0;              // indexed by line number
 
-    const long long nbat = hi > lo ? (hi - lo + 31) >> 5 : 0;
+    // Cells taken through their moments: left of the span [cl0, cl1), right of it [cr0, cr1), all of
+    // whose lines cover the span, far enough for the expansion and for the lines' slow zones. Their
+    // lines [xa, xb) and [xc, xd) leave the span's list, whose other lines are visited one by one.
+    int cl0 = 0, cl1 = 0, cr0 = 0, cr1 = 0;
+    int xa = lo, xb = lo, xc = hi, xd = hi;
+    if (!NU && J.n_cells > 0 && hi > lo) {
+      const int c_end = J.c_first + J.n_cells;
+      cl0 = max((Bw - Lst.c_steps + ROX_CELL - 1) >> ROX_CELL_LOG2, J.c_first);
+      cr1 = min((Aw + Lst.c_steps) >> ROX_CELL_LOG2, c_end);
+      float pm = 0.f, zm = 0.f;
+      for (int c = cl0 + lane; c < cr1; c += 32) {
+        const float4 v = A.mom[4 * (size_t)(J.mom_off + c - J.c_first) + 3];
+        pm = fmaxf(pm, v.z);
+        zm = fmaxf(zm, v.w);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
+      }
+      const float far = fmaxf(4.0f * fmaf(pm, Lst.inv_dnu_f, 0.5f * ROX_CELL), fmaf(zm, Lst.inv_dnu_f, 0.5f * ROX_CELL + 2.0f));
+      // in cells from the span's centre, which lies half a step left of the start of cell cm
+      const int dc = (int)ceilf((fminf(far, 1e7f) + 0.5f * ROX_SPAN) * (1.0f / ROX_CELL) - 0.5f);
+      const int cm = (Aw + ROX_SPAN / 2) >> ROX_CELL_LOG2;
+      cl1 = min(cm - dc, c_end);
+      cr0 = max(cm + dc, J.c_first);
+      if (cl1 > cl0) {
+        xa = A.cstart[J.mom_off + cl0 - J.c_first];
+        xb = A.cstart[J.mom_off + cl1 - J.c_first];
+      } else {
+        cl1 = cl0;
+      }
+      if (cr1 > cr0) {
+        xc = A.cstart[J.mom_off + cr0 - J.c_first];
+        xd = A.cstart[J.mom_off + cr1 - J.c_first];
+      } else {
+        cr1 = cr0;
+      }
+      if (part <= 0 && lane == 0) evals += (unsigned long long)((long long)(xb - xa) + (xd - xc)) * (unsigned)(whi - wlo + 1);
+    }
+    const int n1 = xa - lo, n2 = n1 + (xc - xb), nn = n2 + max(hi - xd, 0);   // lines visited one by one
+    auto line_at = [&](int q) { return q < n1 ? lo + q : (q < n2 ? xb + (q - n1) : xd + (q - n2)); };
+    const int n_far = (cl1 - cl0) + (cr1 - cr0);
+
+    const int nbat = (nn + 31) >> 5;
     const int p_first = part < 0 ? 0 : part, p_last = part < 0 ? ROX_PARTS - 1 : part;
     for (int p = p_first; p <= p_last; p++) {
-      const long long plo = lo + 32 * ((nbat * p) / ROX_PARTS);
-      const long long phi = min(hi, lo + 32 * ((nbat * (p + 1)) / ROX_PARTS));
-      float acc[ROX_K], tot[ROX_K], cmp[ROX_K];
+      const int plo = 32 * ((nbat * p) / ROX_PARTS);
+      const int phi = min(nn, 32 * ((nbat * (p + 1)) / ROX_PARTS));
+      float acc[ROX_K], tot[ROX_K], cmp[ROX_K], nacc = 0.f, nsum = 0.f, ncmp = 0.f;
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) { acc[m] = 0.f; tot[m] = 0.f; cmp[m] = 0.f; zacc[32 * m + lane] = 0.f; }
 
       // stage batch 0; widths go through registers one batch ahead (with an index, the
       // positions' line numbers two batches ahead)
       float gref = 0.f, nt = 0.f;
-      long long li_n = 0;   // IDX: line number of this lane's position in the next batch
+      int li_n = 0;   // IDX: line number of this lane's position in the next batch
       if (plo + lane < phi) {
-        const long long li = IDX ? (long long)Lst.idx[plo + lane] : plo + lane;
+        const int li = IDX ? Lst.idx[line_at(plo + lane)] : line_at(plo + lane);
         cp_async16(&geo_st[0][lane], &Lst.geo[li]);
         if constexpr (PRE) {
 #pragma unroll
-          for (int c = 0; c < 3; c++) cp_async16(&rec_st[0][lane][c], &Lst.rec[3 * li + c]);
+          for (int c = 0; c < 3; c++) cp_async16(&rec_st[0][lane][c], &Lst.rec[3 * (long long)li + c]);
         } else {
           cp_async4(&S_st[0][lane], &S_row[li]);
           load_widths<BRD>(J, Lst, f16, li, gref, nt);
         }
       }
-      if (IDX && plo + 32 + lane < phi) li_n = Lst.idx[plo + 32 + lane];
+      if (IDX && plo + 32 + lane < phi) li_n = Lst.idx[line_at(plo + 32 + lane)];
       cp_async_commit();
       int nb = 0;
-      for (long long b0 = plo; b0 < phi; b0 += 32, nb++) {
-        const int cnt = (int)min((long long)32, phi - b0);
+      for (int b0 = plo; b0 < phi; b0 += 32, nb++) {
+        const int cnt = min(32, phi - b0);
         const int buf = nb & 1;
         float gref_n = 0.f, nt_n = 0.f;
         if (b0 + 32 + lane < phi) {
-          const long long li = IDX ? li_n : b0 + 32 + lane;
+          const int li = IDX ? li_n : line_at(b0 + 32 + lane);
           cp_async16(&geo_st[buf ^ 1][lane], &Lst.geo[li]);
           if constexpr (PRE) {
 #pragma unroll
-            for (int c = 0; c < 3; c++) cp_async16(&rec_st[buf ^ 1][lane][c], &Lst.rec[3 * li + c]);
+            for (int c = 0; c < 3; c++) cp_async16(&rec_st[buf ^ 1][lane][c], &Lst.rec[3 * (long long)li + c]);
           } else {
             cp_async4(&S_st[buf ^ 1][lane], &S_row[li]);
             load_widths<BRD>(J, Lst, f16, li, gref_n, nt_n);
           }
         }
-        if (IDX && b0 + 64 + lane < phi) li_n = Lst.idx[b0 + 64 + lane];
+        if (IDX && b0 + 64 + lane < phi) li_n = Lst.idx[line_at(b0 + 64 + lane)];
         cp_async_commit();
         cp_async_wait1();   // this lane's copies of the current batch have landed
 
         // ---- per-line constants (lane <-> line b0 + lane), written to the line's slot
         const bool live = lane < cnt;
-        bool covers = false, zoned = false;
+        bool covers = false, zoned = false, smooth = false;
         float ax = 0.f, ay = 0.f, vA = 1.f, vB = 0.f, vP = 0.f, vQ = 0.f, tz = 0.f, iGs = 1.f, yv = 0.f, pcv = 0.f;
         float cfv = 0.f;
         int jlo = 1, jhi = 0, zlo = 0, zhi = -1;
@@ -545,10 +793,11 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           const float4 g = geo_st[buf][lane];
           jlo = __float_as_int(g.z);
           jhi = __float_as_int(g.w);
-          const int ov = min(jhi, (int)whi) - max(jlo, (int)wlo) + 1;
+          const int ov = min(jhi, whi) - max(jlo, wlo) + 1;
           if (ov > 0) evals += (unsigned)ov;
-          covers = Aw >= jlo && Bw <= jhi;
+          covers = Aw >= jlo && Bg <= jhi;
           LineK kc;
+          float dmin;
           if constexpr (PRE) {
             // uniform grid, constants from k_line_params
             const float4 r0 = rec_st[buf][lane][0], r1 = rec_st[buf][lane][1], r2 = rec_st[buf][lane][2];
@@ -566,6 +815,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
             ax = (float)Aw - g.x;     // exact: both are integers below 2^24
             ay = -g.y;
             zoned = !(Bw < zlo || Aw > zhi);
+            dmin = r2.w;
           } else {
             const float Sp = S_st[buf][lane];
             float nu0f;   // line centre; its offset state {E, F} (uniform grid) or {c hi, c lo} (nodes)
@@ -592,7 +842,10 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
               zoned = !(Bw < zlo || Aw > zhi);
             }
             if (zoned) kc.cf = fmaf(kc.tz, kc.P, kc.Q) * rox_rcp(fmaf(kc.tz, kc.tz, kc.B));
+            dmin = smooth_dmin(kc.A, kc.B, half);
           }
+          const float D = NU ? half - ax - ay : fmaf(ax + 0.5f * (ROX_SPAN - 1), dnu_f, ay);
+          smooth = covers && !zoned && fabsf(D) >= dmin;
           vA = kc.A;
           vB = kc.B;
           vP = kc.P;
@@ -603,13 +856,15 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           pcv = kc.pc;
           cfv = kc.cf;
         }
-        const unsigned clean = __ballot_sync(0xffffffffu, live && covers && !zoned);
+        const unsigned msm = __ballot_sync(0xffffffffu, live && smooth);
+        const unsigned clean = __ballot_sync(0xffffffffu, live && covers && !zoned && !smooth);
         const unsigned czone = __ballot_sync(0xffffffffu, live && covers && zoned);
         const unsigned edge = __ballot_sync(0xffffffffu, live && !covers);
-        const int nclean = __popc(clean), ncov = nclean + __popc(czone);
+        const int nsm = __popc(msm), nclean = nsm + __popc(clean), ncov = nclean + __popc(czone);
         const unsigned below = (1u << lane) - 1u;
         const int slot = !covers ? ncov + __popc(edge & below)
-                                 : (zoned ? nclean + __popc(czone & below) : __popc(clean & below));
+                         : zoned ? nclean + __popc(czone & below)
+                         : smooth ? __popc(msm & below) : nsm + __popc(clean & below);
         const unsigned zslots = __reduce_or_sync(0xffffffffu, (live && zoned) ? (1u << slot) : 0u);
         if (live) {
           const int k = slot >> 1, h = slot & 1;
@@ -638,8 +893,9 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
         // are; pairs with a zoned line with t clamped to the zone boundary; then the rest (an odd
         // covering line, the window-edge lines) in pairs with window masks. Fixed orders: the sum
         // is reproducible.
-        const int kc = nclean >> 1, kz = ncov >> 1;
-        for (int k = 0; k < kc; k++) cover_pair<NU, false>(PT, k, lanef, dnu_f, D, acc);
+        const int ks = nsm >> 1, kc = nclean >> 1, kz = ncov >> 1;
+        for (int k = 0; k < ks; k++) nacc = smooth_pair<NU>(PT, k, tau, dnu_f, nacc);
+        for (int k = ks; k < kc; k++) cover_pair<NU, false>(PT, k, lanef, dnu_f, D, acc);
         for (int k = kc; k < kz; k++) cover_pair<NU, true>(PT, k, lanef, dnu_f, D, acc);
         for (int s2 = 2 * kz; s2 < cnt; s2 += 2) {
           if (s2 + 1 < cnt) edge_pair<NU>(PT, LT, s2 >> 1, Aw, lane, lanef, dnu_f, D, acc);
@@ -660,9 +916,27 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
             tot[m] = tk;
             acc[m] = 0.f;
           }
+          const float yn = nacc - ncmp;
+          const float tn = nsum + yn;
+          ncmp = ((tn - nsum) - yn) * kw;
+          nsum = tn;
+          nacc = 0.f;
         }
       }
       cp_async_wait0();
+      // this part's share of the far cells, at this lane's Chebyshev point
+      for (int c = n_far * p / ROX_PARTS; c < n_far * (p + 1) / ROX_PARTS; c++) {
+        const int cell = c < cl1 - cl0 ? cl0 + c : cr0 + (c - (cl1 - cl0));
+        const float4* mo = A.mom + 4 * (size_t)(J.mom_off + cell - J.c_first);
+        const float4 v0 = mo[0], v1 = mo[1], v2 = mo[2], v3 = mo[3];
+        const float y = ((float)(Aw - ROX_CELL * cell) + (tau - 0.5f * ROX_CELL)) * (2.0f / ROX_CELL);
+        const float z = rox_rcp(y);
+        float f = fmaf(z, v3.y, v3.x);
+        f = fmaf(z, fmaf(z, fmaf(z, fmaf(z, f, v2.w), v2.z), v2.y), v2.x);
+        f = fmaf(z, fmaf(z, fmaf(z, fmaf(z, f, v1.w), v1.z), v1.y), v1.x);
+        f = fmaf(z, fmaf(z, fmaf(z, fmaf(z, f, v0.w), v0.z), v0.y), v0.x);
+        nsum = fmaf(z * z, f, nsum);
+      }
       // fold in the pass-2 (near-centre) sums
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
@@ -672,10 +946,12 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
         tot[m] = tk;
       }
       if (part >= 0) {           // a split item: this part's sum goes to the tail scratch
-        float* dst = A.tail_part + ((size_t)(item - A.n_whole) * ROX_PARTS + p) * ROX_SPAN;
+        float* dst = A.tail_part + ((size_t)(item - A.n_whole) * ROX_PARTS + p) * ROX_PART_FLOATS;
 #pragma unroll
         for (int m = 0; m < ROX_K; m++) __stcg(&dst[32 * m + lane], tot[m]);
+        __stcg(&dst[ROX_SPAN + lane], nsum);
       } else {
+        ntot = p == 0 ? nsum : ntot + nsum;
 #pragma unroll
         for (int m = 0; m < ROX_K; m++) stot[32 * m + lane] = p == 0 ? tot[m] : stot[32 * m + lane] + tot[m];
       }
@@ -691,22 +967,27 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
       done = __shfl_sync(0xffffffffu, done, 0);
       if (done != ROX_PARTS - 1) continue;
       __threadfence();
-      const float* src = A.tail_part + (size_t)(item - A.n_whole) * ROX_PARTS * ROX_SPAN;
+      const float* src = A.tail_part + (size_t)(item - A.n_whole) * ROX_PARTS * ROX_PART_FLOATS;
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
         float v = __ldcg(&src[32 * m + lane]);
 #pragma unroll
-        for (int pp = 1; pp < ROX_PARTS; pp++) v = v + __ldcg(&src[pp * ROX_SPAN + 32 * m + lane]);
+        for (int pp = 1; pp < ROX_PARTS; pp++) v = v + __ldcg(&src[pp * ROX_PART_FLOATS + 32 * m + lane]);
         stot[32 * m + lane] = v;
       }
+      ntot = __ldcg(&src[ROX_SPAN + lane]);
+#pragma unroll
+      for (int pp = 1; pp < ROX_PARTS; pp++) ntot = ntot + __ldcg(&src[pp * ROX_PART_FLOATS + ROX_SPAN + lane]);
     }
+    // ---- the smooth lines' sum at the Chebyshev points, interpolated to the span's points
+    if (__any_sync(0xffffffffu, ntot != 0.f)) interp_span<NU>(ntot, lane, D, half, stot);
     // ---- write the span once (its part inside the job's window); a value beyond the FP32
     // range is written as it is and flagged (rox_ws_status: ROX_EOVERFLOW)
     float* out = J.sigma - J.first;
     bool bad = false;
 #pragma unroll
     for (int m = 0; m < ROX_K; m++) {
-      const long long j = (long long)Aw + 32 * m + lane;
+      const int j = Aw + 32 * m + lane;
       if (j >= wlo && j <= whi) {
         const float v = ldexpf(stot[32 * m + lane], e);
         const float o = (J.flags & ROX_ACCUMULATE) ? out[j] + v : v;
@@ -834,6 +1115,21 @@ cudaError_t rox_launch_voigt(const RoxVoigtArgs& A, int n_blocks, bool nodes, in
   if (warps == 4) return launch_w<4>(A, n_blocks, nodes, extras, s);
   if (warps == 8) return launch_w<8>(A, n_blocks, nodes, extras, s);
   return cudaErrorInvalidValue;
+}
+
+// moments of the cells of A's jobs (A.n_slots of them) ahead of the Voigt launch
+cudaError_t rox_launch_moments(const RoxVoigtArgs& A, int extras, cudaStream_t s) {
+  if (A.n_slots <= 0) return cudaSuccess;
+  long long b = ((A.n_slots + 3) / 4 + 7) / 8;
+  if (b > 152 * 16) b = 152 * 16;
+  switch (extras) {
+    case 0: k_moments<0><<<(int)b, 256, 0, s>>>(A); break;
+    case ROX_VX_INDEX: k_moments<ROX_VX_INDEX><<<(int)b, 256, 0, s>>>(A); break;
+    case ROX_VX_BROAD: k_moments<ROX_VX_BROAD><<<(int)b, 256, 0, s>>>(A); break;
+    case ROX_VX_PRE: k_moments<ROX_VX_PRE><<<(int)b, 256, 0, s>>>(A); break;
+    default: return cudaErrorNotSupported;
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t rox_voigt_blocks_per_sm(int* nb, bool nodes, bool pre, int warps) {
