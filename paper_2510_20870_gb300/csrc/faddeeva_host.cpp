@@ -16,3 +16,29 @@ extern "C" float rox_host_far_r2(float y) { return rox_far_coefs(y).r2; }
 extern "C" void rox_host_re_w_core(const float* x, const float* y, float* out, int64_t n) {
   for (int64_t i = 0; i < n; i++) out[i] = rox_re_w_core(&rox_daw_taylor[0][0], x[i], y[i]);
 }
+
+// the Voigt kernel's slow-zone forms, one point at a time
+extern "C" void rox_host_core_zone(const float* x, const float* y, float* out, int64_t n) {
+  for (int64_t i = 0; i < n; i++) {
+    const float y2 = y[i] * y[i], x2 = x[i] * x[i];
+    const bool small = y[i] < ROX_Y_CORE;
+    float c[16];
+    for (int k = 0; k < 16; k++) {
+      const float* r = rox_core_r[k];
+      c[k] = small ? rox_core_coef_r(y2, r[0], r[1], r[2], r[3]) : rox_core_coef(y[i], k);
+    }
+    const int np = y[i] < 1.0f ? 7 : 5;
+    const float U = x2 * (1.0f / (y2 + ROX_CORE_KAPPA));
+    float a = c[np], d = c[8 + np];
+    for (int k = np - 1; k >= 0; k--) a = fmaf(a, U, c[k]);
+    for (int k = np - 1; k >= 0; k--) d = fmaf(d, U, c[8 + k]);
+    const float r = a * rox_rcp(fmaf(d, U, 1.0f));
+    if (small) {
+      const float u2 = x2 * (4.0f * y2);
+      const float g = fmaf(fmaf(fmaf(u2, ROX_COS_C6, ROX_COS_C4), u2, -0.5f), u2, 1.0f);
+      out[i] = fmaf(rox_exp2(fmaf(x2, -ROX_LOG2E_F, y2 * ROX_LOG2E_F)), g, y[i] * r);
+    } else {
+      out[i] = r;
+    }
+  }
+}

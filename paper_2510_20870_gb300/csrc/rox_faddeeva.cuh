@@ -34,12 +34,17 @@
 #ifdef __CUDACC__
 #define ROX_FN __device__ __forceinline__
 #define ROX_TABLE static __constant__ const
+#define ROX_GTABLE static __device__ const   // read by different lanes at different places
+#define ROX_ALIGN16 __align__(16)
 #else
 #define ROX_FN static inline
 #define ROX_TABLE static const
+#define ROX_GTABLE static const
+#define ROX_ALIGN16
 #endif
 
 #include "rox_faddeeva_tables.h"
+#include "rox_core_tables.h"
 
 #define ROX_INV_SQRT_PI 0.564189583547756287f
 #define ROX_TWO_INV_SQRT_PI 1.128379167095512574f
@@ -278,6 +283,46 @@ ROX_FN float rox_re_w_cf5g(float x, float y) {
 ROX_FN float rox_re_w_core(const float* daw, float x, float y) {
   return y >= ROX_Y_WEIDEMAN ? rox_re_w_weideman(x, y) : rox_re_w_dawson(daw, x, y);
 }
+
+// ---- the Voigt kernel's slow zones: one rational form per line, by its y ----
+//
+// At fixed y, N(U)/D(U) with U = x^2 / (y^2 + 3/2) and coefficients from rox_core_tables.h:
+//   y < 0.1         Re w = e^{y^2 - x^2} cos 2xy + y N/D, degrees (7,8)
+//   0.1 <= y < 22   Re w = N/D, degrees (7,8) for y < 1, (5,6) or less above
+// Relative error against wofz, in FP32, for x inside the line's slow zone: below 2e-6 everywhere,
+// 2.5e-7 of the profile's norm (all coefficients of D but one or two are positive: Horner's rule
+// loses nothing). 16 operations and a reciprocal a point for y < 1 (plus an exponential and 8
+// operations below 0.1), 11 above, without table reads; Weideman's form takes about 100, the
+// Dawson form 45 and eight reads. The form is written for pairs of points in rox_voigt.cu; here it
+// is for one point, which is how it is tested.
+#define ROX_Y_CORE 0.1f
+ROX_FN int rox_core_row(float y) {
+  int r = 0;
+#pragma unroll
+  for (int k = 1; k < ROX_CORE_ROWS; k++) r += y >= rox_core_y[k][0];
+  return r;
+}
+// coefficient `slot` (n_0 .. n_7, d_1 .. d_8) of a line
+ROX_FN float rox_core_coef(float y, int slot) {
+  const int row = rox_core_row(y);
+#ifdef __CUDA_ARCH__
+  const float t = fmaf(__log2f(y), rox_core_y[row][1], rox_core_y[row][2]);
+#else
+  const float t = fmaf(log2f(y), rox_core_y[row][1], rox_core_y[row][2]);
+#endif
+  float a = rox_core_t[row][ROX_CORE_DEG][slot];
+#pragma unroll
+  for (int k = ROX_CORE_DEG - 1; k >= 0; k--) a = fmaf(a, t, rox_core_t[row][k][slot]);
+  return a;
+}
+ROX_FN float rox_core_coef_r(float y2, float r0, float r1, float r2, float r3) {   // y < 0.1: the slot's rox_core_r
+  return fmaf(fmaf(fmaf(r3, y2, r2), y2, r1), y2, r0);
+}
+// cos u by its Taylor polynomial to u^6, u2 = (2xy)^2 <= 2: the rest matters only where the
+// exponential beside it is below 1e-9 of the sum
+#define ROX_COS_C6 -1.388888888888889e-03f
+#define ROX_COS_C4 4.166666666666667e-02f
+#define ROX_LOG2E_F 1.4426950408889634f
 
 // Re w(x + iy) for x any sign, y >= 0, all regions. `daw` points at rox_daw_taylor.
 ROX_FN float rox_re_w(const float* daw, float x, float y) {

@@ -69,8 +69,8 @@ struct RoxListDev {
   const float2* node_d;
   const float2* span_base;
   // precomputed per-line constants of the launch's one (P,T) point (ROX_VX_PRE lists, else NULL):
-  // per line 3 float4, {A, B, P, Q}, {t_z, 1/gamma_G (negative: core-only zone), y, S/(gamma_G
-  // sqrt(pi))}, {far form at t_z, zlo (int bits), zhi (int bits), 0}
+  // per line 3 float4, {A, B, P, Q}, {t_z, 1/gamma_G, y, S/(gamma_G
+  // sqrt(pi))}, {X^2 of the end of its own zone (LineTab::z), zlo, zhi (int bits), smooth_dmin}
   const float4* rec;
   long long n_lattice;
   float dnu_f;

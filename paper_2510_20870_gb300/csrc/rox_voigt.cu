@@ -35,7 +35,6 @@
 
 namespace {
 
-#define ROX_NDAW (ROX_DAW_NODES * ROX_DAW_STRIDE)
 #define ROX_INV_PI 0.318309886183790672f
 
 // Per-line constants of one (P,T) point for the batch in hand. Each line has a slot; slots are
@@ -55,10 +54,8 @@ struct PairTab {
 struct LineTab {
   int2 W[32];      // window [jlo, jhi] (grid indices)
   int2 Z[32];      // slow zone [zlo, zhi] (grid indices; nodes: the window)
-  float iG[32];    // 1/gamma_G; negative if the slow zone is |z| < 6.5 not widened by the margin
-  float y[32];     // gamma_L / gamma_G
-  float pc[32];    // S / (gamma_G sqrt(pi))
-  float cf[32];    // the far form at t = t_z, which pass 1 adds at every point of the slow zone
+  float4 z[32];    // {1/gamma_G, y = gamma_L/gamma_G, S/(gamma_G sqrt(pi)), X^2 of the end of the
+                   // line's own zone where the precision margin widens it, else huge}
 };
 // one line's field out of a pair table row: half h (0, 1) of {lo, hi} pairs
 __device__ __forceinline__ float row_lo(const float4& v, int h) { return h ? v.y : v.x; }
@@ -73,7 +70,6 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ float load_width(const void* p, int f16, long long i) {
@@ -322,74 +318,151 @@ __device__ __forceinline__ void edge_line(const PairTab& P, const LineTab& L, in
 }
 
 // Pass 2 for the line in slot s, whose slow zone meets the span: at exactly the points where
-// pass 1 clamped t (t < t_z on the same rounded t, inside the window), the full FP32 Faddeeva
-// forms replace the far form's boundary value that pass 1 added there: + S V - cf.
-// A zone of |z| < 6.5 takes the core forms at every point (rox_re_w_core holds 1.1e-5 out to
-// |z| = 7.1); on a uniform grid the lanes then take consecutive points of the zone rather than
-// aligned 32-point sub-spans (fewer, fuller warp steps). Otherwise, per 32-point sub-span, one
-// form for all points where possible: the 3-level fraction if even the sub-span's point nearest
-// the centre has |z| >= 10, the 5-level one if |z| >= 6 there (both only get more accurate
-// further out), else rox_re_w per point. Accumulated into the warp's shared-memory row zacc
-// (one add per line and point; within a warp step the lanes touch distinct points).
+// pass 1 clamped t (t < t_z on the same rounded t, inside the window), the FP32 Faddeeva form of
+// the line's y (rox_faddeeva.cuh; FORM 0: y < 0.1, 1: y < 1, 2: above) replaces the far form's
+// boundary value cf that pass 1 added there: + S V - cf. In a zone widened to the precision margin the
+// points beyond the form's own zone (X^2 >= zc) take the far form on an offset rounded once.
+// The pass is bound by instruction issue, so a lane takes two points at once in paired FP32
+// instructions (two neighbouring points of the uniform grid: 64 points a warp step, one 8-byte
+// update of the warp's shared-memory row zacc; on nodes two sub-spans), the polynomials' coefficients
+// come from shared memory as ready pairs, and points outside the zone are selected away rather than
+// branched over. Within a warp step the lanes touch distinct points.
+struct ZoneC {
+  float A, B, P, Q, tz, cf, pc, zc;
+  f32x2 gU;                    // x2 -> U
+  f32x2 ge, ge0, gc, gy, gp;   // FORM 0: exponent = ge x2 + ge0, (2xy)^2 = gc x2, pc y, pc
+};
+__device__ __forceinline__ f32x2 f2_dup(float v) { return f2_pack(v, v); }
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// N(U)/D(U) of degrees (NP, NP + 1); cb: the 16 coefficients as pairs
+template <int NP>
+__device__ __forceinline__ f32x2 rat_pair(const ulonglong2* cb, f32x2 U) {
+  f32x2 c[16];
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    if (i < 4 ? 2 * i > NP : 2 * (i - 4) > NP) continue;
+    const ulonglong2 v = cb[i];
+    c[2 * i] = v.x;
+    c[2 * i + 1] = v.y;
+  }
+  f32x2 n = c[NP], d = c[8 + NP];
+#pragma unroll
+  for (int k = NP - 1; k >= 0; k--) {
+    n = f2_fma(n, U, c[k]);
+    d = f2_fma(d, U, c[8 + k]);
+  }
+  d = f2_fma(d, U, f2_dup(1.0f));
+  float d0, d1;
+  f2_unpack(d, d0, d1);
+  return f2_mul(n, f2_pack(rox_rcp(d0), rox_rcp(d1)));
+}
+// S V - cf for the pair of offsets X
+template <int FORM>
+__device__ __forceinline__ f32x2 zone_pair(const ZoneC& z, const ulonglong2* cb, f32x2 X) {
+  const f32x2 x2 = f2_mul(X, X);
+  const f32x2 r = rat_pair<FORM == 2 ? 5 : 7>(cb, f2_mul(x2, z.gU));
+  f32x2 v = f2_dup(-z.cf);
+  if constexpr (FORM == 0) {
+    float e0, e1;
+    f2_unpack(f2_fma(x2, z.ge, z.ge0), e0, e1);
+    const f32x2 u2 = f2_mul(x2, z.gc);
+    f32x2 g = f2_fma(u2, f2_dup(ROX_COS_C6), f2_dup(ROX_COS_C4));
+    g = f2_fma(u2, g, f2_dup(-0.5f));
+    g = f2_fma(u2, g, f2_dup(1.0f));
+    v = f2_fma(f2_pack(rox_exp2(e0), rox_exp2(e1)), f2_mul(g, z.gp), v);
+    v = f2_fma(r, z.gy, v);
+  } else {
+    v = f2_fma(r, z.gp, v);
+  }
+  if (z.zc < 1e38f) {
+    float x0, x1, v0, v1, d0, d1, w0, w1;
+    const f32x2 t = f2_add(x2, f2_dup(z.A));
+    f2_unpack(x2, x0, x1);
+    f2_unpack(v, v0, v1);
+    f2_unpack(f2_fma(t, t, f2_dup(z.B)), d0, d1);
+    f2_unpack(f2_fma(t, f2_dup(z.P), f2_dup(z.Q)), w0, w1);
+    v = f2_pack(x0 < z.zc ? v0 : fmaf(w0, rox_rcp(d0), -z.cf), x1 < z.zc ? v1 : fmaf(w1, rox_rcp(d1), -z.cf));
+  }
+  return v;
+}
+template <bool NU, int FORM>
+__device__ __forceinline__ void zone_points(const ZoneC& z, const ulonglong2* cb, float e, float f, int q0, int q1,
+                                            int lane, float dnu_f, const float2* D, float* zacc) {
+  float t0, t1, v0, v1;
+  if constexpr (NU) {
+    for (int m = (q0 >> 5) & ~1; m <= q1 >> 5; m += 2) {
+      const int q = 32 * m + lane;
+      const f32x2 X = f2_pack(pos<NU>(m, 0.f, e, f, D, dnu_f), pos<NU>(m + 1, 0.f, e, f, D, dnu_f));   // exact already
+      f2_unpack(f2_fma(X, X, f2_dup(z.A)), t0, t1);
+      const bool u0 = t0 < z.tz && q >= q0 && q <= q1, u1 = t1 < z.tz && q + 32 >= q0 && q + 32 <= q1;
+      if (!__any_sync(0xffffffffu, u0 || u1)) continue;
+      f2_unpack(zone_pair<FORM>(z, cb, X), v0, v1);
+      if (u0) zacc[q] += v0;
+      if (u1) zacc[q + 32] += v1;
+    }
+  } else {
+    int q = (q0 & ~1) + 2 * lane;
+    float mf = (float)(q & ~31);
+    const f32x2 dn = f2_dup(dnu_f), ff = f2_dup(f);
+    const float l0 = (float)(q & 31);
+    const f32x2 le = f2_add(f2_pack(l0, l0 + 1.0f), f2_dup(e));
+    const f32x2 X0 = f2_fma(le, dn, ff);                       // t rounded exactly as pass 1 rounds it
+    for (; q <= q1; q += 64, mf += 64.0f) {
+      const f32x2 Xm = f2_fma(f2_dup(mf), dn, X0);
+      f2_unpack(f2_fma(Xm, Xm, f2_dup(z.A)), t0, t1);
+      const f32x2 X = f2_fma(f2_add(le, f2_dup(mf)), dn, ff);  // the offset rounded once
+      f2_unpack(zone_pair<FORM>(z, cb, X), v0, v1);
+      float2* p = reinterpret_cast<float2*>(zacc + q);
+      float2 s = *p;
+      s.x += t0 < z.tz && q >= q0 ? v0 : 0.0f;
+      s.y += t1 < z.tz && q < q1 ? v1 : 0.0f;
+      *p = s;
+    }
+  }
+}
 template <bool NU>
-__device__ __forceinline__ void zone_line(const PairTab& P, const LineTab& L, int s, int Aw, int lane, float lanef,
-                                          float dnu_f, float inv_dnu, const float* daw, const float2* D, float* zacc) {
-  const int k = s >> 1, h = s & 1;
-  const float4 ab = P.ab[k], ef = P.ef[k];
-  const float A = row_lo(ab, h), e = row_lo(ef, h), f = row_hi(ef, h);
-  const float tz = h ? P.tz[k].y : P.tz[k].x;
-  const int2 w = L.W[s], z = L.Z[s];
-  const int lo = max(max(z.x, w.x), Aw), hi = min(min(z.y, w.y), Aw + ROX_SPAN - 1);
+__device__ __forceinline__ void zone_line(const PairTab& P, const LineTab& L, int s, int Aw, int lane, float dnu_f,
+                                          const float4& r, const float2* D, f32x2* cbuf, float* zacc) {
+  const int2 w = L.W[s], zw = L.Z[s];
+  const int lo = max(max(zw.x, w.x) - Aw, 0), hi = min(min(zw.y, w.y) - Aw, ROX_SPAN - 1);
   if (lo > hi) return;
-  const float iGs = L.iG[s], y = L.y[s], pcore = L.pc[s], cf = L.cf[s];
-  const float invG = fabsf(iGs);
-  if (!NU && iGs < 0.0f) {
-    // lanes on consecutive points of [lo, hi]; t rounded exactly as pass 1 rounds it
-    for (int q = lo - Aw + lane; q <= hi - Aw; q += 32) {
-      const float X0q = fmaf((float)(q & 31) + e, dnu_f, f);
-      const float Xm = fmaf((float)(q & ~31), dnu_f, X0q);
-      if (!(fmaf(Xm, Xm, A) < tz)) continue;
-      const float X = fmaf((float)q + e, dnu_f, f);
-      zacc[q] += fmaf(pcore, rox_re_w_core(daw, fabsf(X) * invG, y), -cf);
-    }
-    return;
-  }
-  const float X0 = NU ? 0.0f : fmaf(lanef + e, dnu_f, f);
-  if (iGs < 0.0f) {
-    for (int m = (lo - Aw) >> 5; m <= ((hi - Aw) >> 5); m++) {
-      const int j = Aw + 32 * m + lane;
-      const float Xm = pos<NU>(m, X0, e, f, D, dnu_f);
-      if (!(fmaf(Xm, Xm, A) < tz) || j < w.x || j > w.y) continue;
-      // the uniform grid recomputes X from the index in one rounding; node offsets are exact already
-      const float X = NU ? Xm : fmaf((float)(32 * m + lane) + e, dnu_f, f);
-      zacc[32 * m + lane] += fmaf(pcore, rox_re_w_core(daw, fabsf(X) * invG, y), -cf);
-    }
-    return;
-  }
-  const float centre = (float)Aw - e - f * inv_dnu;     // k0 + f, within 0.25 grid steps (uniform grid)
-  const float y2 = y * y;
-  for (int m = (lo - Aw) >> 5; m <= ((hi - Aw) >> 5); m++) {
-    const int am = Aw + 32 * m, bm = am + 31;
-    const int j = am + lane;
-    const float Xm = pos<NU>(m, X0, e, f, D, dnu_f);
-    float xm;   // |X| of the sub-span's point nearest the line centre, in units of gamma_G
-    if constexpr (NU) {
-      const float Xa = __shfl_sync(0xffffffffu, Xm, 0), Xb = __shfl_sync(0xffffffffu, Xm, 31);
-      xm = (Xa <= 0.0f && Xb >= 0.0f ? 0.0f : fminf(fabsf(Xa), fabsf(Xb))) * invG;
-    } else {
-      const float dc = (centre >= (float)am && centre <= (float)bm)
-                           ? 0.0f : fminf(fabsf((float)am - centre), fabsf((float)bm - centre));
-      xm = fmaxf(dc - 1.0f, 0.0f) * dnu_f * invG;
-    }
-    if (!(fmaf(Xm, Xm, A) < tz) || j < w.x || j > w.y) continue;
-    const float sm = fmaf(xm, xm, y2);
-    const float X = NU ? Xm : fmaf((float)(32 * m + lane) + e, dnu_f, f);
-    const float x = fabsf(X) * invG;
-    float r;
-    if (sm >= ROX_S_CF3) r = rox_re_w_cf3(x, y);
-    else if (sm >= ROX_S_CF5) r = rox_re_w_cf5g(x, y);
-    else r = rox_re_w(daw, x, y);
-    zacc[32 * m + lane] += fmaf(pcore, r, -cf);
+  const int k = s >> 1, h = s & 1;
+  const float4 ab = P.ab[k], pq = P.pq[k], ef = P.ef[k];
+  const float4 zl = L.z[s];                     // {1/gamma_G, y, S/(gamma_G sqrt(pi)), zc}
+  const float y = zl.y, y2 = y * y;
+  // the form's coefficients, one a lane, handed round through shared memory
+  const float c = y < ROX_Y_CORE ? rox_core_coef_r(y2, r.x, r.y, r.z, r.w) : rox_core_coef(y, lane & 15);
+  __syncwarp();
+  if (lane < 16) cbuf[lane] = f2_dup(c);
+  __syncwarp();
+  ZoneC z;
+  z.A = row_lo(ab, h);
+  z.B = row_hi(ab, h);
+  z.P = row_lo(pq, h);
+  z.Q = row_hi(pq, h);
+  z.tz = h ? P.tz[k].y : P.tz[k].x;
+  z.cf = fmaf(z.tz, z.P, z.Q) * rox_rcp(fmaf(z.tz, z.tz, z.B));
+  z.pc = zl.z;
+  z.zc = zl.w;
+  const float g2 = zl.x * zl.x;
+  z.gU = f2_dup(g2 * rox_rcp(y2 + ROX_CORE_KAPPA));
+  z.gp = f2_dup(zl.z);
+  const ulonglong2* cb = reinterpret_cast<const ulonglong2*>(cbuf);
+  const float e = row_lo(ef, h), f = row_hi(ef, h);
+  if (y < ROX_Y_CORE) {
+    z.ge = f2_dup(-ROX_LOG2E_F * g2);
+    z.ge0 = f2_dup(ROX_LOG2E_F * y2);
+    z.gc = f2_dup(4.0f * y2 * g2);
+    z.gy = f2_dup(zl.z * y);
+    zone_points<NU, 0>(z, cb, e, f, lo, hi, lane, dnu_f, D, zacc);
+  } else if (y < 1.0f) {
+    zone_points<NU, 1>(z, cb, e, f, lo, hi, lane, dnu_f, D, zacc);
+  } else {
+    zone_points<NU, 2>(z, cb, e, f, lo, hi, lane, dnu_f, D, zacc);
   }
 }
 
@@ -399,11 +472,11 @@ __device__ __forceinline__ void zone_line(const PairTab& P, const LineTab& L, in
 // (see load_widths). The Voigt kernel computes them per line and span, or (ROX_VX_PRE) reads
 // them from k_line_params, which computes them once per line with this same function.
 struct LineK {
-  float A, B, P, Q, tz, iGs, y, pc, cf, hz;
+  float A, B, P, Q, tz, iG, y, pc, zc, hz;
 };
 template <bool BRD>
 __device__ __forceinline__ LineK line_consts(float nu0f, float Sp, float gref, float nt, const RoxJobDev& J,
-                                             float margin_cm, bool want_cf) {
+                                             float margin_cm) {
   LineK k;
   const float gG = nu0f * J.gG_fac;
   const float gL = BRD ? fmaf(gref, J.p_fac, nt) : gref * rox_exp2(nt * J.l2_ratio) * J.p_fac;
@@ -416,17 +489,15 @@ __device__ __forceinline__ LineK line_consts(float nu0f, float Sp, float gref, f
   const float hz2 = fmaxf(0.0f, fc.r2 * gG2 - gL2);
   float hz = hz2 * rox_rsqrt(hz2);            // 0 for hz2 = 0 (rsqrt(0) = inf, product taken as 0 below)
   hz = hz2 > 0.0f ? hz : 0.0f;
-  // zone |z| < 6.5 not widened by the margin: the core forms cover all of it
-  const bool core_only = fc.r2 == ROX_S_PADE && hz >= margin_cm;
+  k.zc = hz >= margin_cm ? 3e38f : hz2;
   k.hz = fmaxf(hz, margin_cm);
   k.A = fc.alpha * gG2;
   k.B = fc.beta * (gG2 * gG2);
   k.P = pY;
   k.Q = pY * (fc.kappa * gG2);
   k.tz = fmaf(k.hz, k.hz, k.A);
-  k.iGs = core_only ? -invG : invG;
+  k.iG = invG;
   k.pc = Sp * invG * ROX_INV_SQRT_PI;
-  k.cf = want_cf ? fmaf(k.tz, k.P, k.Q) * rox_rcp(fmaf(k.tz, k.tz, k.B)) : 0.0f;
   return k;
 }
 
@@ -455,12 +526,12 @@ __global__ void k_line_params(const RoxListDev L, const RoxJobDev J, float4* rec
     const float Sp = J.S32[i - J.l0];
     const float gref = load_width(L.gamma_ref, L.width_f16, i), nt = load_width(L.n_t, L.width_f16, i);
     const float nu0f = L.nu_min_f + fmaf(g.x, L.dnu_f, g.y);
-    const LineK k = line_consts<false>(nu0f, Sp, gref, nt, J, margin_cm, true);
+    const LineK k = line_consts<false>(nu0f, Sp, gref, nt, J, margin_cm);
     int zlo, zhi;
     zone_bounds(g, k.hz, L.inv_dnu_f, zlo, zhi);
     rec[3 * i] = make_float4(k.A, k.B, k.P, k.Q);
-    rec[3 * i + 1] = make_float4(k.tz, k.iGs, k.y, k.pc);
-    rec[3 * i + 2] = make_float4(k.cf, __int_as_float(zlo), __int_as_float(zhi),
+    rec[3 * i + 1] = make_float4(k.tz, k.iG, k.y, k.pc);
+    rec[3 * i + 2] = make_float4(k.zc, __int_as_float(zlo), __int_as_float(zhi),
                                  smooth_dmin(k.A, k.B, 0.5f * (ROX_SPAN - 1) * L.dnu_f));
   }
 }
@@ -544,7 +615,7 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
           } else {
             float gref, nt;
             load_widths<BRD>(J, L, L.width_f16, li, gref, nt);
-            const LineK kc = line_consts<BRD>(L.nu_min_f + fmaf(g.x, dnu_f, g.y), S_row[li], gref, nt, J, margin_cm, false);
+            const LineK kc = line_consts<BRD>(L.nu_min_f + fmaf(g.x, dnu_f, g.y), S_row[li], gref, nt, J, margin_cm);
             a = kc.A;
             b = kc.B;
             p = kc.P;
@@ -610,33 +681,36 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
   constexpr bool BRD = (X & ROX_VX_BROAD) != 0;
   constexpr bool PRE = (X & ROX_VX_PRE) != 0;
   extern __shared__ __align__(16) float2 s_nodes[];   // NU: node offsets; PRE: the staged per-line constants
-  __shared__ float4 s_geo[W][2][32];
-  __shared__ float s_S[W][2][32];
+  __shared__ float4 s_geo[W][32];
+  __shared__ float s_S[PRE ? 1 : W][32];
   __shared__ PairTab s_pairs[W];
   __shared__ LineTab s_lines[W];
-  __shared__ float s_zacc[W][ROX_SPAN];
+  __shared__ __align__(8) float s_zacc[W][ROX_SPAN];
   __shared__ float s_tot[W][ROX_SPAN];    // the span's sum over its parts
-  __shared__ float s_daw[ROX_NDAW];
+  __shared__ float s_part[W][2][ROX_SPAN];  // a part's sum and its compensation
+  __shared__ __align__(16) f32x2 s_cf[W][16];   // a zoned line's form coefficients
   __shared__ int s_status;
 
   const int tid = threadIdx.x;
   const int lane = tid & 31, w = tid >> 5;
-  for (int i = tid; i < ROX_NDAW; i += W * 32) s_daw[i] = (&rox_daw_taylor[0][0])[i];
   if (tid == 0) s_status = *(volatile int32_t*)&A.hdr->status;
   __syncthreads();
   if (s_status != ROX_OK) return;   // e.g. unsorted input: leave sigma untouched
 
-  float4(*geo_st)[32] = s_geo[w];
-  float(*S_st)[32] = s_S[w];
+  float4* geo_st = s_geo[w];   // this lane's line of the batch; the next batch's copy starts once it is read
+  float* S_st = s_S[PRE ? 0 : w];
   PairTab& PT = s_pairs[w];
   LineTab& LT = s_lines[w];
   const float lanef = (float)lane;
   const float cheb = rox_cheb_x[lane];
   float* zacc = s_zacc[w];
   float* stot = s_tot[w];
+  float *part_tot = s_part[w][0] + lane, *part_cmp = s_part[w][1] + lane;   // [32 m]: this lane's points
+  f32x2* cbuf = s_cf[w];
+  const float4 core_r = *reinterpret_cast<const float4*>(rox_core_r[lane & 15]);
   float2* Drow = NU ? s_nodes + w * ROX_SPAN : nullptr;   // this span's node offsets
-  // PRE: per warp two buffers of 32 lines x 3 float4 of per-line constants
-  float4(*rec_st)[32][3] = PRE ? reinterpret_cast<float4(*)[32][3]>(s_nodes) + 2 * w : nullptr;
+  // PRE: per warp 32 lines x 3 float4 of per-line constants
+  float4(*rec_st)[3] = PRE ? reinterpret_cast<float4(*)[3]>(s_nodes) + 32 * w : nullptr;
   const float2* D = NU ? Drow + lane : nullptr;
   unsigned long long evals = 0;   // (line, point) pairs inside the cutoff and the job's window
 
@@ -742,55 +816,52 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
     for (int p = p_first; p <= p_last; p++) {
       const int plo = 32 * ((nbat * p) / ROX_PARTS);
       const int phi = min(nn, 32 * ((nbat * (p + 1)) / ROX_PARTS));
-      float acc[ROX_K], tot[ROX_K], cmp[ROX_K], nacc = 0.f, nsum = 0.f, ncmp = 0.f;
+      // the part's total and its compensation: in shared memory (touched once in four batches),
+      // Chebyshev point in nsum, ncmp
+      float acc[ROX_K], nacc = 0.f, nsum = 0.f, ncmp = 0.f;
 #pragma unroll
-      for (int m = 0; m < ROX_K; m++) { acc[m] = 0.f; tot[m] = 0.f; cmp[m] = 0.f; zacc[32 * m + lane] = 0.f; }
+      for (int m = 0; m < ROX_K; m++) {
+        acc[m] = 0.f;
+        part_tot[32 * m] = 0.f;
+        part_cmp[32 * m] = 0.f;
+        zacc[32 * m + lane] = 0.f;
+      }
 
-      // stage batch 0; widths go through registers one batch ahead (with an index, the
-      // positions' line numbers two batches ahead)
+      // stage a batch's lines, one a lane: batch 0 here, each next one as soon as the lanes have
+      // turned the current one into constants; widths go through registers (with an index, the
+      // positions' line numbers one batch further ahead)
       float gref = 0.f, nt = 0.f;
       int li_n = 0;   // IDX: line number of this lane's position in the next batch
-      if (plo + lane < phi) {
-        const int li = IDX ? Lst.idx[line_at(plo + lane)] : line_at(plo + lane);
-        cp_async16(&geo_st[0][lane], &Lst.geo[li]);
-        if constexpr (PRE) {
+      if (IDX && plo + lane < phi) li_n = Lst.idx[line_at(plo + lane)];
+      auto stage = [&](int q) {
+        if (q < phi) {
+          const int li = IDX ? li_n : line_at(q);
+          cp_async16(&geo_st[lane], &Lst.geo[li]);
+          if constexpr (PRE) {
 #pragma unroll
-          for (int c = 0; c < 3; c++) cp_async16(&rec_st[0][lane][c], &Lst.rec[3 * (long long)li + c]);
-        } else {
-          cp_async4(&S_st[0][lane], &S_row[li]);
-          load_widths<BRD>(J, Lst, f16, li, gref, nt);
+            for (int c = 0; c < 3; c++) cp_async16(&rec_st[lane][c], &Lst.rec[3 * (long long)li + c]);
+          } else {
+            cp_async4(&S_st[lane], &S_row[li]);
+            load_widths<BRD>(J, Lst, f16, li, gref, nt);
+          }
         }
-      }
-      if (IDX && plo + 32 + lane < phi) li_n = Lst.idx[line_at(plo + 32 + lane)];
-      cp_async_commit();
+        if (IDX && q + 32 < phi) li_n = Lst.idx[line_at(q + 32)];
+        cp_async_commit();
+      };
+      stage(plo + lane);
       int nb = 0;
       for (int b0 = plo; b0 < phi; b0 += 32, nb++) {
         const int cnt = min(32, phi - b0);
-        const int buf = nb & 1;
-        float gref_n = 0.f, nt_n = 0.f;
-        if (b0 + 32 + lane < phi) {
-          const int li = IDX ? li_n : line_at(b0 + 32 + lane);
-          cp_async16(&geo_st[buf ^ 1][lane], &Lst.geo[li]);
-          if constexpr (PRE) {
-#pragma unroll
-            for (int c = 0; c < 3; c++) cp_async16(&rec_st[buf ^ 1][lane][c], &Lst.rec[3 * (long long)li + c]);
-          } else {
-            cp_async4(&S_st[buf ^ 1][lane], &S_row[li]);
-            load_widths<BRD>(J, Lst, f16, li, gref_n, nt_n);
-          }
-        }
-        if (IDX && b0 + 64 + lane < phi) li_n = Lst.idx[line_at(b0 + 64 + lane)];
-        cp_async_commit();
-        cp_async_wait1();   // this lane's copies of the current batch have landed
+        cp_async_wait0();   // this lane's copies of the current batch have landed
 
         // ---- per-line constants (lane <-> line b0 + lane), written to the line's slot
         const bool live = lane < cnt;
         bool covers = false, zoned = false, smooth = false;
-        float ax = 0.f, ay = 0.f, vA = 1.f, vB = 0.f, vP = 0.f, vQ = 0.f, tz = 0.f, iGs = 1.f, yv = 0.f, pcv = 0.f;
-        float cfv = 0.f;
+        float ax = 0.f, ay = 0.f, vA = 1.f, vB = 0.f, vP = 0.f, vQ = 0.f, tz = 0.f;
+        float4 zl = make_float4(1.f, 0.f, 0.f, 0.f);
         int jlo = 1, jhi = 0, zlo = 0, zhi = -1;
         if (live) {
-          const float4 g = geo_st[buf][lane];
+          const float4 g = geo_st[lane];
           jlo = __float_as_int(g.z);
           jhi = __float_as_int(g.w);
           const int ov = min(jhi, whi) - max(jlo, wlo) + 1;
@@ -800,16 +871,16 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           float dmin;
           if constexpr (PRE) {
             // uniform grid, constants from k_line_params
-            const float4 r0 = rec_st[buf][lane][0], r1 = rec_st[buf][lane][1], r2 = rec_st[buf][lane][2];
+            const float4 r0 = rec_st[lane][0], r1 = rec_st[lane][1], r2 = rec_st[lane][2];
             kc.A = r0.x;
             kc.B = r0.y;
             kc.P = r0.z;
             kc.Q = r0.w;
             kc.tz = r1.x;
-            kc.iGs = r1.y;
+            kc.iG = r1.y;
             kc.y = r1.z;
             kc.pc = r1.w;
-            kc.cf = r2.x;
+            kc.zc = r2.x;
             zlo = __float_as_int(r2.y);
             zhi = __float_as_int(r2.z);
             ax = (float)Aw - g.x;     // exact: both are integers below 2^24
@@ -817,7 +888,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
             zoned = !(Bw < zlo || Aw > zhi);
             dmin = r2.w;
           } else {
-            const float Sp = S_st[buf][lane];
+            const float Sp = S_st[lane];
             float nu0f;   // line centre; its offset state {E, F} (uniform grid) or {c hi, c lo} (nodes)
             if constexpr (NU) {
               // c = nu0 - (span's first node) as a double-float pair (the hi parts cancel exactly)
@@ -830,7 +901,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
               ax = (float)Aw - g.x;     // exact: both are integers below 2^24
               ay = -g.y;
             }
-            kc = line_consts<BRD>(nu0f, Sp, gref, nt, J, margin_cm, false);
+            kc = line_consts<BRD>(nu0f, Sp, gref, nt, J, margin_cm);
             if constexpr (NU) {
               // the span's offsets run from -c to Ws - c; pass 2 then scans the window itself
               const float hzp = kc.hz * 1.001f + 1e-6f * (fabsf(ax) + Ws);
@@ -841,7 +912,6 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
               zone_bounds(g, kc.hz, Lst.inv_dnu_f, zlo, zhi);
               zoned = !(Bw < zlo || Aw > zhi);
             }
-            if (zoned) kc.cf = fmaf(kc.tz, kc.P, kc.Q) * rox_rcp(fmaf(kc.tz, kc.tz, kc.B));
             dmin = smooth_dmin(kc.A, kc.B, half);
           }
           const float D = NU ? half - ax - ay : fmaf(ax + 0.5f * (ROX_SPAN - 1), dnu_f, ay);
@@ -851,10 +921,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           vP = kc.P;
           vQ = kc.Q;
           tz = kc.tz;
-          iGs = kc.iGs;
-          yv = kc.y;
-          pcv = kc.pc;
-          cfv = kc.cf;
+          zl = make_float4(kc.iG, kc.y, kc.pc, kc.zc);
         }
         const unsigned msm = __ballot_sync(0xffffffffu, live && smooth);
         const unsigned clean = __ballot_sync(0xffffffffu, live && covers && !zoned && !smooth);
@@ -880,13 +947,9 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           reinterpret_cast<float*>(&PT.tz[k])[h] = tz;
           LT.W[slot] = make_int2(jlo, jhi);
           LT.Z[slot] = make_int2(zlo, zhi);
-          LT.iG[slot] = iGs;
-          LT.y[slot] = yv;
-          LT.pc[slot] = pcv;
-          LT.cf[slot] = cfv;
+          LT.z[slot] = zl;
         }
-        gref = gref_n;
-        nt = nt_n;
+        stage(b0 + 32 + lane);
         __syncwarp();
 
         // ---- pass 1: far formula at every point of every line's window. Clean pairs as they
@@ -903,17 +966,17 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
         }
         // ---- pass 2: at the points each zoned line had clamped, the full Faddeeva forms
         for (unsigned z = zslots; z; z &= z - 1)
-          zone_line<NU>(PT, LT, __ffs(z) - 1, Aw, lane, lanef, dnu_f, Lst.inv_dnu_f, s_daw, D, zacc);
+          zone_line<NU>(PT, LT, __ffs(z) - 1, Aw, lane, dnu_f, core_r, D, cbuf, zacc);
         __syncwarp();
         // the partial sums into the part's total every 4 batches: compensated (Kahan) with
         // ROX_KAHAN, else plainly (kw = 0: the correction term stays 0)
         if ((nb & 3) == 3 || b0 + 32 >= phi) {
 #pragma unroll
           for (int m = 0; m < ROX_K; m++) {
-            const float yk = acc[m] - cmp[m];
-            const float tk = tot[m] + yk;
-            cmp[m] = ((tk - tot[m]) - yk) * kw;
-            tot[m] = tk;
+            const float t0 = part_tot[32 * m], yk = acc[m] - part_cmp[32 * m];
+            const float tk = t0 + yk;
+            part_cmp[32 * m] = ((tk - t0) - yk) * kw;
+            part_tot[32 * m] = tk;
             acc[m] = 0.f;
           }
           const float yn = nacc - ncmp;
@@ -923,7 +986,6 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           nacc = 0.f;
         }
       }
-      cp_async_wait0();
       // this part's share of the far cells, at this lane's Chebyshev point
       for (int c = n_far * p / ROX_PARTS; c < n_far * (p + 1) / ROX_PARTS; c++) {
         const int cell = c < cl1 - cl0 ? cl0 + c : cr0 + (c - (cl1 - cl0));
@@ -940,20 +1002,17 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
       // fold in the pass-2 (near-centre) sums
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
-        const float yk = zacc[32 * m + lane] - cmp[m];
-        const float tk = tot[m] + yk;
-        cmp[m] = ((tk - tot[m]) - yk) * kw;
-        tot[m] = tk;
+        part_tot[32 * m] += zacc[32 * m + lane] - part_cmp[32 * m];
       }
       if (part >= 0) {           // a split item: this part's sum goes to the tail scratch
         float* dst = A.tail_part + ((size_t)(item - A.n_whole) * ROX_PARTS + p) * ROX_PART_FLOATS;
 #pragma unroll
-        for (int m = 0; m < ROX_K; m++) __stcg(&dst[32 * m + lane], tot[m]);
+        for (int m = 0; m < ROX_K; m++) __stcg(&dst[32 * m + lane], part_tot[32 * m]);
         __stcg(&dst[ROX_SPAN + lane], nsum);
       } else {
         ntot = p == 0 ? nsum : ntot + nsum;
 #pragma unroll
-        for (int m = 0; m < ROX_K; m++) stot[32 * m + lane] = p == 0 ? tot[m] : stot[32 * m + lane] + tot[m];
+        for (int m = 0; m < ROX_K; m++) stot[32 * m + lane] = p == 0 ? part_tot[32 * m] : stot[32 * m + lane] + part_tot[32 * m];
       }
       __syncwarp();
     }   // parts
@@ -1049,7 +1108,7 @@ namespace {
 template <bool NU, int X, int W>
 constexpr size_t voigt_dyn_smem() {
   return NU ? (size_t)W * ROX_SPAN * sizeof(float2)
-            : ((X & ROX_VX_PRE) ? (size_t)W * 2 * 32 * 3 * sizeof(float4) : (size_t)0);
+            : ((X & ROX_VX_PRE) ? (size_t)W * 32 * 3 * sizeof(float4) : (size_t)0);
 }
 }  // namespace
 
