@@ -23,9 +23,10 @@ extern "C" void rox_host_core_zone(const float* x, const float* y, float* out, i
     const float y2 = y[i] * y[i], x2 = x[i] * x[i];
     const bool small = y[i] < ROX_Y_CORE;
     float c[16];
+    const int row = rox_core_row(y[i]);
     for (int k = 0; k < 16; k++) {
       const float* r = rox_core_r[k];
-      c[k] = small ? rox_core_coef_r(y2, r[0], r[1], r[2], r[3]) : rox_core_coef(y[i], k);
+      c[k] = small ? rox_core_coef_r(y2, r[0], r[1], r[2], r[3]) : rox_core_coef(row, rox_core_arg(row, y[i]), k);
     }
     const int np = y[i] < 1.0f ? 7 : 5;
     const float U = x2 * (1.0f / (y2 + ROX_CORE_KAPPA));

@@ -129,13 +129,13 @@ def main():
     for ya, yb, *_ in ROWS:
         la, lb = np.log2(ya), np.log2(yb)
         o.append("  {%.9ef, %.9ef, %.9ef}," % (ya, 2 / (lb - la), -(la + lb) / (lb - la)))
-    o += ["};", "/* [interval][power of t][slot]: n_0 .. in slots 0 .., d_1 .. in slots 8 .. */",
-          "ROX_GTABLE float rox_core_t[%d][%d][16] = {" % (len(ROWS), DEG + 1)]
+    o += ["};", "/* [interval][slot][power of t]: n_0 .. in slots 0 .., d_1 .. in slots 8 .. */",
+          "ROX_GTABLE ROX_ALIGN16 float rox_core_t[%d][16][%d] = {" % (len(ROWS), DEG + 1)]
     for r in ROWS:
-        o.append("{" + ",\n ".join("{" + ", ".join("%.9ef" % v for v in line) + "}" for line in row(*r)) + "},")
+        o.append("{" + ",\n ".join("{" + ", ".join("%.9ef" % v for v in line) + "}" for line in row(*r).T) + "},")
     o.append("};")
     o += ["/* y < 0.1: [slot][power of y^2] */", "#define ROX_CORE_DEG_R %d" % DEG_R,
-          "ROX_GTABLE ROX_ALIGN16 float rox_core_r[16][%d] = {" % (DEG_R + 1)]
+          "ROX_TABLE float rox_core_r[16][%d] = {" % (DEG_R + 1)]
     o.append(",\n".join("{" + ", ".join("%.9ef" % v for v in col) + "}" for col in row_r().T))
     o.append("};")
     print("\n".join(o))

@@ -639,6 +639,7 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
   L0.idx = nullptr;
   L0.inv_dnu_f = on_nodes ? 0.0f : (float)(1.0 / grid->dnu);
   L0.rec = pre ? w.rec : nullptr;
+  L0.cutoff_f = (float)cutoff;
   L0.c_steps = on_nodes ? 0 : cutoff_steps(cutoff, grid->dnu);
   std::vector<RoxJobDev> jobs(n_pt);
   for (int k = 0; k < n_pt; k++) {
@@ -1038,6 +1039,7 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     L[l].width_f16 = P.lines.width_dtype == ROX_WIDTH_F16;
     L[l].inv_dnu_f = (float)(1.0 / P.lattice.dnu);
     L[l].rec = nullptr;
+    L[l].cutoff_f = (float)P.cutoff;
     L[l].c_steps = cutoff_steps(P.cutoff, P.lattice.dnu);
   }
   std::vector<RoxJobDev> J(n_jobs);

@@ -302,18 +302,25 @@ ROX_FN int rox_core_row(float y) {
   for (int k = 1; k < ROX_CORE_ROWS; k++) r += y >= rox_core_y[k][0];
   return r;
 }
-// coefficient `slot` (n_0 .. n_7, d_1 .. d_8) of a line
-ROX_FN float rox_core_coef(float y, int slot) {
-  const int row = rox_core_row(y);
+// argument of a line's coefficient polynomials, and coefficient `slot` (n_0 .. n_7, d_1 .. d_8)
+ROX_FN float rox_core_arg(int row, float y) {
 #ifdef __CUDA_ARCH__
-  const float t = fmaf(__log2f(y), rox_core_y[row][1], rox_core_y[row][2]);
+  return fmaf(__log2f(y), rox_core_y[row][1], rox_core_y[row][2]);
 #else
-  const float t = fmaf(log2f(y), rox_core_y[row][1], rox_core_y[row][2]);
+  return fmaf(log2f(y), rox_core_y[row][1], rox_core_y[row][2]);
 #endif
-  float a = rox_core_t[row][ROX_CORE_DEG][slot];
-#pragma unroll
-  for (int k = ROX_CORE_DEG - 1; k >= 0; k--) a = fmaf(a, t, rox_core_t[row][k][slot]);
+}
+ROX_FN float rox_core_coef(int row, float t, int slot) {
+  const float* c = rox_core_t[row][slot];
+#ifdef __CUDA_ARCH__
+  const float4 lo = *reinterpret_cast<const float4*>(c), hi = *reinterpret_cast<const float4*>(c + 4);
+  const float a = fmaf(fmaf(fmaf(hi.w, t, hi.z), t, hi.y), t, hi.x);
+  return fmaf(fmaf(fmaf(fmaf(a, t, lo.w), t, lo.z), t, lo.y), t, lo.x);
+#else
+  float a = c[ROX_CORE_DEG];
+  for (int k = ROX_CORE_DEG - 1; k >= 0; k--) a = fmaf(a, t, c[k]);
   return a;
+#endif
 }
 ROX_FN float rox_core_coef_r(float y2, float r0, float r1, float r2, float r3) {   // y < 0.1: the slot's rox_core_r
   return fmaf(fmaf(fmaf(r3, y2, r2), y2, r1), y2, r0);

@@ -77,6 +77,7 @@ struct RoxListDev {
   float nu_min_f;
   int32_t width_f16;
   float inv_dnu_f;            // 1/dnu (uniform grid; 0 on nodes)
+  float cutoff_f;             // wing cutoff (cm^-1)
   int32_t c_steps;            // floor(cutoff / dnu) - 2: points every line's window surely reaches on each side
 };
 

@@ -57,6 +57,23 @@ struct LineTab {
   float4 z[32];    // {1/gamma_G, y = gamma_L/gamma_G, S/(gamma_G sqrt(pi)), X^2 of the end of the
                    // line's own zone where the precision margin widens it, else huge}
 };
+// The warp's tables of a batch; before they are written the same memory holds the edge lines' scan.
+#define ROX_EDGE_TERMS 10
+struct EdgeRec {
+  float m[ROX_EDGE_TERMS];   // moments of the edge lines up to this one
+  int key;                   // first point (counted from the side the lines come from) that has them
+  int pad;
+};
+struct BatchTab {
+  union {
+    struct {
+      PairTab pairs;
+      LineTab lines;
+    };
+    EdgeRec scan[33];        // [0]: the lines before the batch
+  };
+  __device__ BatchTab() {}
+};
 // one line's field out of a pair table row: half h (0, 1) of {lo, hi} pairs
 __device__ __forceinline__ float row_lo(const float4& v, int h) { return h ? v.y : v.x; }
 __device__ __forceinline__ float row_hi(const float4& v, int h) { return h ? v.w : v.z; }
@@ -264,11 +281,10 @@ __device__ __forceinline__ void interp_span(float v, int lane, const float2* D, 
   }
 }
 
-// Pass 1 for pair k of which at least one line is cut by a window edge: the sub-spans outside
-// both windows are skipped (warp-uniform test); the sub-spans inside both windows take every
-// point; elsewhere each point takes line i iff it lies in the line's window, m in
-// [ceil((jlo-Aw-lane)/32), floor((jhi-Aw-lane)/32)] (the exact integer window). Lines arrive
-// sorted by nu0, so paired edge lines have their edges in the same or a neighbouring sub-span.
+// Pass 1 for pair k of which at least one line is cut by a window edge that the edge scan does not
+// take: the sub-spans outside both windows are skipped (warp-uniform test); elsewhere each point
+// takes line i iff it lies in the line's window, m in [ceil((jlo-Aw-lane)/32),
+// floor((jhi-Aw-lane)/32)] (the exact integer window).
 template <bool NU>
 __device__ __forceinline__ void edge_pair(const PairTab& P, const LineTab& L, int k, int Aw, int lane, float lanef,
                                           float dnu_f, const float2* D, float (&acc)[ROX_K]) {
@@ -278,18 +294,13 @@ __device__ __forceinline__ void edge_pair(const PairTab& P, const LineTab& L, in
   const int mf = max(0, min(lo0, lo1) >> 5), ml = min(ROX_K - 1, max(hi0, hi1) >> 5);
   const int mlo0 = (lo0 - lane + 31) >> 5, mhi0 = (hi0 - lane) >> 5;   // this lane's window, in m
   const int mlo1 = (lo1 - lane + 31) >> 5, mhi1 = (hi1 - lane) >> 5;
-  const int cf = max((lo0 + 31) >> 5, (lo1 + 31) >> 5), cl = min((hi0 - 31) >> 5, (hi1 - 31) >> 5);
   float X0, X1;
   pair_x0<NU>(c, lanef, dnu_f, X0, X1);
 #pragma unroll
   for (int m = 0; m < ROX_K; m++) {
     if (m < mf || m > ml) continue;
     const float x0 = pos<NU>(m, X0, c.e0, c.f0, D, dnu_f), x1 = pos<NU>(m, X1, c.e1, c.f1, D, dnu_f);
-    if (m >= cf && m <= cl) {
-      acc[m] = pair_add<true, false>(x0, x1, c, true, true, acc[m]);
-    } else {
-      acc[m] = pair_add<true, true>(x0, x1, c, m >= mlo0 && m <= mhi0, m >= mlo1 && m <= mhi1, acc[m]);
-    }
+    acc[m] = pair_add<true, true>(x0, x1, c, m >= mlo0 && m <= mhi0, m >= mlo1 && m <= mhi1, acc[m]);
   }
 }
 
@@ -435,7 +446,9 @@ __device__ __forceinline__ void zone_line(const PairTab& P, const LineTab& L, in
   const float4 zl = L.z[s];                     // {1/gamma_G, y, S/(gamma_G sqrt(pi)), zc}
   const float y = zl.y, y2 = y * y;
   // the form's coefficients, one a lane, handed round through shared memory
-  const float c = y < ROX_Y_CORE ? rox_core_coef_r(y2, r.x, r.y, r.z, r.w) : rox_core_coef(y, lane & 15);
+  const int row = rox_core_row(y);
+  const float c = y < ROX_Y_CORE ? rox_core_coef_r(y2, r.x, r.y, r.z, r.w)
+                                 : rox_core_coef(row, rox_core_arg(row, y), lane & 15);
   __syncwarp();
   if (lane < 16) cbuf[lane] = f2_dup(c);
   __syncwarp();
@@ -499,6 +512,200 @@ __device__ __forceinline__ LineK line_consts(float nu0f, float Sp, float gref, f
   k.iG = invG;
   k.pc = Sp * invG * ROX_INV_SQRT_PI;
   return k;
+}
+
+// Sum of v[0..7] over the warp: lane l ends with the sum of v[i], i = bits 4, 3, 2 of l (as 4 2 1),
+// by a fixed tree that halves the values held at each exchange.
+__device__ __forceinline__ float warp_sum8(const float (&v)[8], int lane) {
+  float a[4], b[2], c;
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const float keep = h16 ? v[4 + i] : v[i], give = h16 ? v[i] : v[4 + i];
+    a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; i++) {
+    const float keep = h8 ? a[2 + i] : a[i], give = h8 ? a[i] : a[2 + i];
+    b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+  const float keep = h4 ? b[1] : b[0], give = h4 ? b[0] : b[1];
+  c = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+
+#define ROX_ZONE_DENSE 8   // points of the common zone per zoned line up to which the batch form is taken
+// Pass 2 for all zoned lines of a batch at once, one line a lane: where the lines lie close together
+// their zones share most of their points, and the warp walks those points [qa, qb] with every
+// lane evaluating its own line (coefficients in registers, computed once for the batch) and a
+// warp sum of eight points at a time. Against the line by line form this takes a point's work
+// to a thirty-second of 23 instructions per line, where that takes some 70 for 32 points plus 60
+// per line (measured: 297 + 62 warp instructions a line on the 1e7-line ExoMol list). on: this
+// lane's line is zoned; [q0, q1]: its zone inside its window (span positions).
+template <bool NU>
+__device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int qb, bool cut, const LineK& k, float e,
+                                           float f, float dnu_f, const float2* Drow, int lane, float* zacc) {
+  const bool small = k.y < ROX_Y_CORE;
+  const float y2 = k.y * k.y;
+  float c[16];
+#pragma unroll
+  for (int i = 0; i < 16; i++)
+    c[i] = rox_core_coef_r(y2, rox_core_r[i][0], rox_core_r[i][1], rox_core_r[i][2], rox_core_r[i][3]);
+  if (__any_sync(0xffffffffu, on && !small)) {
+    const int row = rox_core_row(k.y);
+    const float t = rox_core_arg(row, k.y);
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const float v = rox_core_coef(row, t, i);
+      c[i] = small ? c[i] : v;
+    }
+  }
+  const float g2 = k.iG * k.iG;
+  const f32x2 gU = f2_dup(g2 * rox_rcp(y2 + ROX_CORE_KAPPA));
+  // the Gaussian part: none above y = 0.1 (exponent 0, factor 0)
+  const f32x2 ge = f2_dup(small ? -ROX_LOG2E_F * g2 : 0.0f), ge0 = f2_dup(small ? ROX_LOG2E_F * y2 : 0.0f);
+  const f32x2 gc = f2_dup(small ? 4.0f * y2 * g2 : 0.0f), gp = f2_dup(small ? k.pc : 0.0f);
+  const f32x2 gy = f2_dup(small ? k.pc * k.y : k.pc);
+  const f32x2 ncf = f2_dup(-fmaf(k.tz, k.P, k.Q) * rox_rcp(fmaf(k.tz, k.tz, k.B)));
+  const float zt = on ? k.tz - k.A : -1.0f;                 // the zone: X^2 < t_z - A
+  const bool wide = __any_sync(0xffffffffu, on && k.zc < 1e38f);
+  const f32x2 ee = f2_dup(e), ff = f2_dup(f), dn = f2_dup(dnu_f), one = f2_dup(1.0f);
+  for (int q = qa & ~7; q <= qb; q += 8) {
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      f32x2 X;
+      if constexpr (NU) {
+        const float2 da = Drow[q + i], db = Drow[q + i + 1];
+        X = f2_pack((da.x - e) + (da.y - f), (db.x - e) + (db.y - f));
+      } else {
+        const float qf = (float)(q + i);
+        X = f2_fma(f2_add(f2_pack(qf, qf + 1.0f), ee), dn, ff);
+      }
+      const f32x2 x2 = f2_mul(X, X), U = f2_mul(x2, gU);
+      f32x2 n = f2_dup(c[7]), d = f2_dup(c[15]);
+#pragma unroll
+      for (int j = 6; j >= 0; j--) {
+        n = f2_fma(n, U, f2_dup(c[j]));
+        d = f2_fma(d, U, f2_dup(c[8 + j]));
+      }
+      float d0, d1, e0, e1, x0, x1;
+      f2_unpack(f2_fma(d, U, one), d0, d1);
+      f2_unpack(f2_fma(x2, ge, ge0), e0, e1);
+      const f32x2 u2 = f2_mul(x2, gc);
+      f32x2 g = f2_fma(u2, f2_dup(ROX_COS_C6), f2_dup(ROX_COS_C4));
+      g = f2_fma(u2, g, f2_dup(-0.5f));
+      g = f2_fma(u2, g, one);
+      f32x2 s = f2_fma(f2_pack(rox_exp2(e0), rox_exp2(e1)), f2_mul(g, gp), ncf);
+      s = f2_fma(f2_mul(n, f2_pack(rox_rcp(d0), rox_rcp(d1))), gy, s);
+      f2_unpack(s, v[i], v[i + 1]);
+      f2_unpack(x2, x0, x1);
+      if (wide) {
+        float w0, w1, n0, n1;
+        const f32x2 t = f2_add(x2, f2_dup(k.A));
+        f2_unpack(f2_fma(t, f2_dup(k.P), f2_dup(k.Q)), n0, n1);
+        f2_unpack(f2_fma(t, t, f2_dup(k.B)), w0, w1);
+        float c0, c1;
+        f2_unpack(ncf, c0, c1);
+        v[i] = x0 < k.zc ? v[i] : fmaf(n0, rox_rcp(w0), c0);
+        v[i + 1] = x1 < k.zc ? v[i + 1] : fmaf(n1, rox_rcp(w1), c1);
+      }
+      v[i] = x0 < zt ? v[i] : 0.0f;
+      v[i + 1] = x1 < zt ? v[i + 1] : 0.0f;
+      if (cut) {
+        v[i] = q + i >= q0 && q + i <= q1 ? v[i] : 0.0f;
+        v[i + 1] = q + i + 1 >= q0 && q + i + 1 <= q1 ? v[i + 1] : 0.0f;
+      }
+    }
+    const float r = warp_sum8(v, lane);
+    if ((lane & 3) == 0) zacc[q + (lane >> 2)] += r;
+  }
+}
+
+// ---- Window edges. A line whose window ends inside the span reaches only the points on one
+// side of its last (or first) point; at a cutoff many spans away its far form is as smooth there as a
+// cell's. Sorted by centre, such lines have sorted edges, so point j has the lines up to some i(j):
+// the lanes, one line each, form their moments about a common centre (the span's centre minus or
+// plus the cutoff), a warp scan turns them into running sums, and each point evaluates the sum
+// that belongs to it once. Per line about 8 warp instructions, where evaluating its points
+// under a mask took 95. The left lines (edge jhi) run through the list downwards, so that both sides
+// count points from the side the lines come from: key = Bw - jhi or jlo - Aw, non-decreasing.
+// Centre distances are one cutoff give or take the span's half-width; with (half-width + pole
+// modulus) / (cutoff - half-width) at most ROX_EDGE_R, ten terms err by 11 r^10 < 1e-7.
+#define ROX_EDGE_R 0.15f
+// points [k0, k1) of one side: their line's sum from the records rec[0 .. n_rec - 1] (n_rec 33, or 1 to take rec[0])
+template <bool NU>
+__device__ __forceinline__ void edge_points(const EdgeRec* rec, int n_rec, bool left, int k0, int k1, int lane,
+                                            float centre, float inv_cut, float dnu_f, const float2* Drow, float* zacc) {
+  for (int k = k0 + lane; k < k1; k += 32) {
+    int i = 0;                       // records 1 .. i have key <= k
+    if (n_rec > 1) {
+#pragma unroll
+      for (int st = 16; st > 0; st >>= 1)
+        if (rec[i + st].key <= k) i += st;
+      if (i == 31 && rec[32].key <= k) i = 32;
+    }
+    const EdgeRec& r = rec[i];
+    const int q = left ? ROX_SPAN - 1 - k : k;
+    const float y = ((NU ? Drow[q].x : (float)q * dnu_f) - centre) * inv_cut;
+    const float z = rox_rcp(y);
+    float f = r.m[ROX_EDGE_TERMS - 1];
+#pragma unroll
+    for (int l = ROX_EDGE_TERMS - 2; l >= 0; l--) f = fmaf(f, z, r.m[l]);
+    zacc[q] += z * z * f;
+  }
+}
+// one batch's lines of one side (mine: this lane's line is one of them, at d = offset of its centre from
+// `centre` in cutoffs): kcur is the side's first point without its final sum
+template <bool NU>
+__device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left, bool mine, int key, float d,
+                                           const LineK& k, int& kcur, int lane, float centre, float inv_cut,
+                                           float dnu_f, const float2* Drow, float* zacc) {
+  const float i2 = inv_cut * inv_cut, i4 = i2 * i2;
+  const float pu = mine ? k.P * i2 : 0.f, qu = mine ? k.Q * i4 : 0.f, bu = mine ? k.B * i4 : 0.f;
+  const float dd = mine ? d : 0.f, e = fmaf(dd, dd, mine ? k.A * i2 : 0.f);
+  const float d3 = 4.0f * dd, d2 = -fmaf(d3, dd, 2.0f * e), d1 = d3 * e, d0 = -fmaf(e, e, bu);
+  float m[ROX_EDGE_TERMS];
+  m[0] = pu;
+  m[1] = 2.0f * pu * dd;
+  m[2] = fmaf(d3, m[1], fmaf(d2, m[0], fmaf(pu, e, qu)));
+  m[3] = fmaf(d3, m[2], fmaf(d2, m[1], d1 * m[0]));
+#pragma unroll
+  for (int l = 4; l < ROX_EDGE_TERMS; l++) m[l] = fmaf(d3, m[l - 1], fmaf(d2, m[l - 2], fmaf(d1, m[l - 3], d0 * m[l - 4])));
+  int kk = mine ? key : -1;
+  __syncwarp();                      // the tables of the batch before are no longer read
+  if (lane == 0) {
+#pragma unroll
+    for (int l = 0; l < ROX_EDGE_TERMS; l++) {
+      const float c = carry[l];
+      rec[0].m[l] = c;
+      m[l] += c;
+    }
+    rec[0].key = -1;
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int ko = __shfl_up_sync(0xffffffffu, kk, o);
+    kk = lane >= o ? max(kk, ko) : kk;
+#pragma unroll
+    for (int l = 0; l < ROX_EDGE_TERMS; l++) {
+      const float t = __shfl_up_sync(0xffffffffu, m[l], o);
+      if (lane >= o) m[l] += t;
+    }
+  }
+#pragma unroll
+  for (int l = 0; l < ROX_EDGE_TERMS; l++) rec[lane + 1].m[l] = m[l];
+  rec[lane + 1].key = kk;
+  if (lane == 31) {
+#pragma unroll
+    for (int l = 0; l < ROX_EDGE_TERMS; l++) carry[l] = m[l];
+  }
+  __syncwarp();
+  const int klast = min(__shfl_sync(0xffffffffu, kk, 31), ROX_SPAN);
+  edge_points<NU>(rec, 33, left, kcur, klast, lane, centre, inv_cut, dnu_f, Drow, zacc);
+  kcur = max(kcur, klast);
+  __syncwarp();
 }
 
 // Grid indices of a line's slow zone on a uniform grid, |j - (k0 + f)| < hz / dnu, widened by 1e-4
@@ -676,15 +883,15 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
 // extra is compiled only into the instantiations that use it: in this kernel even a few added
 // instructions per line batch cost several percent of the plain launch.
 template <bool NU, int X, int W>
-__global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant__ RoxVoigtArgs A) {
+__global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant__ RoxVoigtArgs A) {
   constexpr bool IDX = (X & ROX_VX_INDEX) != 0;
   constexpr bool BRD = (X & ROX_VX_BROAD) != 0;
   constexpr bool PRE = (X & ROX_VX_PRE) != 0;
   extern __shared__ __align__(16) float2 s_nodes[];   // NU: node offsets; PRE: the staged per-line constants
   __shared__ float4 s_geo[W][32];
   __shared__ float s_S[PRE ? 1 : W][32];
-  __shared__ PairTab s_pairs[W];
-  __shared__ LineTab s_lines[W];
+  __shared__ __align__(16) unsigned char s_tab[W][sizeof(BatchTab)];
+  __shared__ __align__(16) float s_carry[W][2][12];   // moments of the edge lines so far, per side
   __shared__ __align__(8) float s_zacc[W][ROX_SPAN];
   __shared__ float s_tot[W][ROX_SPAN];    // the span's sum over its parts
   __shared__ float s_part[W][2][ROX_SPAN];  // a part's sum and its compensation
@@ -699,15 +906,18 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
 
   float4* geo_st = s_geo[w];   // this lane's line of the batch; the next batch's copy starts once it is read
   float* S_st = s_S[PRE ? 0 : w];
-  PairTab& PT = s_pairs[w];
-  LineTab& LT = s_lines[w];
+  BatchTab& BT = *reinterpret_cast<BatchTab*>(s_tab[w]);
+  PairTab& PT = BT.pairs;
+  LineTab& LT = BT.lines;
   const float lanef = (float)lane;
   const float cheb = rox_cheb_x[lane];
   float* zacc = s_zacc[w];
   float* stot = s_tot[w];
   float *part_tot = s_part[w][0] + lane, *part_cmp = s_part[w][1] + lane;   // [32 m]: this lane's points
   f32x2* cbuf = s_cf[w];
-  const float4 core_r = *reinterpret_cast<const float4*>(rox_core_r[lane & 15]);
+  float* carry = s_carry[w][0];
+  const float* cr = rox_core_r[lane & 15];
+  const float4 core_r = make_float4(cr[0], cr[1], cr[2], cr[3]);
   float2* Drow = NU ? s_nodes + w * ROX_SPAN : nullptr;   // this span's node offsets
   // PRE: per warp 32 lines x 3 float4 of per-line constants
   float4(*rec_st)[3] = PRE ? reinterpret_cast<float4(*)[3]>(s_nodes) + 32 * w : nullptr;
@@ -759,6 +969,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
     }
     const float half = NU ? 0.5f * Ws : 0.5f * (ROX_SPAN - 1) * dnu_f;
     const float tau = NU ? fmaf(cheb, half, half) : fmaf(cheb, 0.5f * (ROX_SPAN - 1), 0.5f * (ROX_SPAN - 1));
+    const float inv_cut = rox_rcp(Lst.cutoff_f);
     float ntot = 0.f;   // whole items: this lane's Chebyshev point, over the parts
     const int lo = (int)max(Lst.span_lo[span], J.l0), hi = (int)min(Lst.span_hi[span], J.l1);   // at most 2e9 lines
     const int wlo = (int)max(J.first, (long long)Aw);              // evaluated points of this span
@@ -807,8 +1018,24 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
       }
       if (part <= 0 && lane == 0) evals += (unsigned long long)((long long)(xb - xa) + (xd - xc)) * (unsigned)(whi - wlo + 1);
     }
+    // without cells on the left the list is cut at the span's centre, so that the lines left of it
+    // can run downwards (their window edges then come in order, see edge_batch)
+    if (cl1 <= cl0 && hi > lo) {
+      const float mid = NU ? bh + half : (float)(Aw + ROX_SPAN / 2);
+      int a = lo, len = hi - lo;
+      while (len > 0) {
+        const int step = (len + 31) >> 5, off = lane * step;
+        const bool less = off < len && cell_k0(Lst, a + off) < mid;
+        const int c = __popc(__ballot_sync(0xffffffffu, less));
+        if (c == 0) break;
+        const int na = a + (c - 1) * step + 1;
+        len = min(step - 1, a + len - na);
+        a = na;
+      }
+      xa = xb = min(a, xc);
+    }
     const int n1 = xa - lo, n2 = n1 + (xc - xb), nn = n2 + max(hi - xd, 0);   // lines visited one by one
-    auto line_at = [&](int q) { return q < n1 ? lo + q : (q < n2 ? xb + (q - n1) : xd + (q - n2)); };
+    auto line_at = [&](int q) { return q < n1 ? xa - 1 - q : (q < n2 ? xb + (q - n1) : xd + (q - n2)); };
     const int n_far = (cl1 - cl0) + (cr1 - cr0);
 
     const int nbat = (nn + 31) >> 5;
@@ -818,6 +1045,9 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
       const int phi = min(nn, 32 * ((nbat * (p + 1)) / ROX_PARTS));
       // the part's total and its compensation: in shared memory (touched once in four batches),
       // Chebyshev point in nsum, ncmp
+      int ekL = 0, ekR = 0;             // edge lines: first point without its final sum, per side
+      bool edgeL = false, edgeR = false;
+      if (lane < 24) carry[lane] = 0.f;
       float acc[ROX_K], nacc = 0.f, nsum = 0.f, ncmp = 0.f;
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
@@ -859,6 +1089,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
         bool covers = false, zoned = false, smooth = false;
         float ax = 0.f, ay = 0.f, vA = 1.f, vB = 0.f, vP = 0.f, vQ = 0.f, tz = 0.f;
         float4 zl = make_float4(1.f, 0.f, 0.f, 0.f);
+        LineK kk = {1.f, 1.f, 0.f, 0.f, 1.f, 1.f, 0.f, 0.f, 3e38f, 0.f};
         int jlo = 1, jhi = 0, zlo = 0, zhi = -1;
         if (live) {
           const float4 g = geo_st[lane];
@@ -906,13 +1137,24 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
               // the span's offsets run from -c to Ws - c; pass 2 then scans the window itself
               const float hzp = kc.hz * 1.001f + 1e-6f * (fabsf(ax) + Ws);
               zoned = -ax < hzp && Ws - ax > -hzp;
-              zlo = jlo;
-              zhi = jhi;
             } else {
               zone_bounds(g, kc.hz, Lst.inv_dnu_f, zlo, zhi);
               zoned = !(Bw < zlo || Aw > zhi);
             }
             dmin = smooth_dmin(kc.A, kc.B, half);
+          }
+          if constexpr (NU) {
+            if (zoned) {   // the span's nodes within the zone, by bisection on their offsets (widened a little)
+              const float hb = kc.hz * 1.001f + 1e-6f * (fabsf(ax) + Ws);
+              int q0 = 0, q1 = 0;
+#pragma unroll
+              for (int st = ROX_SPAN / 2; st > 0; st >>= 1) {
+                if (Drow[q0 + st - 1].x - ax < -hb) q0 += st;
+                if (Drow[q1 + st - 1].x - ax <= hb) q1 += st;
+              }
+              zlo = Aw + q0;
+              zhi = Aw + q1;      // one past, at most: harmless, each point has its own test
+            }
           }
           const float D = NU ? half - ax - ay : fmaf(ax + 0.5f * (ROX_SPAN - 1), dnu_f, ay);
           smooth = covers && !zoned && fabsf(D) >= dmin;
@@ -922,18 +1164,55 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           vQ = kc.Q;
           tz = kc.tz;
           zl = make_float4(kc.iG, kc.y, kc.pc, kc.zc);
+          kk = kc;
+        }
+        // ---- pass 2, all zoned lines of the batch at once where they lie close enough together: at
+        // the points each zoned line has clamped in pass 1, the Faddeeva form
+        int q0 = max(max(zlo, jlo) - Aw, 0), q1 = min(min(zhi, jhi) - Aw, ROX_SPAN - 1);
+        zoned = zoned && live;
+        const bool on = zoned && q0 <= q1;
+        const int nz = __popc(__ballot_sync(0xffffffffu, on));
+        bool batched = false;
+        if (nz > 0) {
+          const int qa = __reduce_min_sync(0xffffffffu, on ? q0 : ROX_SPAN), qb = __reduce_max_sync(0xffffffffu, on ? q1 : -1);
+          batched = qb - qa + 1 <= ROX_ZONE_DENSE * nz;
+          if (batched)
+            zone_batch<NU>(on, q0, q1, qa, qb, __any_sync(0xffffffffu, on && (jlo > zlo || jhi < zhi)), kk, ax, ay, dnu_f,
+                           Drow, lane, zacc);
+        }
+        // ---- window edges in order, where the lines are smooth on the span
+        bool scanned = false;
+        {
+          const bool eL = live && !covers && !zoned && jlo <= Aw && jhi < Bg, eR = live && !covers && !zoned && jlo > Aw && jhi >= Bg;
+          if (__any_sync(0xffffffffu, eL || eR)) {
+            const float cL = half - Lst.cutoff_f, cR = half + Lst.cutoff_f;   // from the span's first point
+            const float v = NU ? ax + ay : -fmaf(ax, dnu_f, ay);              // the line, from there
+            const float bm = fabsf(kk.B) + 1e-30f, r2 = fabsf(kk.A) + bm * rox_rsqrt(bm) + 1e-30f;
+            const float dL = v - cL, dR = v - cR, room = ROX_EDGE_R * (Lst.cutoff_f - half) - r2 * rox_rsqrt(r2);
+            const bool mL = eL && fabsf(dL) <= room, mR = eR && fabsf(dR) <= room;
+            if (__any_sync(0xffffffffu, mL)) {
+              edgeL = true;
+              edge_batch<NU>(BT.scan, carry, true, mL, Bw - jhi, dL * inv_cut, kk, ekL, lane, cL, inv_cut, dnu_f, Drow, zacc);
+            }
+            if (__any_sync(0xffffffffu, mR)) {
+              edgeR = true;
+              edge_batch<NU>(BT.scan, carry + 12, false, mR, jlo - Aw, dR * inv_cut, kk, ekR, lane, cR, inv_cut, dnu_f, Drow, zacc);
+            }
+            scanned = mL || mR;
+          }
         }
         const unsigned msm = __ballot_sync(0xffffffffu, live && smooth);
         const unsigned clean = __ballot_sync(0xffffffffu, live && covers && !zoned && !smooth);
         const unsigned czone = __ballot_sync(0xffffffffu, live && covers && zoned);
-        const unsigned edge = __ballot_sync(0xffffffffu, live && !covers);
+        const unsigned edge = __ballot_sync(0xffffffffu, live && !covers && !scanned);
         const int nsm = __popc(msm), nclean = nsm + __popc(clean), ncov = nclean + __popc(czone);
+        const int nslot = ncov + __popc(edge);
         const unsigned below = (1u << lane) - 1u;
         const int slot = !covers ? ncov + __popc(edge & below)
                          : zoned ? nclean + __popc(czone & below)
                          : smooth ? __popc(msm & below) : nsm + __popc(clean & below);
-        const unsigned zslots = __reduce_or_sync(0xffffffffu, (live && zoned) ? (1u << slot) : 0u);
-        if (live) {
+        const unsigned zslots = __reduce_or_sync(0xffffffffu, (on && !batched) ? (1u << slot) : 0u);
+        if (live && !scanned) {
           const int k = slot >> 1, h = slot & 1;
           float* ab = reinterpret_cast<float*>(&PT.ab[k]);
           float* pq = reinterpret_cast<float*>(&PT.pq[k]);
@@ -960,11 +1239,11 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
         for (int k = 0; k < ks; k++) nacc = smooth_pair<NU>(PT, k, tau, dnu_f, nacc);
         for (int k = ks; k < kc; k++) cover_pair<NU, false>(PT, k, lanef, dnu_f, D, acc);
         for (int k = kc; k < kz; k++) cover_pair<NU, true>(PT, k, lanef, dnu_f, D, acc);
-        for (int s2 = 2 * kz; s2 < cnt; s2 += 2) {
-          if (s2 + 1 < cnt) edge_pair<NU>(PT, LT, s2 >> 1, Aw, lane, lanef, dnu_f, D, acc);
+        for (int s2 = 2 * kz; s2 < nslot; s2 += 2) {
+          if (s2 + 1 < nslot) edge_pair<NU>(PT, LT, s2 >> 1, Aw, lane, lanef, dnu_f, D, acc);
           else edge_line<NU>(PT, LT, s2, Aw, lane, lanef, dnu_f, D, acc);
         }
-        // ---- pass 2: at the points each zoned line had clamped, the full Faddeeva forms
+        // ---- pass 2 line by line otherwise
         for (unsigned z = zslots; z; z &= z - 1)
           zone_line<NU>(PT, LT, __ffs(z) - 1, Aw, lane, dnu_f, core_r, D, cbuf, zacc);
         __syncwarp();
@@ -986,6 +1265,14 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_voigt(const __grid_constant_
           nacc = 0.f;
         }
       }
+      // edge lines: the points beyond the last edge have all of the part's lines of that side
+      __syncwarp();
+#pragma unroll 1
+      for (int side = 0; side < 2; side++)
+        if (side ? edgeR : edgeL)
+          edge_points<NU>(reinterpret_cast<const EdgeRec*>(carry + 12 * side), 1, side == 0, side ? ekR : ekL, ROX_SPAN, lane,
+                          side ? half + Lst.cutoff_f : half - Lst.cutoff_f, inv_cut, dnu_f, Drow, zacc);
+      __syncwarp();
       // this part's share of the far cells, at this lane's Chebyshev point
       for (int c = n_far * p / ROX_PARTS; c < n_far * (p + 1) / ROX_PARTS; c++) {
         const int cell = c < cl1 - cl0 ? cl0 + c : cr0 + (c - (cl1 - cl0));
