@@ -21,8 +21,6 @@ cudaError_t rox_launch_widths(const rox_lines* L, double mass_amu, double P_bar,
 cudaError_t rox_launch_strengths_multi(const rox_lines* L, int n_temps, const double* temps,
                                        const double* q_of_temp, double Q_ref, double* S_T,
                                        unsigned long long* smax_bits, bool exact, cudaStream_t s);
-cudaError_t rox_launch_scale_strengths(const double* S_T, long long n, int n_temps,
-                                       const unsigned long long* smax_bits, float* S32, cudaStream_t s);
 cudaError_t rox_launch_windows(const double* nu0, long long n_lines, const rox_grid* g, double cutoff,
                                int32_t* jlo, int32_t* jhi, int32_t* k0, float* f, float4* geo,
                                unsigned long long* evals, int32_t* unsorted, int32_t unsorted_value,
@@ -45,7 +43,12 @@ cudaError_t rox_launch_node_offsets(const double* nodes, long long n, long long 
 void rox_fill_strength_consts(int convention, double T, double Q_T, double Q_ref, RoxStrengthJob* jb);
 cudaError_t rox_launch_strengths_jobs(const RoxStrengthJobs& J, long long max_count, cudaStream_t s);
 cudaError_t rox_voigt_blocks_per_sm(int* nb, bool nodes, bool pre, int warps);
-cudaError_t rox_launch_line_params(const RoxListDev& L, const RoxJobDev& J, float4* rec, cudaStream_t s);
+cudaError_t rox_launch_prep_lines(const rox_lines* L, const rox_grid* g, double cutoff, int n_temps, const double* temps,
+                                  const double* q_of_temp, double Q_ref, double* S_T, RoxWsHeader* hdr, float4* geo,
+                                  cudaStream_t s);
+cudaError_t rox_launch_prep_scaled(const RoxListDev& L, const RoxJobDev& J, long long n, int n_temps, const double* S_T,
+                                   const RoxWsHeader* hdr, float* S32, const float4* geo, long long n_spans,
+                                   long long* lo, long long* hi, float4* rec, cudaStream_t s);
 cudaError_t rox_launch_select(const double* nu0, const double* S_T, long long n, int n_temps,
                               const unsigned long long* smax_bits, double origin, double width, long long n_bins,
                               double rel, int32_t* bin, unsigned long long* binmax_bits, float* S32, cudaStream_t s);
@@ -164,6 +167,7 @@ struct WsLayout {
   float* tail_part;
   int32_t* tail_cnt;
   long long tail_cap;
+  size_t clear_bytes;  // header and tail counters
   float2* node_d;      // user-provided nodes only: [n_tiles * ROX_SPAN] offsets, [n_tiles] bases
   float2* span_base;
   int32_t* line_bin;   // main-contributor selection only: [n_lines] bins, [n_temps][n_bins] maxima,
@@ -191,9 +195,13 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
   size_t off = 0;
   w.hdr = (RoxWsHeader*)(base + off);
   off += ROX_WS_HEADER_BYTES;
+  long long nt = n_tiles_of(n_grid);
+  w.tail_cap = nt < tail_max ? nt : tail_max;
+  w.tail_cnt = (int32_t*)(base + off);         // next to the header: one memset clears both
+  off += rox_align256((size_t)w.tail_cap * 4);
+  w.clear_bytes = off;
   w.geo = (float4*)(base + off);
   off += rox_align256((size_t)(n_lines > 0 ? n_lines : 1) * sizeof(float4));
-  long long nt = n_tiles_of(n_grid);
   w.tlo = (long long*)(base + off);
   off += rox_align256((size_t)nt * 8);
   w.thi = (long long*)(base + off);
@@ -202,10 +210,8 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
   off += rox_align256((size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 8);
   w.S32 = (float*)(base + off);
   off += rox_align256((size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 4);
-  w.tail_cap = nt < tail_max ? nt : tail_max;
   w.tail_part = (float*)(base + off);
-  w.tail_cnt = (int32_t*)(base + off + rox_tail_part_bytes(w.tail_cap));
-  off += rox_tail_bytes(w.tail_cap);
+  off += rox_tail_part_bytes(w.tail_cap);
   w.node_d = nullptr;
   w.span_base = nullptr;
   if (nodes) {
@@ -377,7 +383,7 @@ long long job_cells(RoxJobDev* J, int32_t c_steps) {
 // up to tail_cap and half a round of the launch's warps, are split into their parts.
 int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* jobs, int n_jobs, RoxWsHeader* hdr,
                       float* tail_part, int32_t* tail_cnt, long long tail_cap, const RoxMoments& mom, int nblocks,
-                      cudaStream_t s, const rox_launch_config& cfg, bool nodes = false, int extras = 0) {
+                      cudaStream_t s, const rox_launch_config& cfg, bool nodes = false, int extras = 0, bool cleared = true) {
   static thread_local RoxVoigtArgs A;   // ~30 KB of per-job parameters, passed by value
   A.hdr = hdr;
   A.tail_part = tail_part;
@@ -400,10 +406,10 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
       A.item_end[nj] = items;
     }
     A.n_slots = (int32_t)slots;
-    const int blocks = items < nblocks ? items : nblocks;
+    A.cells_task = slots < 152 * 64 ? 1 : 4;
     // whole items in complete rounds of the launch's warps, then at least one round of items in
     // parts, so the launch ends in pieces of 1/ROX_PARTS of an item
-    const long long warps = (long long)blocks * cfg.warps_per_cta;
+    const long long warps = (long long)nblocks * cfg.warps_per_cta;
     long long split = items <= warps ? items : items % warps + (long long)cfg.split_rounds * warps;
     if (split > items) split = items;
     if (split > tail_cap) split = tail_cap;
@@ -411,9 +417,14 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
     A.n_items = items;
     A.n_whole = items - (int)split;
     A.n_queue = A.n_whole + (int)split * ROX_PARTS;
+    const long long need = ((long long)A.n_queue + cfg.warps_per_cta - 1) / cfg.warps_per_cta;
+    const int blocks = need < nblocks ? (int)need : nblocks;
     int rc;
-    if ((rc = cuda_check(cudaMemsetAsync(&hdr->work_counter, 0, sizeof(int32_t), s), "memset"))) return rc;
-    if (split > 0 && (rc = cuda_check(cudaMemsetAsync(tail_cnt, 0, (size_t)split * 4, s), "memset"))) return rc;
+    if (!cleared) {   // the call's first launch finds the work counter and the split items' counters clear
+      if ((rc = cuda_check(cudaMemsetAsync(&hdr->work_counter, 0, sizeof(int32_t), s), "memset"))) return rc;
+      if (split > 0 && (rc = cuda_check(cudaMemsetAsync(tail_cnt, 0, (size_t)split * 4, s), "memset"))) return rc;
+    }
+    cleared = false;
     if (j0 == 0 && g_prof_start && (rc = cuda_check(cudaEventRecord(g_prof_start, s), "cudaEventRecord"))) return rc;
     if (items == 0) continue;
     if ((rc = cuda_check(rox_launch_moments(A, extras, s), "moments kernel"))) return rc;
@@ -577,29 +588,32 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
   const long long nt = n_tiles_of(n_grid);
   const long long nl = lines->n;
 
-  if ((rc = cuda_check(cudaMemsetAsync(w.hdr, 0, sizeof(RoxWsHeader), s), "memset"))) return rc;
+  if ((rc = cuda_check(cudaMemsetAsync(w.hdr, 0, w.clear_bytes, s), "memset"))) return rc;
   if (on_nodes &&
       (rc = cuda_check(rox_launch_node_offsets(nodes->nu, nodes->n, nt * ROX_SPAN, w.node_d, w.span_base,
                                                &w.hdr->status, ROX_EGRID, s),
                        "node offsets kernel")))
     return rc;
   if (nl > 0) {
-    const cudaError_t we =
-        on_nodes ? rox_launch_node_windows(lines->nu0, nl, nodes->nu, nodes->n, cutoff, nullptr, nullptr, w.geo,
-                                           &w.hdr->evals_lines, &w.hdr->status, ROX_EUNSORTED, s)
-                 : rox_launch_windows(lines->nu0, nl, grid, cutoff, nullptr, nullptr, nullptr, nullptr, w.geo,
-                                      &w.hdr->evals_lines, &w.hdr->status, ROX_EUNSORTED, s);
-    if ((rc = cuda_check(we, "windows kernel"))) return rc;
-    if ((rc = cuda_check(rox_launch_strengths_multi(lines, n_temps, temps.data(), qs.data(), Q_ref, w.S_T,
-                                                    w.hdr->smax_bits, false, s),
-                         "strengths kernel")))
+    if (on_nodes) {
+      if ((rc = cuda_check(rox_launch_node_windows(lines->nu0, nl, nodes->nu, nodes->n, cutoff, nullptr, nullptr, w.geo,
+                                                   &w.hdr->evals_lines, &w.hdr->status, ROX_EUNSORTED, s),
+                           "node windows kernel")))
+        return rc;
+      if ((rc = cuda_check(rox_launch_strengths_multi(lines, n_temps, temps.data(), qs.data(), Q_ref, w.S_T,
+                                                      w.hdr->smax_bits, false, s),
+                           "strengths kernel")))
+        return rc;
+    } else if ((rc = cuda_check(rox_launch_prep_lines(lines, grid, cutoff, n_temps, temps.data(), qs.data(), Q_ref, w.S_T,
+                                                      w.hdr, w.geo, s),
+                                "windows and strengths kernel"))) {
       return rc;
-    const cudaError_t se =
-        sel ? rox_launch_select_reduced(lines, n_temps, temps.data(), qs.data(), Q_ref, w.S_T, w.hdr->smax_bits,
-                                        sel_origin, sel->bin_width, n_bins, sel->rel, w.line_bin, w.binmax,
-                                        w.binmax_exact, w.S32, s)
-            : rox_launch_scale_strengths(w.S_T, nl, n_temps, w.hdr->smax_bits, w.S32, s);
-    if ((rc = cuda_check(se, "strength scaling kernel"))) return rc;
+    }
+    if (sel && (rc = cuda_check(rox_launch_select_reduced(lines, n_temps, temps.data(), qs.data(), Q_ref, w.S_T,
+                                                          w.hdr->smax_bits, sel_origin, sel->bin_width, n_bins, sel->rel,
+                                                          w.line_bin, w.binmax, w.binmax_exact, w.S32, s),
+                                "selection kernels")))
+      return rc;
     if (sel) {
       // per temperature the kept lines as an index into the sorted list, and span ranges over it
       if ((rc = cuda_check(rox_launch_compact(w.S32, nl, n_temps, w.keep_flags, w.keep_idx, w.keep_count,
@@ -618,8 +632,6 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
                                "broadening kernel")))
       return rc;
   }
-  if ((rc = cuda_check(rox_launch_tile_ranges_geo(w.geo, nl, nt, ROX_TILE, w.tlo, w.thi, s), "tile ranges")))
-    return rc;
   RoxListDev L0;
   L0.status = &w.hdr->status;
   L0.geo = w.geo;
@@ -654,6 +666,7 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
     J.list = 0;
     J.span_first = 0;
     J.n_spans = (int32_t)nt;
+    J.part_shift = nt >= ROX_MANY_SPANS ? ROX_PART_SHIFT : 0;
     J.p_fac = (float)(P_bar[k] / ROX_P_REF);
     J.gG_fac = (float)(sqrt(2.0 * ROX_KB * T[k] / (mass_amu * ROX_AMU)) / ROX_C_M);
     J.l2_ratio = (float)log2(ROX_T_REF / T[k]);
@@ -678,12 +691,15 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
           jg.back().list = tidx[k] - g0;
         }
       if ((rc = launch_voigt_jobs(Ls, ng, jg.data(), (int)jg.size(), w.hdr, w.tail_part, w.tail_cnt, w.tail_cap,
-                                  w.mom, nblocks, s, cfg, false, ROX_VX_INDEX)))
+                                  w.mom, nblocks, s, cfg, false, ROX_VX_INDEX, g0 == 0)))
         return rc;
     }
     return ok();
   }
-  if (pre && (rc = cuda_check(rox_launch_line_params(L0, jobs[0], w.rec, s), "line parameter kernel"))) return rc;
+  if ((rc = cuda_check(rox_launch_prep_scaled(L0, jobs[0], nl, nl > 0 ? n_temps : 1, w.S_T, w.hdr, w.S32, w.geo, nt, w.tlo,
+                                              w.thi, pre ? w.rec : nullptr, s),
+                       "scaling and span ranges kernel")))
+    return rc;
   const int extras = br ? ROX_VX_BROAD : (pre ? ROX_VX_PRE : 0);
   if ((rc = launch_voigt_jobs(&L0, 1, jobs.data(), n_pt, w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, w.mom, nblocks, s,
                               cfg, on_nodes, extras)))
@@ -914,17 +930,12 @@ struct JobsTail {
   float* part;
   int32_t* cnt;
   long long cap;
+  size_t clear_bytes;      // header and counters
   RoxMoments mom;
 };
 size_t jobs_layout(const rox_job* jobs, int n_jobs, void* ws, double** S64, float** S32, JobsTail* tail) {
-  size_t off = ROX_WS_HEADER_BYTES;
   long long spans = 0, slots = 0;
   for (int k = 0; k < n_jobs; k++) {
-    const size_t c = (size_t)(jobs[k].line_count > 0 ? jobs[k].line_count : 1);
-    if (S64) S64[k] = (double*)((char*)ws + off);
-    off += rox_align256(c * 8);
-    if (S32) S32[k] = (float*)((char*)ws + off);
-    off += rox_align256(c * 4);
     if (jobs[k].n > 0 && jobs[k].first >= 0) {
       const long long ns = (jobs[k].first + jobs[k].n - 1) / ROX_SPAN - jobs[k].first / ROX_SPAN + 1;
       spans += ns;
@@ -932,12 +943,21 @@ size_t jobs_layout(const rox_job* jobs, int n_jobs, void* ws, double** S64, floa
     }
   }
   const long long cap = spans < ROX_TAIL_ITEMS_MAX ? spans : ROX_TAIL_ITEMS_MAX;
+  size_t off = ROX_WS_HEADER_BYTES + rox_align256((size_t)cap * 4);     // counters next to the header
+  if (tail) tail->clear_bytes = off;
+  for (int k = 0; k < n_jobs; k++) {
+    const size_t c = (size_t)(jobs[k].line_count > 0 ? jobs[k].line_count : 1);
+    if (S64) S64[k] = (double*)((char*)ws + off);
+    off += rox_align256(c * 8);
+    if (S32) S32[k] = (float*)((char*)ws + off);
+    off += rox_align256(c * 4);
+  }
   if (tail) {
     tail->cap = cap;
     tail->part = (float*)((char*)ws + off);
-    tail->cnt = (int32_t*)((char*)ws + off + rox_tail_part_bytes(cap));
+    tail->cnt = (int32_t*)((char*)ws + ROX_WS_HEADER_BYTES);
   }
-  off += rox_tail_bytes(cap);
+  off += rox_tail_part_bytes(cap);
   if (tail) tail->mom = moments_at((char*)ws + off, slots);
   off += rox_mom_bytes(slots);
   return off;
@@ -985,7 +1005,7 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
   std::vector<float*> S32(n_jobs);
   JobsTail tail;
   jobs_layout(jobs, n_jobs, ws, S64.data(), S32.data(), &tail);
-  if ((rc = cuda_check(cudaMemsetAsync(hdr, 0, sizeof(RoxWsHeader), s), "memset"))) return rc;
+  if ((rc = cuda_check(cudaMemsetAsync(hdr, 0, tail.clear_bytes, s), "memset"))) return rc;
 
   // strengths of every job's line range at its temperature
   static thread_local RoxStrengthJobs SJ;
@@ -1056,6 +1076,7 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     d.list = j.list;
     d.span_first = (int32_t)(j.first / ROX_SPAN);
     d.n_spans = (int32_t)((j.first + j.n - 1) / ROX_SPAN - j.first / ROX_SPAN + 1);
+    d.part_shift = d.n_spans >= ROX_MANY_SPANS ? ROX_PART_SHIFT : 0;
     d.p_fac = (float)(j.P_bar / ROX_P_REF);
     d.gG_fac = (float)(sqrt(2.0 * ROX_KB * j.T / (j.mass_amu * ROX_AMU)) / ROX_C_M);
     d.l2_ratio = (float)log2(ROX_T_REF / j.T);

@@ -131,11 +131,15 @@ struct RoxJobDev {
   int32_t t_row;    // broadened lists: the job's temperature row of the list's gLT
   int32_t mom_off;  // the job's first slot in RoxVoigtArgs::mom and cstart (a multiple of 4)
   int32_t c_first;  // the cell of that slot
+  int32_t part_shift;  // a span's parts: its batches of lines >> part_shift, 1 .. ROX_PARTS
   int32_t n_cells;  // cells with moments (slot n_cells holds only the first line beyond them); 0: none
 };
 
-// Every span's lines are summed as ROX_PARTS consecutive parts (batch-aligned), each from
-// zero, and the part sums are added in part order. A work item is normally a whole span; the
+// Every span's lines are summed as up to ROX_PARTS consecutive parts (batch-aligned), each from
+// zero, and the part sums are added in part order. How many is fixed by the job and the span: a job of
+// many spans fills the GPU with whole items and takes a part per 2^part_shift batches (a part's
+// fixed work, some 400 instructions and the wait for its first batch, is not worth less), a short one a
+// part per batch. A work item is normally a whole span; the
 // last items of a launch are split into their parts, taken by different warps: each part stores
 // its sum in the tail scratch and the last of them to finish adds the parts in the same order.
 // The result is the same either way, so it depends neither on the split nor on the launch grid.
@@ -143,6 +147,8 @@ struct RoxJobDev {
 // the launch's warps and the split ones end the launch in pieces of 1/ROX_PARTS of an item
 // (at most ROX_TAIL_ITEMS_MAX items, the size of the workspace's tail scratch).
 #define ROX_PARTS 16
+#define ROX_MANY_SPANS 2048
+#define ROX_PART_SHIFT 4
 #define ROX_TAIL_ITEMS_MAX 8192
 // A part's sum: its ROX_SPAN points, then its values at the span's ROX_NODES Chebyshev points
 // (the lines that are smooth on the span, rox_voigt.cu)
@@ -156,6 +162,7 @@ struct RoxVoigtArgs {
   float4* mom;                      // [slots][4] moments of the jobs' cells
   int32_t* cstart;                  // [slots] first line (position) of each cell
   int32_t n_jobs;
+  int32_t cells_task;               // cells a warp of k_moments takes at a time: 4, or 1 in small launches
   int32_t n_slots;                  // slots over all jobs (0: no moments in this launch)
   int32_t n_items;                  // items (spans over all jobs); the last n_items - n_whole split
   int32_t n_whole;
@@ -200,8 +207,8 @@ static inline long long rox_job_slots(long long n_spans) {
 static inline size_t rox_mom_bytes(long long slots) {
   return rox_align256((size_t)slots * 64) + rox_align256((size_t)slots * 4);
 }
-// tail scratch of a workspace: `cap` items x ROX_PARTS x ROX_PART_FLOATS floats, then cap counters
+// tail scratch of a workspace: `cap` items x ROX_PARTS x ROX_PART_FLOATS floats (the items' counters
+// lie next to the header)
 static inline size_t rox_tail_part_bytes(long long cap) {
   return rox_align256((size_t)cap * ROX_PARTS * ROX_PART_FLOATS * sizeof(float));
 }
-static inline size_t rox_tail_bytes(long long cap) { return rox_tail_part_bytes(cap) + rox_align256((size_t)cap * 4); }

@@ -30,12 +30,11 @@
 // per 32-point sub-span where possible, accumulated in warp-private shared memory.
 #include <cuda_fp16.h>
 #include "rox_internal.cuh"
-#include "rox_faddeeva.cuh"
+#include "rox_lines.cuh"
 #include "rox_interp_table.h"   // generated by gen_interp_table.py
 
 namespace {
 
-#define ROX_INV_PI 0.318309886183790672f
 
 // Per-line constants of one (P,T) point for the batch in hand. Each line has a slot; slots are
 // ordered by class -- lines whose window covers the whole span and whose slow zone misses it
@@ -88,25 +87,6 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-__device__ __forceinline__ float load_width(const void* p, int f16, long long i) {
-  return f16 ? __half2float(reinterpret_cast<const __half*>(p)[i])
-             : reinterpret_cast<const float*>(p)[i];
-}
-
-// the two per-line width inputs of line i: {gamma_ref, n_T} of the single power law, or, for
-// broadened lists (BRD), {the broadeners' sum at the job's temperature, the natural width}
-template <bool BRD>
-__device__ __forceinline__ void load_widths(const RoxJobDev& J, const RoxListDev& L, int f16, long long i, float& a,
-                                            float& b) {
-  if constexpr (BRD) {
-    a = L.gLT[(long long)J.t_row * L.gLT_stride + i];
-    b = L.gN ? L.gN[i] : 0.0f;
-  } else {
-    a = load_width(L.gamma_ref, f16, i);
-    b = load_width(L.n_t, f16, i);
-  }
-}
 
 // Two FP32 values in one 64-bit register pair, for the paired FP32 instructions of sm_100 and
 // later (fma.rn.f32x2 / add.rn.f32x2: two IEEE operations, each rounded as the scalar one). A
@@ -231,19 +211,6 @@ __device__ __forceinline__ float smooth_pair(const PairTab& P, int k, float tau,
     pair_x0<NU>(c, tau, dnu_f, x0, x1);
   }
   return pair_add<false, false>(x0, x1, c, true, true, nacc);
-}
-
-// Whether a line whose window covers the span and whose slow zone misses it is smooth there: its
-// far form at the span's 32 Chebyshev points then gives it at every point of the span by
-// polynomial interpolation. D: |offset| of the span's centre from the line, h: the span's
-// half-width. The far form's poles X^2 = -A +- sqrt(-B) have real parts of at most
-// Rp = sqrt(max(0, -A) + sqrt|B|); with none within 1.25 h of the centre the error of degree 31 is
-// below 1e-7 (a Bernstein ellipse of parameter 2: 2^-32 times 128 / (1.25^2 - 1)).
-#define ROX_SMOOTH_R 1.25f
-__device__ __forceinline__ float smooth_dmin(float A, float B, float h) {
-  const float b = fabsf(B) + 1e-30f;
-  const float rp2 = fmaxf(0.0f, -A) + b * rox_rsqrt(b) + 1e-30f;
-  return fmaf(ROX_SMOOTH_R, h, rp2 * rox_rsqrt(rp2));
 }
 
 // Adds to stot (the span's points) the polynomial through the values v at the span's 32 Chebyshev
@@ -479,40 +446,6 @@ __device__ __forceinline__ void zone_line(const PairTab& P, const LineTab& L, in
   }
 }
 
-// Per-line constants of one (P,T) point that do not depend on the span: the far-form
-// constants, the slow zone's half-width hz (at least the precision margin) and threshold t_z,
-// and what pass 2 needs. nu0f: the line centre in FP32; Sp: S 2^-e; gref, nt: the width inputs
-// (see load_widths). The Voigt kernel computes them per line and span, or (ROX_VX_PRE) reads
-// them from k_line_params, which computes them once per line with this same function.
-struct LineK {
-  float A, B, P, Q, tz, iG, y, pc, zc, hz;
-};
-template <bool BRD>
-__device__ __forceinline__ LineK line_consts(float nu0f, float Sp, float gref, float nt, const RoxJobDev& J,
-                                             float margin_cm) {
-  LineK k;
-  const float gG = nu0f * J.gG_fac;
-  const float gL = BRD ? fmaf(gref, J.p_fac, nt) : gref * rox_exp2(nt * J.l2_ratio) * J.p_fac;
-  const float gG2 = gG * gG, gL2 = gL * gL;
-  const float pY = Sp * gL * ROX_INV_PI;
-  const float invG = rox_rcp(gG);
-  k.y = gL * invG;
-  const rox_far fc = rox_far_coefs(k.y);      // far-zone form of this line (rox_faddeeva.cuh)
-  // slow zone: |X| < sqrt(r2 gamma_G^2 - gamma_L^2), at least the precision margin
-  const float hz2 = fmaxf(0.0f, fc.r2 * gG2 - gL2);
-  float hz = hz2 * rox_rsqrt(hz2);            // 0 for hz2 = 0 (rsqrt(0) = inf, product taken as 0 below)
-  hz = hz2 > 0.0f ? hz : 0.0f;
-  k.zc = hz >= margin_cm ? 3e38f : hz2;
-  k.hz = fmaxf(hz, margin_cm);
-  k.A = fc.alpha * gG2;
-  k.B = fc.beta * (gG2 * gG2);
-  k.P = pY;
-  k.Q = pY * (fc.kappa * gG2);
-  k.tz = fmaf(k.hz, k.hz, k.A);
-  k.iG = invG;
-  k.pc = Sp * invG * ROX_INV_SQRT_PI;
-  return k;
-}
 
 // Sum of v[0..7] over the warp: lane l ends with the sum of v[i], i = bits 4, 3, 2 of l (as 4 2 1),
 // by a fixed tree that halves the values held at each exchange.
@@ -708,47 +641,12 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
   __syncwarp();
 }
 
-// Grid indices of a line's slow zone on a uniform grid, |j - (k0 + f)| < hz / dnu, widened by 1e-4
-// relative and one point on each side (covers every point with t < t_z despite the roundings).
-// g: the line's geometry record {k0, f dnu, jlo, jhi}.
-__device__ __forceinline__ void zone_bounds(const float4& g, float hz, float inv_dnu, int& zlo, int& zhi) {
-  const int k0 = (int)g.x;
-  const float hzg = fminf(hz * inv_dnu * 1.0001f, 8.0e6f);
-  const float fr = g.y * inv_dnu;
-  zlo = k0 + __float2int_rd(fr - hzg) - 1;
-  zhi = k0 + __float2int_ru(fr + hzg) + 1;
-}
-
-// the uniform grid's precision margin of the slow zones (cm^-1; see ROX_FAST_MARGIN)
-__device__ __forceinline__ float fast_margin(float dnu_f) { return ROX_FAST_MARGIN * 32.0f * (ROX_K - 1) * dnu_f; }
-
-// k_line_params: the per-line constants of one job ((P,T) point) for lines [J.l0, J.l1) of a
-// uniform-grid list, once per line, for the ROX_VX_PRE Voigt launch (which otherwise recomputes
-// them in every span a line reaches). One thread per line, coalesced loads and 48-byte stores.
-__global__ void k_line_params(const RoxListDev L, const RoxJobDev J, float4* rec) {
-  const float margin_cm = fast_margin(L.dnu_f);
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long i = J.l0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < J.l1; i += stride) {
-    const float4 g = L.geo[i];
-    const float Sp = J.S32[i - J.l0];
-    const float gref = load_width(L.gamma_ref, L.width_f16, i), nt = load_width(L.n_t, L.width_f16, i);
-    const float nu0f = L.nu_min_f + fmaf(g.x, L.dnu_f, g.y);
-    const LineK k = line_consts<false>(nu0f, Sp, gref, nt, J, margin_cm);
-    int zlo, zhi;
-    zone_bounds(g, k.hz, L.inv_dnu_f, zlo, zhi);
-    rec[3 * i] = make_float4(k.A, k.B, k.P, k.Q);
-    rec[3 * i + 1] = make_float4(k.tz, k.iG, k.y, k.pc);
-    rec[3 * i + 2] = make_float4(k.zc, __int_as_float(zlo), __int_as_float(zhi),
-                                 smooth_dmin(k.A, k.B, 0.5f * (ROX_SPAN - 1) * L.dnu_f));
-  }
-}
-
 // k_moments: the far forms of a cell's lines summed into one multipole expansion. With the cell's
 // centre as origin and its half-width as unit, a line at d has f(Y) = (P t + Q)/(t^2 + B),
 // t = (Y - d)^2 + A, a rational function whose expansion f = sum_l m_l / Y^(l+2) follows from
 // f (Y^4 + d3 Y^3 + d2 Y^2 + d1 Y + d0) = P Y^2 - 2 P d Y + P (d^2 + A) + Q by a four-term
-// recurrence, exact for every order. One warp takes four consecutive cells of one job, finds the
-// first by a 32-way search of the sorted centres and walks its lines 32 at a time; lanes' sums
+// recurrence, exact for every order. One warp takes four consecutive cells of one job (one where
+// there are too few to fill the GPU: 9.8 us with four against 5.2 on a list of 1e4 lines), finds the first by a 32-way search of the sorted centres and walks its lines 32 at a time; lanes' sums
 // are added by a fixed tree. Truncated after ROX_MOMENTS terms the expansion errs by
 // (r^14)(15 - 14 r) of a line's value, r = (half-width + pole modulus)/|Y|: k_voigt takes a cell only
 // where r <= 1/4 (5e-8).
@@ -763,16 +661,17 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
   if (*(volatile int32_t*)&A.hdr->status != ROX_OK) return;
   const int lane = threadIdx.x & 31;
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  for (int task = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); 4 * task < A.n_slots; task += nw) {
-    int k = 0, k_hi = A.n_jobs - 1;            // last job with mom_off <= 4 task
+  for (int task = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); A.cells_task * task < A.n_slots; task += nw) {
+    const int slot = A.cells_task * task;
+    int k = 0, k_hi = A.n_jobs - 1;            // last job with mom_off <= slot
     while (k < k_hi) {
       const int mid = (k + k_hi + 1) >> 1;
-      if (A.job[mid].mom_off <= 4 * task) k = mid; else k_hi = mid - 1;
+      if (A.job[mid].mom_off <= slot) k = mid; else k_hi = mid - 1;
     }
     const RoxJobDev& J = A.job[k];
     const RoxListDev& L = A.list[J.list];
     if (J.n_cells <= 0 || *L.status != ROX_OK) continue;
-    const int s0 = 4 * task - J.mom_off;
+    const int s0 = slot - J.mom_off;
     const long long p0 = max(L.span_lo[J.span_first], J.l0);
     const long long p1 = min(L.span_hi[J.span_first + J.n_spans - 1], J.l1);
     const float dnu_f = L.dnu_f, margin_cm = fast_margin(dnu_f);
@@ -790,7 +689,7 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
       len = min(step - 1, lo + len - nlo);
       lo = nlo;
     }
-    for (int s = s0; s < s0 + 4 && s <= J.n_cells; s++) {
+    for (int s = s0; s < s0 + A.cells_task && s <= J.n_cells; s++) {
       const int cell = J.c_first + s;
       const float centre = (float)(ROX_CELL * cell) + 0.5f * ROX_CELL, end = (float)(ROX_CELL * (cell + 1));
       if (lane == 0) A.cstart[J.mom_off + s] = (int32_t)lo;
@@ -1039,10 +938,12 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     const int n_far = (cl1 - cl0) + (cr1 - cr0);
 
     const int nbat = (nn + 31) >> 5;
-    const int p_first = part < 0 ? 0 : part, p_last = part < 0 ? ROX_PARTS - 1 : part;
+    const int np = min(ROX_PARTS, max(1, nbat >> J.part_shift));     // parts of this span
+    if (part >= np) continue;
+    const int p_first = part < 0 ? 0 : part, p_last = part < 0 ? np - 1 : part;
     for (int p = p_first; p <= p_last; p++) {
-      const int plo = 32 * ((nbat * p) / ROX_PARTS);
-      const int phi = min(nn, 32 * ((nbat * (p + 1)) / ROX_PARTS));
+      const int plo = 32 * ((nbat * p) / np);
+      const int phi = min(nn, 32 * ((nbat * (p + 1)) / np));
       // the part's total and its compensation: in shared memory (touched once in four batches),
       // Chebyshev point in nsum, ncmp
       int ekL = 0, ekR = 0;             // edge lines: first point without its final sum, per side
@@ -1274,7 +1175,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
                           side ? half + Lst.cutoff_f : half - Lst.cutoff_f, inv_cut, dnu_f, Drow, zacc);
       __syncwarp();
       // this part's share of the far cells, at this lane's Chebyshev point
-      for (int c = n_far * p / ROX_PARTS; c < n_far * (p + 1) / ROX_PARTS; c++) {
+      for (int c = n_far * p / np; c < n_far * (p + 1) / np; c++) {
         const int cell = c < cl1 - cl0 ? cl0 + c : cr0 + (c - (cl1 - cl0));
         const float4* mo = A.mom + 4 * (size_t)(J.mom_off + cell - J.c_first);
         const float4 v0 = mo[0], v1 = mo[1], v2 = mo[2], v3 = mo[3];
@@ -1311,19 +1212,19 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
       int done = 0;
       if (lane == 0) done = atomicAdd(&A.tail_cnt[item - A.n_whole], 1);
       done = __shfl_sync(0xffffffffu, done, 0);
-      if (done != ROX_PARTS - 1) continue;
+      if (done != np - 1) continue;
       __threadfence();
       const float* src = A.tail_part + (size_t)(item - A.n_whole) * ROX_PARTS * ROX_PART_FLOATS;
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
         float v = __ldcg(&src[32 * m + lane]);
-#pragma unroll
-        for (int pp = 1; pp < ROX_PARTS; pp++) v = v + __ldcg(&src[pp * ROX_PART_FLOATS + 32 * m + lane]);
+#pragma unroll 4
+        for (int pp = 1; pp < np; pp++) v = v + __ldcg(&src[pp * ROX_PART_FLOATS + 32 * m + lane]);
         stot[32 * m + lane] = v;
       }
       ntot = __ldcg(&src[ROX_SPAN + lane]);
-#pragma unroll
-      for (int pp = 1; pp < ROX_PARTS; pp++) ntot = ntot + __ldcg(&src[pp * ROX_PART_FLOATS + ROX_SPAN + lane]);
+#pragma unroll 4
+      for (int pp = 1; pp < np; pp++) ntot = ntot + __ldcg(&src[pp * ROX_PART_FLOATS + ROX_SPAN + lane]);
     }
     // ---- the smooth lines' sum at the Chebyshev points, interpolated to the span's points
     if (__any_sync(0xffffffffu, ntot != 0.f)) interp_span<NU>(ntot, lane, D, half, stot);
@@ -1399,16 +1300,6 @@ constexpr size_t voigt_dyn_smem() {
 }
 }  // namespace
 
-// per-line constants of job J (one (P,T) point) for its lines [J.l0, J.l1): rec[3 i .. 3 i + 2]
-cudaError_t rox_launch_line_params(const RoxListDev& L, const RoxJobDev& J, float4* rec, cudaStream_t s) {
-  const long long n = J.l1 - J.l0;
-  if (n <= 0) return cudaSuccess;
-  long long b = (n + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
-  k_line_params<<<(int)b, 256, 0, s>>>(L, J, rec);
-  return cudaGetLastError();
-}
-
 namespace {
 
 template <bool NU, int X, int W>
@@ -1466,7 +1357,7 @@ cudaError_t rox_launch_voigt(const RoxVoigtArgs& A, int n_blocks, bool nodes, in
 // moments of the cells of A's jobs (A.n_slots of them) ahead of the Voigt launch
 cudaError_t rox_launch_moments(const RoxVoigtArgs& A, int extras, cudaStream_t s) {
   if (A.n_slots <= 0) return cudaSuccess;
-  long long b = ((A.n_slots + 3) / 4 + 7) / 8;
+  long long b = (A.n_slots / A.cells_task + 7) / 8;      // n_slots is a multiple of 4
   if (b > 152 * 16) b = 152 * 16;
   switch (extras) {
     case 0: k_moments<0><<<(int)b, 256, 0, s>>>(A); break;
