@@ -60,12 +60,16 @@ __device__ __forceinline__ LineK line_consts(float nu0f, float Sp, float gref, f
   const float invG = rox_rcp(gG);
   k.y = gL * invG;
   const rox_far fc = rox_far_coefs(k.y);      // far-zone form of this line (rox_faddeeva.cuh)
-  // slow zone: |X| < sqrt(r2 gamma_G^2 - gamma_L^2), at least the precision margin
+  // slow zone: |X| < sqrt(r2 gamma_G^2 - gamma_L^2), at least the precision margin (see below)
   const float hz2 = fmaxf(0.0f, fc.r2 * gG2 - gL2);
   float hz = hz2 * rox_rsqrt(hz2);            // 0 for hz2 = 0 (rsqrt(0) = inf, product taken as 0 below)
   hz = hz2 > 0.0f ? hz : 0.0f;
-  k.zc = hz >= margin_cm ? 3e38f : hz2;
-  k.hz = fmaxf(hz, margin_cm);
+  // the margin keeps the offset's rounding small against |X|, or against gamma_L where that is the larger
+  // scale of the profile (its poles lie gamma_L off the axis): a broad line needs less of it, or none
+  const float mg2 = fmaxf(0.0f, fmaf(margin_cm, margin_cm, -gL2));
+  const float mg = mg2 > 0.0f ? mg2 * rox_rsqrt(mg2) : 0.0f;
+  k.zc = hz >= mg ? 3e38f : hz2;
+  k.hz = fmaxf(hz, mg);
   k.A = fc.alpha * gG2;
   k.B = fc.beta * (gG2 * gG2);
   k.P = pY;

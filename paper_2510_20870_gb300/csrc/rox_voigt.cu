@@ -249,56 +249,29 @@ __device__ __forceinline__ void interp_span(float v, int lane, const float2* D, 
 }
 
 // Pass 1 for pair k of which at least one line is cut by a window edge that the edge scan does not
-// take: the sub-spans outside both windows are skipped (warp-uniform test); elsewhere each point
-// takes line i iff it lies in the line's window, m in [ceil((jlo-Aw-lane)/32),
-// floor((jhi-Aw-lane)/32)] (the exact integer window).
+// take: the sub-spans outside both windows are skipped; elsewhere each point takes line i iff it lies
+// in the line's window (the exact integer window). Rare on long cutoffs, so the loop is kept short
+// rather than fast, and adds into the warp's row zacc.
 template <bool NU>
 __device__ __forceinline__ void edge_pair(const PairTab& P, const LineTab& L, int k, int Aw, int lane, float lanef,
-                                          float dnu_f, const float2* D, float (&acc)[ROX_K]) {
+                                          float dnu_f, const float2* D, float* zacc) {
   const PairC c = pair_consts<true>(P, k);
   const int2 w0 = L.W[2 * k], w1 = L.W[2 * k + 1];
   const int lo0 = w0.x - Aw, hi0 = w0.y - Aw, lo1 = w1.x - Aw, hi1 = w1.y - Aw;
   const int mf = max(0, min(lo0, lo1) >> 5), ml = min(ROX_K - 1, max(hi0, hi1) >> 5);
-  const int mlo0 = (lo0 - lane + 31) >> 5, mhi0 = (hi0 - lane) >> 5;   // this lane's window, in m
-  const int mlo1 = (lo1 - lane + 31) >> 5, mhi1 = (hi1 - lane) >> 5;
   float X0, X1;
   pair_x0<NU>(c, lanef, dnu_f, X0, X1);
-#pragma unroll
-  for (int m = 0; m < ROX_K; m++) {
-    if (m < mf || m > ml) continue;
-    const float x0 = pos<NU>(m, X0, c.e0, c.f0, D, dnu_f), x1 = pos<NU>(m, X1, c.e1, c.f1, D, dnu_f);
-    acc[m] = pair_add<true, true>(x0, x1, c, m >= mlo0 && m <= mhi0, m >= mlo1 && m <= mhi1, acc[m]);
-  }
-}
-
-// Pass 1 for the line in slot s alone (the last of an odd count), window-masked per sub-span
-// and point.
-template <bool NU>
-__device__ __forceinline__ void edge_line(const PairTab& P, const LineTab& L, int s, int Aw, int lane, float lanef,
-                                          float dnu_f, const float2* D, float (&acc)[ROX_K]) {
-  const int k = s >> 1, h = s & 1;
-  const float4 ab = P.ab[k], pq = P.pq[k], ef = P.ef[k];
-  const float A = row_lo(ab, h), B = row_hi(ab, h), Pc = row_lo(pq, h), Qc = row_hi(pq, h);
-  const float e = row_lo(ef, h), f = row_hi(ef, h);
-  const float tz = h ? P.tz[k].y : P.tz[k].x;
-  const int2 w = L.W[s];
-  const float X0 = NU ? 0.0f : fmaf(lanef + e, dnu_f, f);
-#pragma unroll
-  for (int m = 0; m < ROX_K; m++) {
-    const int am = Aw + 32 * m, bm = am + 31;
-    if (bm < w.x || am > w.y) continue;
-    const int j = am + lane;
-    const float x = pos<NU>(m, X0, e, f, D, dnu_f);
-    const float t = fmaxf(fmaf(x, x, A), tz);
-    const float v = fmaf(t, Pc, Qc) * rox_rcp(fmaf(t, t, B));
-    acc[m] += (j >= w.x && j <= w.y) ? v : 0.0f;
+#pragma unroll 1
+  for (int m = mf; m <= ml; m++) {
+    const int q = 32 * m + lane;
+    zacc[q] = pair_add<true, true>(pos<NU>(m, X0, c.e0, c.f0, D, dnu_f), pos<NU>(m, X1, c.e1, c.f1, D, dnu_f), c,
+                                   q >= lo0 && q <= hi0, q >= lo1 && q <= hi1, zacc[q]);
   }
 }
 
 // Pass 2 for the line in slot s, whose slow zone meets the span: at exactly the points where
 // pass 1 clamped t (t < t_z on the same rounded t, inside the window), the FP32 Faddeeva form of
-// the line's y (rox_faddeeva.cuh; FORM 0: y < 0.1, 1: y < 1, 2: above) replaces the far form's
-// boundary value cf that pass 1 added there: + S V - cf. In a zone widened to the precision margin the
+// the line's y (rox_faddeeva.cuh) replaces the far form's boundary value cf that pass 1 added there: + S V - cf. In a zone widened to the precision margin the
 // points beyond the form's own zone (X^2 >= zc) take the far form on an offset rounded once.
 // The pass is bound by instruction issue, so a lane takes two points at once in paired FP32
 // instructions (two neighbouring points of the uniform grid: 64 points a warp step, one 8-byte
@@ -306,9 +279,9 @@ __device__ __forceinline__ void edge_line(const PairTab& P, const LineTab& L, in
 // come from shared memory as ready pairs, and points outside the zone are selected away rather than
 // branched over. Within a warp step the lanes touch distinct points.
 struct ZoneC {
-  float A, B, P, Q, tz, cf, pc, zc;
+  float A, B, P, Q, tz, cf, zc;
   f32x2 gU;                    // x2 -> U
-  f32x2 ge, ge0, gc, gy, gp;   // FORM 0: exponent = ge x2 + ge0, (2xy)^2 = gc x2, pc y, pc
+  f32x2 ge, ge0, gc, gy, gp;   // Gaussian part (y < 0.1): exponent ge x2 + ge0, (2xy)^2 = gc x2, factor gp; N/D's factor gy
 };
 __device__ __forceinline__ f32x2 f2_dup(float v) { return f2_pack(v, v); }
 __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
@@ -316,20 +289,18 @@ __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// N(U)/D(U) of degrees (NP, NP + 1); cb: the 16 coefficients as pairs
-template <int NP>
+// N(U)/D(U); cb: the 16 coefficients as pairs
 __device__ __forceinline__ f32x2 rat_pair(const ulonglong2* cb, f32x2 U) {
   f32x2 c[16];
 #pragma unroll
   for (int i = 0; i < 8; i++) {
-    if (i < 4 ? 2 * i > NP : 2 * (i - 4) > NP) continue;
     const ulonglong2 v = cb[i];
     c[2 * i] = v.x;
     c[2 * i + 1] = v.y;
   }
-  f32x2 n = c[NP], d = c[8 + NP];
+  f32x2 n = c[7], d = c[15];
 #pragma unroll
-  for (int k = NP - 1; k >= 0; k--) {
+  for (int k = 6; k >= 0; k--) {
     n = f2_fma(n, U, c[k]);
     d = f2_fma(d, U, c[8 + k]);
   }
@@ -339,23 +310,17 @@ __device__ __forceinline__ f32x2 rat_pair(const ulonglong2* cb, f32x2 U) {
   return f2_mul(n, f2_pack(rox_rcp(d0), rox_rcp(d1)));
 }
 // S V - cf for the pair of offsets X
-template <int FORM>
 __device__ __forceinline__ f32x2 zone_pair(const ZoneC& z, const ulonglong2* cb, f32x2 X) {
   const f32x2 x2 = f2_mul(X, X);
-  const f32x2 r = rat_pair<FORM == 2 ? 5 : 7>(cb, f2_mul(x2, z.gU));
-  f32x2 v = f2_dup(-z.cf);
-  if constexpr (FORM == 0) {
-    float e0, e1;
-    f2_unpack(f2_fma(x2, z.ge, z.ge0), e0, e1);
-    const f32x2 u2 = f2_mul(x2, z.gc);
-    f32x2 g = f2_fma(u2, f2_dup(ROX_COS_C6), f2_dup(ROX_COS_C4));
-    g = f2_fma(u2, g, f2_dup(-0.5f));
-    g = f2_fma(u2, g, f2_dup(1.0f));
-    v = f2_fma(f2_pack(rox_exp2(e0), rox_exp2(e1)), f2_mul(g, z.gp), v);
-    v = f2_fma(r, z.gy, v);
-  } else {
-    v = f2_fma(r, z.gp, v);
-  }
+  const f32x2 r = rat_pair(cb, f2_mul(x2, z.gU));
+  float e0, e1;
+  f2_unpack(f2_fma(x2, z.ge, z.ge0), e0, e1);
+  const f32x2 u2 = f2_mul(x2, z.gc);
+  f32x2 g = f2_fma(u2, f2_dup(ROX_COS_C6), f2_dup(ROX_COS_C4));
+  g = f2_fma(u2, g, f2_dup(-0.5f));
+  g = f2_fma(u2, g, f2_dup(1.0f));
+  f32x2 v = f2_fma(f2_pack(rox_exp2(e0), rox_exp2(e1)), f2_mul(g, z.gp), f2_dup(-z.cf));
+  v = f2_fma(r, z.gy, v);
   if (z.zc < 1e38f) {
     float x0, x1, v0, v1, d0, d1, w0, w1;
     const f32x2 t = f2_add(x2, f2_dup(z.A));
@@ -367,7 +332,7 @@ __device__ __forceinline__ f32x2 zone_pair(const ZoneC& z, const ulonglong2* cb,
   }
   return v;
 }
-template <bool NU, int FORM>
+template <bool NU>
 __device__ __forceinline__ void zone_points(const ZoneC& z, const ulonglong2* cb, float e, float f, int q0, int q1,
                                             int lane, float dnu_f, const float2* D, float* zacc) {
   float t0, t1, v0, v1;
@@ -378,7 +343,7 @@ __device__ __forceinline__ void zone_points(const ZoneC& z, const ulonglong2* cb
       f2_unpack(f2_fma(X, X, f2_dup(z.A)), t0, t1);
       const bool u0 = t0 < z.tz && q >= q0 && q <= q1, u1 = t1 < z.tz && q + 32 >= q0 && q + 32 <= q1;
       if (!__any_sync(0xffffffffu, u0 || u1)) continue;
-      f2_unpack(zone_pair<FORM>(z, cb, X), v0, v1);
+      f2_unpack(zone_pair(z, cb, X), v0, v1);
       if (u0) zacc[q] += v0;
       if (u1) zacc[q + 32] += v1;
     }
@@ -393,7 +358,7 @@ __device__ __forceinline__ void zone_points(const ZoneC& z, const ulonglong2* cb
       const f32x2 Xm = f2_fma(f2_dup(mf), dn, X0);
       f2_unpack(f2_fma(Xm, Xm, f2_dup(z.A)), t0, t1);
       const f32x2 X = f2_fma(f2_add(le, f2_dup(mf)), dn, ff);  // the offset rounded once
-      f2_unpack(zone_pair<FORM>(z, cb, X), v0, v1);
+      f2_unpack(zone_pair(z, cb, X), v0, v1);
       float2* p = reinterpret_cast<float2*>(zacc + q);
       float2 s = *p;
       s.x += t0 < z.tz && q >= q0 ? v0 : 0.0f;
@@ -426,49 +391,21 @@ __device__ __forceinline__ void zone_line(const PairTab& P, const LineTab& L, in
   z.Q = row_hi(pq, h);
   z.tz = h ? P.tz[k].y : P.tz[k].x;
   z.cf = fmaf(z.tz, z.P, z.Q) * rox_rcp(fmaf(z.tz, z.tz, z.B));
-  z.pc = zl.z;
   z.zc = zl.w;
   const float g2 = zl.x * zl.x;
   z.gU = f2_dup(g2 * rox_rcp(y2 + ROX_CORE_KAPPA));
-  z.gp = f2_dup(zl.z);
-  const ulonglong2* cb = reinterpret_cast<const ulonglong2*>(cbuf);
-  const float e = row_lo(ef, h), f = row_hi(ef, h);
-  if (y < ROX_Y_CORE) {
-    z.ge = f2_dup(-ROX_LOG2E_F * g2);
-    z.ge0 = f2_dup(ROX_LOG2E_F * y2);
-    z.gc = f2_dup(4.0f * y2 * g2);
-    z.gy = f2_dup(zl.z * y);
-    zone_points<NU, 0>(z, cb, e, f, lo, hi, lane, dnu_f, D, zacc);
-  } else if (y < 1.0f) {
-    zone_points<NU, 1>(z, cb, e, f, lo, hi, lane, dnu_f, D, zacc);
-  } else {
-    zone_points<NU, 2>(z, cb, e, f, lo, hi, lane, dnu_f, D, zacc);
-  }
+  const bool small = y < ROX_Y_CORE;
+  z.ge = f2_dup(small ? -ROX_LOG2E_F * g2 : 0.0f);
+  z.ge0 = f2_dup(small ? ROX_LOG2E_F * y2 : 0.0f);
+  z.gc = f2_dup(small ? 4.0f * y2 * g2 : 0.0f);
+  z.gp = f2_dup(small ? zl.z : 0.0f);
+  z.gy = f2_dup(small ? zl.z * y : zl.z);
+  zone_points<NU>(z, reinterpret_cast<const ulonglong2*>(cbuf), row_lo(ef, h), row_hi(ef, h), lo, hi, lane, dnu_f, D,
+                  zacc);
 }
 
 
-// Sum of v[0..7] over the warp: lane l ends with the sum of v[i], i = bits 4, 3, 2 of l (as 4 2 1),
-// by a fixed tree that halves the values held at each exchange.
-__device__ __forceinline__ float warp_sum8(const float (&v)[8], int lane) {
-  float a[4], b[2], c;
-  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const float keep = h16 ? v[4 + i] : v[i], give = h16 ? v[i] : v[4 + i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; i++) {
-    const float keep = h8 ? a[2 + i] : a[i], give = h8 ? a[i] : a[2 + i];
-    b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-  }
-  const float keep = h4 ? b[1] : b[0], give = h4 ? b[0] : b[1];
-  c = keep + __shfl_xor_sync(0xffffffffu, give, 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  return c + __shfl_xor_sync(0xffffffffu, c, 1);
-}
-
-#define ROX_ZONE_DENSE 8   // points of the common zone per zoned line up to which the batch form is taken
+#define ROX_ZONE_DENSE 16   // points of the common zone per zoned line up to which the batch form is taken
 // Pass 2 for all zoned lines of a batch at once, one line a lane: where the lines lie close together
 // their zones share most of their points, and the warp walks those points [qa, qb] with every
 // lane evaluating its own line (coefficients in registers, computed once for the batch) and a
@@ -478,7 +415,7 @@ __device__ __forceinline__ float warp_sum8(const float (&v)[8], int lane) {
 // lane's line is zoned; [q0, q1]: its zone inside its window (span positions).
 template <bool NU>
 __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int qb, bool cut, const LineK& k, float e,
-                                           float f, float dnu_f, const float2* Drow, int lane, float* zacc) {
+                                           float f, float dnu_f, const float2* Drow, int lane, float* sm, float* zacc) {
   const bool small = k.y < ROX_Y_CORE;
   const float y2 = k.y * k.y;
   float c[16];
@@ -504,9 +441,13 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
   const float zt = on ? k.tz - k.A : -1.0f;                 // the zone: X^2 < t_z - A
   const bool wide = __any_sync(0xffffffffu, on && k.zc < 1e38f);
   const f32x2 ee = f2_dup(e), ff = f2_dup(f), dn = f2_dup(dnu_f), one = f2_dup(1.0f);
+  // sum over the lanes, eight points at a time through shared memory: row i holds point q + i of every
+  // line; lane l then adds eight lines of row l / 4, conflict-free with rows 36 floats apart
+  const float* row = sm + 36 * (lane >> 2) + 8 * (lane & 3);
   for (int q = qa & ~7; q <= qb; q += 8) {
-    float v[8];
-#pragma unroll
+    // one pair of points a round, not unrolled: the kernel's code is larger than the instruction
+    // caches, and a loop body that fits the first of them is fetched once
+#pragma unroll 1
     for (int i = 0; i < 8; i += 2) {
       f32x2 X;
       if constexpr (NU) {
@@ -523,7 +464,7 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
         n = f2_fma(n, U, f2_dup(c[j]));
         d = f2_fma(d, U, f2_dup(c[8 + j]));
       }
-      float d0, d1, e0, e1, x0, x1;
+      float d0, d1, e0, e1, x0, x1, v0, v1;
       f2_unpack(f2_fma(d, U, one), d0, d1);
       f2_unpack(f2_fma(x2, ge, ge0), e0, e1);
       const f32x2 u2 = f2_mul(x2, gc);
@@ -532,27 +473,33 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
       g = f2_fma(u2, g, one);
       f32x2 s = f2_fma(f2_pack(rox_exp2(e0), rox_exp2(e1)), f2_mul(g, gp), ncf);
       s = f2_fma(f2_mul(n, f2_pack(rox_rcp(d0), rox_rcp(d1))), gy, s);
-      f2_unpack(s, v[i], v[i + 1]);
+      f2_unpack(s, v0, v1);
       f2_unpack(x2, x0, x1);
       if (wide) {
-        float w0, w1, n0, n1;
+        float w0, w1, n0, n1, c0, c1;
         const f32x2 t = f2_add(x2, f2_dup(k.A));
         f2_unpack(f2_fma(t, f2_dup(k.P), f2_dup(k.Q)), n0, n1);
         f2_unpack(f2_fma(t, t, f2_dup(k.B)), w0, w1);
-        float c0, c1;
         f2_unpack(ncf, c0, c1);
-        v[i] = x0 < k.zc ? v[i] : fmaf(n0, rox_rcp(w0), c0);
-        v[i + 1] = x1 < k.zc ? v[i + 1] : fmaf(n1, rox_rcp(w1), c1);
+        v0 = x0 < k.zc ? v0 : fmaf(n0, rox_rcp(w0), c0);
+        v1 = x1 < k.zc ? v1 : fmaf(n1, rox_rcp(w1), c1);
       }
-      v[i] = x0 < zt ? v[i] : 0.0f;
-      v[i + 1] = x1 < zt ? v[i + 1] : 0.0f;
+      v0 = x0 < zt ? v0 : 0.0f;
+      v1 = x1 < zt ? v1 : 0.0f;
       if (cut) {
-        v[i] = q + i >= q0 && q + i <= q1 ? v[i] : 0.0f;
-        v[i + 1] = q + i + 1 >= q0 && q + i + 1 <= q1 ? v[i + 1] : 0.0f;
+        v0 = q + i >= q0 && q + i <= q1 ? v0 : 0.0f;
+        v1 = q + i + 1 >= q0 && q + i + 1 <= q1 ? v1 : 0.0f;
       }
+      sm[36 * i + lane] = v0;
+      sm[36 * i + 36 + lane] = v1;
     }
-    const float r = warp_sum8(v, lane);
+    __syncwarp();
+    const float4 a = *reinterpret_cast<const float4*>(row), b = *reinterpret_cast<const float4*>(row + 4);
+    float r = ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
     if ((lane & 3) == 0) zacc[q + (lane >> 2)] += r;
+    __syncwarp();
   }
 }
 
@@ -617,7 +564,7 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
     }
     rec[0].key = -1;
   }
-#pragma unroll
+#pragma unroll 1
   for (int o = 1; o < 32; o <<= 1) {
     const int ko = __shfl_up_sync(0xffffffffu, kk, o);
     kk = lane >= o ? max(kk, ko) : kk;
@@ -881,13 +828,16 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     // whose lines cover the span, far enough for the expansion and for the lines' slow zones. Their
     // lines [xa, xb) and [xc, xd) leave the span's list, whose other lines are visited one by one.
     int cl0 = 0, cl1 = 0, cr0 = 0, cr1 = 0;
+    bool runL = false, runR = false;   // the lines beyond the cells on that side run through the edge scan
     int xa = lo, xb = lo, xc = hi, xd = hi;
     if (!NU && J.n_cells > 0 && hi > lo) {
       const int c_end = J.c_first + J.n_cells;
       cl0 = max((Bw - Lst.c_steps + ROX_CELL - 1) >> ROX_CELL_LOG2, J.c_first);
       cr1 = min((Aw + Lst.c_steps) >> ROX_CELL_LOG2, c_end);
       float pm = 0.f, zm = 0.f;
-      for (int c = cl0 + lane; c < cr1; c += 32) {
+      // over every cell that can hold a line of the span, edge cells included
+      const int ca = max(cl0 - (ROX_CELLS_PER_SPAN + 2), J.c_first), cb = min(cr1 + ROX_CELLS_PER_SPAN + 2, c_end);
+      for (int c = ca + lane; c < cb; c += 32) {
         const float4 v = A.mom[4 * (size_t)(J.mom_off + c - J.c_first) + 3];
         pm = fmaxf(pm, v.z);
         zm = fmaxf(zm, v.w);
@@ -915,6 +865,12 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
       } else {
         cr1 = cr0;
       }
+      // all of them no farther from their expansion centre than edge_batch allows, none with its zone
+      // in the span
+      const float dist = half + (ROX_CELL + 2) * dnu_f;
+      const bool fits = dist + pm <= ROX_EDGE_R * (Lst.cutoff_f - half) && zm + dist + half < Lst.cutoff_f;
+      runL = fits && cl1 > cl0 && cl0 - (ROX_CELLS_PER_SPAN + 2) >= J.c_first;
+      runR = fits && cr1 > cr0 && cr1 + (ROX_CELLS_PER_SPAN + 2) <= c_end;
       if (part <= 0 && lane == 0) evals += (unsigned long long)((long long)(xb - xa) + (xd - xc)) * (unsigned)(whi - wlo + 1);
     }
     // without cells on the left the list is cut at the span's centre, so that the lines left of it
@@ -958,14 +914,63 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         zacc[32 * m + lane] = 0.f;
       }
 
+      // the runs of edge lines beyond the cells: moments only, two 16-byte records a line, loaded one
+      // batch ahead (per line about 7 warp instructions, where the general batch takes 20)
+      if constexpr (!NU) {
+        __syncwarp();
+#pragma unroll 1
+        for (int side = 0; side < 2; side++) {
+          const bool left = side == 0;
+          const int ea = left ? plo : max(plo, n2), eb = left ? min(phi, n1) : phi;
+          if (!(left ? runL : runR) || ea >= eb) continue;
+          if (left) edgeL = true; else edgeR = true;
+          const float centre = left ? half - Lst.cutoff_f : half + Lst.cutoff_f;
+          int kcur = 0;
+          float4 g_n = make_float4(0.f, 0.f, 0.f, 0.f);
+          LineK k_n = {1.f, 1.f, 0.f, 0.f, 1.f, 1.f, 0.f, 0.f, 3e38f, 0.f};
+          auto fetch = [&](int q) {
+            if (q >= eb) return;
+            const int li = IDX ? Lst.idx[line_at(q)] : line_at(q);
+            g_n = Lst.geo[li];
+            if constexpr (PRE) {
+              const float4 r0 = Lst.rec[3 * (long long)li];
+              k_n.A = r0.x;
+              k_n.B = r0.y;
+              k_n.P = r0.z;
+              k_n.Q = r0.w;
+            } else {
+              float ga, gb;
+              load_widths<BRD>(J, Lst, f16, li, ga, gb);
+              k_n = line_consts<BRD>(Lst.nu_min_f + fmaf(g_n.x, dnu_f, g_n.y), S_row[li], ga, gb, J, margin_cm);
+            }
+          };
+          fetch(ea + lane);
+          for (int b0 = ea; b0 < eb; b0 += 32) {
+            const bool mine = b0 + lane < eb;
+            const float4 g = g_n;
+            const LineK k = k_n;
+            fetch(b0 + 32 + lane);
+            const int jlo = __float_as_int(g.z), jhi = __float_as_int(g.w);
+            const int ov = min(jhi, whi) - max(jlo, wlo) + 1;
+            if (mine && ov > 0) evals += (unsigned)ov;
+            const int key = left ? (jhi < Bg ? Bw - jhi : 0) : max(jlo - Aw, 0);
+            const float v = -fmaf((float)Aw - g.x, dnu_f, -g.y);
+            edge_batch<NU>(BT.scan, carry + 12 * side, left, mine, key, (v - centre) * inv_cut, k, kcur, lane, centre, inv_cut,
+                           dnu_f, Drow, zacc);
+          }
+          if (left) ekL = kcur; else ekR = kcur;
+        }
+      }
+      const int mlo = runL ? max(plo, n1) : plo, mhi = runR ? min(phi, n2) : phi;   // the rest, in general batches
+
       // stage a batch's lines, one a lane: batch 0 here, each next one as soon as the lanes have
       // turned the current one into constants; widths go through registers (with an index, the
       // positions' line numbers one batch further ahead)
       float gref = 0.f, nt = 0.f;
       int li_n = 0;   // IDX: line number of this lane's position in the next batch
-      if (IDX && plo + lane < phi) li_n = Lst.idx[line_at(plo + lane)];
+      if (IDX && mlo + lane < mhi) li_n = Lst.idx[line_at(mlo + lane)];
       auto stage = [&](int q) {
-        if (q < phi) {
+        if (q < mhi) {
           const int li = IDX ? li_n : line_at(q);
           cp_async16(&geo_st[lane], &Lst.geo[li]);
           if constexpr (PRE) {
@@ -976,13 +981,13 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
             load_widths<BRD>(J, Lst, f16, li, gref, nt);
           }
         }
-        if (IDX && q + 32 < phi) li_n = Lst.idx[line_at(q + 32)];
+        if (IDX && q + 32 < mhi) li_n = Lst.idx[line_at(q + 32)];
         cp_async_commit();
       };
-      stage(plo + lane);
+      stage(mlo + lane);
       int nb = 0;
-      for (int b0 = plo; b0 < phi; b0 += 32, nb++) {
-        const int cnt = min(32, phi - b0);
+      for (int b0 = mlo; b0 < mhi; b0 += 32, nb++) {
+        const int cnt = min(32, mhi - b0);
         cp_async_wait0();   // this lane's copies of the current batch have landed
 
         // ---- per-line constants (lane <-> line b0 + lane), written to the line's slot
@@ -1077,9 +1082,9 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         if (nz > 0) {
           const int qa = __reduce_min_sync(0xffffffffu, on ? q0 : ROX_SPAN), qb = __reduce_max_sync(0xffffffffu, on ? q1 : -1);
           batched = qb - qa + 1 <= ROX_ZONE_DENSE * nz;
-          if (batched)
+          if (batched)       // (the tables of the batch before are no longer read: the loop ends in a __syncwarp)
             zone_batch<NU>(on, q0, q1, qa, qb, __any_sync(0xffffffffu, on && (jlo > zlo || jhi < zhi)), kk, ax, ay, dnu_f,
-                           Drow, lane, zacc);
+                           Drow, lane, reinterpret_cast<float*>(s_tab[w]), zacc);
         }
         // ---- window edges in order, where the lines are smooth on the span
         bool scanned = false;
@@ -1103,16 +1108,15 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
           }
         }
         const unsigned msm = __ballot_sync(0xffffffffu, live && smooth);
-        const unsigned clean = __ballot_sync(0xffffffffu, live && covers && !zoned && !smooth);
-        const unsigned czone = __ballot_sync(0xffffffffu, live && covers && zoned);
+        const unsigned cov = __ballot_sync(0xffffffffu, live && covers && !smooth);
         const unsigned edge = __ballot_sync(0xffffffffu, live && !covers && !scanned);
-        const int nsm = __popc(msm), nclean = nsm + __popc(clean), ncov = nclean + __popc(czone);
-        const int nslot = ncov + __popc(edge);
+        const int nsm = __popc(msm), ncov = nsm + __popc(cov), nslot = ncov + __popc(edge);
         const unsigned below = (1u << lane) - 1u;
         const int slot = !covers ? ncov + __popc(edge & below)
-                         : zoned ? nclean + __popc(czone & below)
-                         : smooth ? __popc(msm & below) : nsm + __popc(clean & below);
+                         : smooth ? __popc(msm & below) : nsm + __popc(cov & below);
         const unsigned zslots = __reduce_or_sync(0xffffffffu, (on && !batched) ? (1u << slot) : 0u);
+        // the line table serves the masked pairs (an odd covering line among them) and pass 2 line by line
+        const bool lines_used = (edge != 0) | ((ncov & 1) != 0) | (zslots != 0);
         if (live && !scanned) {
           const int k = slot >> 1, h = slot & 1;
           float* ab = reinterpret_cast<float*>(&PT.ab[k]);
@@ -1125,32 +1129,40 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
           ef[h] = ax;
           ef[2 + h] = ay;
           reinterpret_cast<float*>(&PT.tz[k])[h] = tz;
-          LT.W[slot] = make_int2(jlo, jhi);
-          LT.Z[slot] = make_int2(zlo, zhi);
-          LT.z[slot] = zl;
+          if (lines_used) {
+            LT.W[slot] = make_int2(jlo, jhi);
+            LT.Z[slot] = make_int2(zlo, zhi);
+            LT.z[slot] = zl;
+          }
+        }
+        if ((nslot & 1) && lane == 0) {    // an empty line completes the last pair
+          const int k = nslot >> 1;
+          float *ab = reinterpret_cast<float*>(&PT.ab[k]), *pq = reinterpret_cast<float*>(&PT.pq[k]);
+          float* ef = reinterpret_cast<float*>(&PT.ef[k]);
+          ab[1] = ab[3] = 1.f;
+          pq[1] = pq[3] = ef[1] = ef[3] = 0.f;
+          PT.tz[k].y = 1.f;
+          LT.W[nslot] = make_int2(1 << 29, -(1 << 29));
         }
         stage(b0 + 32 + lane);
         __syncwarp();
 
-        // ---- pass 1: far formula at every point of every line's window. Clean pairs as they
-        // are; pairs with a zoned line with t clamped to the zone boundary; then the rest (an odd
-        // covering line, the window-edge lines) in pairs with window masks. Fixed orders: the sum
-        // is reproducible.
-        const int ks = nsm >> 1, kc = nclean >> 1, kz = ncov >> 1;
+        // ---- pass 1: smooth pairs at the Chebyshev points; covering pairs at every point of the span,
+        // t clamped to the zone boundary (which a line without a slow zone there never meets: one
+        // code for both, as the instruction caches are the scarcer resource); the rest (an odd
+        // covering line, window-edge lines) in pairs with window masks. Fixed orders: the sum is
+        // reproducible.
+        const int ks = nsm >> 1, kz = ncov >> 1, ke = (nslot + 1) >> 1;
         for (int k = 0; k < ks; k++) nacc = smooth_pair<NU>(PT, k, tau, dnu_f, nacc);
-        for (int k = ks; k < kc; k++) cover_pair<NU, false>(PT, k, lanef, dnu_f, D, acc);
-        for (int k = kc; k < kz; k++) cover_pair<NU, true>(PT, k, lanef, dnu_f, D, acc);
-        for (int s2 = 2 * kz; s2 < nslot; s2 += 2) {
-          if (s2 + 1 < nslot) edge_pair<NU>(PT, LT, s2 >> 1, Aw, lane, lanef, dnu_f, D, acc);
-          else edge_line<NU>(PT, LT, s2, Aw, lane, lanef, dnu_f, D, acc);
-        }
+        for (int k = ks; k < kz; k++) cover_pair<NU, true>(PT, k, lanef, dnu_f, D, acc);
+        for (int k = kz; k < ke; k++) edge_pair<NU>(PT, LT, k, Aw, lane, lanef, dnu_f, D, zacc);
         // ---- pass 2 line by line otherwise
         for (unsigned z = zslots; z; z &= z - 1)
           zone_line<NU>(PT, LT, __ffs(z) - 1, Aw, lane, dnu_f, core_r, D, cbuf, zacc);
         __syncwarp();
         // the partial sums into the part's total every 4 batches: compensated (Kahan) with
         // ROX_KAHAN, else plainly (kw = 0: the correction term stays 0)
-        if ((nb & 3) == 3 || b0 + 32 >= phi) {
+        if ((nb & 3) == 3 || b0 + 32 >= mhi) {
 #pragma unroll
           for (int m = 0; m < ROX_K; m++) {
             const float t0 = part_tot[32 * m], yk = acc[m] - part_cmp[32 * m];
