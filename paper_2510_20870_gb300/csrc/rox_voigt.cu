@@ -57,11 +57,11 @@ struct LineTab {
                    // line's own zone where the precision margin widens it, else huge}
 };
 // The warp's tables of a batch; before they are written the same memory holds the edge lines' scan.
-#define ROX_EDGE_TERMS 10
-struct EdgeRec {
+#define ROX_EDGE_TERMS 8
+struct __align__(16) EdgeRec {
   float m[ROX_EDGE_TERMS];   // moments of the edge lines up to this one
   int key;                   // first point (counted from the side the lines come from) that has them
-  int pad;
+  int pad[3];
 };
 struct BatchTab {
   union {
@@ -445,9 +445,9 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
   // line; lane l then adds eight lines of row l / 4, conflict-free with rows 36 floats apart
   const float* row = sm + 36 * (lane >> 2) + 8 * (lane & 3);
   for (int q = qa & ~7; q <= qb; q += 8) {
-    // one pair of points a round, not unrolled: the kernel's code is larger than the instruction
-    // caches, and a loop body that fits the first of them is fetched once
-#pragma unroll 1
+    // two pairs of points a round, not all four: the kernel's code is larger than the instruction
+    // caches (fully unrolled, warps spent 46% of their stalls waiting for instructions)
+#pragma unroll 2
     for (int i = 0; i < 8; i += 2) {
       f32x2 X;
       if constexpr (NU) {
@@ -512,8 +512,8 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
 // under a mask took 95. The left lines (edge jhi) run through the list downwards, so that both sides
 // count points from the side the lines come from: key = Bw - jhi or jlo - Aw, non-decreasing.
 // Centre distances are one cutoff give or take the span's half-width; with (half-width + pole
-// modulus) / (cutoff - half-width) at most ROX_EDGE_R, ten terms err by 11 r^10 < 1e-7.
-#define ROX_EDGE_R 0.15f
+// modulus) / (cutoff - half-width) at most ROX_EDGE_R, eight terms err by 9 r^8 = 1e-7.
+#define ROX_EDGE_R 0.1f
 // points [k0, k1) of one side: their line's sum from the records rec[0 .. n_rec - 1] (n_rec 33, or 1 to take rec[0])
 template <bool NU>
 __device__ __forceinline__ void edge_points(const EdgeRec* rec, int n_rec, bool left, int k0, int k1, int lane,
@@ -526,13 +526,13 @@ __device__ __forceinline__ void edge_points(const EdgeRec* rec, int n_rec, bool 
         if (rec[i + st].key <= k) i += st;
       if (i == 31 && rec[32].key <= k) i = 32;
     }
-    const EdgeRec& r = rec[i];
+    const float4 ra = reinterpret_cast<const float4*>(rec[i].m)[0], rb = reinterpret_cast<const float4*>(rec[i].m)[1];
     const int q = left ? ROX_SPAN - 1 - k : k;
     const float y = ((NU ? Drow[q].x : (float)q * dnu_f) - centre) * inv_cut;
     const float z = rox_rcp(y);
-    float f = r.m[ROX_EDGE_TERMS - 1];
-#pragma unroll
-    for (int l = ROX_EDGE_TERMS - 2; l >= 0; l--) f = fmaf(f, z, r.m[l]);
+    float f = fmaf(rb.w, z, rb.z);
+    f = fmaf(fmaf(fmaf(f, z, rb.y), z, rb.x), z, ra.w);
+    f = fmaf(fmaf(fmaf(f, z, ra.z), z, ra.y), z, ra.x);
     zacc[q] += z * z * f;
   }
 }
@@ -555,16 +555,22 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
   for (int l = 4; l < ROX_EDGE_TERMS; l++) m[l] = fmaf(d3, m[l - 1], fmaf(d2, m[l - 2], fmaf(d1, m[l - 3], d0 * m[l - 4])));
   int kk = mine ? key : -1;
   __syncwarp();                      // the tables of the batch before are no longer read
-  if (lane == 0) {
-#pragma unroll
-    for (int l = 0; l < ROX_EDGE_TERMS; l++) {
-      const float c = carry[l];
-      rec[0].m[l] = c;
-      m[l] += c;
+  {
+    const float4 ca = reinterpret_cast<const float4*>(carry)[0], cb = reinterpret_cast<const float4*>(carry)[1];
+    if (lane == 0) {
+      reinterpret_cast<float4*>(rec[0].m)[0] = ca;
+      reinterpret_cast<float4*>(rec[0].m)[1] = cb;
+      m[0] += ca.x;
+      m[1] += ca.y;
+      m[2] += ca.z;
+      m[3] += ca.w;
+      m[4] += cb.x;
+      m[5] += cb.y;
+      m[6] += cb.z;
+      m[7] += cb.w;
     }
-    rec[0].key = -1;
   }
-#pragma unroll 1
+#pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int ko = __shfl_up_sync(0xffffffffu, kk, o);
     kk = lane >= o ? max(kk, ko) : kk;
@@ -574,12 +580,14 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
       if (lane >= o) m[l] += t;
     }
   }
-#pragma unroll
-  for (int l = 0; l < ROX_EDGE_TERMS; l++) rec[lane + 1].m[l] = m[l];
+  const float4 ma = make_float4(m[0], m[1], m[2], m[3]), mb = make_float4(m[4], m[5], m[6], m[7]);
+  float4* r = reinterpret_cast<float4*>(rec[lane + 1].m);
+  r[0] = ma;
+  r[1] = mb;
   rec[lane + 1].key = kk;
   if (lane == 31) {
-#pragma unroll
-    for (int l = 0; l < ROX_EDGE_TERMS; l++) carry[l] = m[l];
+    reinterpret_cast<float4*>(carry)[0] = ma;
+    reinterpret_cast<float4*>(carry)[1] = mb;
   }
   __syncwarp();
   const int klast = min(__shfl_sync(0xffffffffu, kk, 31), ROX_SPAN);
