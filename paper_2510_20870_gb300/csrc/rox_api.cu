@@ -375,7 +375,25 @@ long long job_cells(RoxJobDev* J, int32_t c_steps) {
   const long long ext = std::min<long long>((c_steps + 4) / ROX_CELL + 1, ROX_CELL_EXT);
   J->c_first = J->span_first * ROX_CELLS_PER_SPAN - (int32_t)ext;
   J->n_cells = J->n_spans * ROX_CELLS_PER_SPAN + 2 * (int32_t)ext;
+  if (J->l1 - J->l0 < J->n_cells) {   // sparse: under a line a cell, no span would take them
+    J->n_cells = 0;
+    return 0;
+  }
   return ((long long)J->n_cells + 1 + 3) & ~3LL;
+}
+
+// Parts of a job's spans (see ROX_PARTS): from the job's lines and spans alone, so that its result does
+// not depend on what it is launched with.
+void set_parts(RoxJobDev* J, int32_t c_steps) {
+  J->part_shift = rox_part_shift(J->n_spans);
+  J->max_parts = ROX_PARTS;
+  if (c_steps <= 0) return;      // nodes: a span's share of the lines is not known beforehand
+  // lines that an average span visits one by one: those within about 700 points where cells take the
+  // rest, else all within the cutoff
+  const double pts = (double)J->n_spans * ROX_SPAN + 2.0 * c_steps, reach = 2.0 * c_steps + ROX_SPAN;
+  const double lines = (double)(J->l1 - J->l0) * (c_steps >= 2 * ROX_SPAN && reach > 1400.0 ? 1400.0 : reach) / pts;
+  const double parts = std::ceil(2.0 * lines / 32.0) / (1 << J->part_shift);
+  J->max_parts = parts >= ROX_PARTS ? ROX_PARTS : (parts < 1.0 ? 1 : (int32_t)parts);
 }
 
 // Voigt launches over the jobs, at most ROX_MAX_JOBS per launch; the work counter is reset
@@ -405,6 +423,8 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
       items += J.n_spans;
       A.item_end[nj] = items;
     }
+    A.split_parts = 1;
+    for (int k = 0; k < nj; k++) A.split_parts = std::max(A.split_parts, A.job[k].max_parts);
     A.n_slots = (int32_t)slots;
     A.cells_task = slots < 152 * 64 ? 1 : 4;
     // whole items in complete rounds of the launch's warps, then at least one round of items in
@@ -416,7 +436,7 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
     A.n_jobs = nj;
     A.n_items = items;
     A.n_whole = items - (int)split;
-    A.n_queue = A.n_whole + (int)split * ROX_PARTS;
+    A.n_queue = A.n_whole + (int)split * A.split_parts;
     const long long need = ((long long)A.n_queue + cfg.warps_per_cta - 1) / cfg.warps_per_cta;
     const int blocks = need < nblocks ? (int)need : nblocks;
     int rc;
@@ -666,7 +686,7 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
     J.list = 0;
     J.span_first = 0;
     J.n_spans = (int32_t)nt;
-    J.part_shift = nt >= ROX_MANY_SPANS ? ROX_PART_SHIFT : 0;
+    set_parts(&J, L0.c_steps);
     J.p_fac = (float)(P_bar[k] / ROX_P_REF);
     J.gG_fac = (float)(sqrt(2.0 * ROX_KB * T[k] / (mass_amu * ROX_AMU)) / ROX_C_M);
     J.l2_ratio = (float)log2(ROX_T_REF / T[k]);
@@ -1076,12 +1096,12 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     d.list = j.list;
     d.span_first = (int32_t)(j.first / ROX_SPAN);
     d.n_spans = (int32_t)((j.first + j.n - 1) / ROX_SPAN - j.first / ROX_SPAN + 1);
-    d.part_shift = d.n_spans >= ROX_MANY_SPANS ? ROX_PART_SHIFT : 0;
     d.p_fac = (float)(j.P_bar / ROX_P_REF);
     d.gG_fac = (float)(sqrt(2.0 * ROX_KB * j.T / (j.mass_amu * ROX_AMU)) / ROX_C_M);
     d.l2_ratio = (float)log2(ROX_T_REF / j.T);
     d.flags = j.flags;
     d.t_row = 0;
+    set_parts(&d, L[j.list].c_steps);
   }
   if ((rc = launch_voigt_jobs(L, n_lists, J.data(), n_jobs, hdr, tail.part, tail.cnt, tail.cap, tail.mom, nblocks, s,
                               cfg)))

@@ -88,6 +88,8 @@ struct RoxListDev {
 #define ROX_CELL_LOG2 6
 #define ROX_CELL (1 << ROX_CELL_LOG2)
 #define ROX_MOMENTS 14
+#define ROX_CELL_LINES 2           // lines a cell on average from which a span takes its cells: reading a cell
+                                   // takes 25 instructions, a line that is smooth on the span about 20
 #define ROX_CELL_EXT 512           // cells kept on each side of a job's spans (further lines: one by one)
 #define ROX_MOM_JOBS 16            // jobs whose cells the workspace of a cross-section call holds at a time
 #define ROX_CELL_BYTES 68          // 16 floats and the cell's first line (int32)
@@ -131,15 +133,17 @@ struct RoxJobDev {
   int32_t t_row;    // broadened lists: the job's temperature row of the list's gLT
   int32_t mom_off;  // the job's first slot in RoxVoigtArgs::mom and cstart (a multiple of 4)
   int32_t c_first;  // the cell of that slot
-  int32_t part_shift;  // a span's parts: its batches of lines >> part_shift, 1 .. ROX_PARTS
+  int32_t part_shift;  // a span's parts: its batches of lines >> part_shift, 1 .. max_parts
+  int32_t max_parts;   // 1 .. ROX_PARTS
   int32_t n_cells;  // cells with moments (slot n_cells holds only the first line beyond them); 0: none
 };
 
 // Every span's lines are summed as up to ROX_PARTS consecutive parts (batch-aligned), each from
 // zero, and the part sums are added in part order. How many is fixed by the job and the span: a job of
-// many spans fills the GPU with whole items and takes a part per 2^part_shift batches (a part's
-// fixed work, some 400 instructions and the wait for its first batch, is not worth less), a short one a
-// part per batch. A work item is normally a whole span; the
+// many spans (three rounds of the GPU's warps or more) fills it with whole items and takes a part per 16
+// batches (a part's fixed work, some 400 instructions and the wait for its first batch, is not worth
+// less), a shorter one a part per 4 or per batch, at most about twice what its spans have on average (a
+// split item has a queue entry per possible part). A work item is normally a whole span; the
 // last items of a launch are split into their parts, taken by different warps: each part stores
 // its sum in the tail scratch and the last of them to finish adds the parts in the same order.
 // The result is the same either way, so it depends neither on the split nor on the launch grid.
@@ -147,8 +151,7 @@ struct RoxJobDev {
 // the launch's warps and the split ones end the launch in pieces of 1/ROX_PARTS of an item
 // (at most ROX_TAIL_ITEMS_MAX items, the size of the workspace's tail scratch).
 #define ROX_PARTS 16
-#define ROX_MANY_SPANS 2048
-#define ROX_PART_SHIFT 4
+static inline int32_t rox_part_shift(long long n_spans) { return n_spans >= 8192 ? 4 : (n_spans >= 2048 ? 2 : 0); }
 #define ROX_TAIL_ITEMS_MAX 8192
 // A part's sum: its ROX_SPAN points, then its values at the span's ROX_NODES Chebyshev points
 // (the lines that are smooth on the span, rox_voigt.cu)
@@ -166,7 +169,8 @@ struct RoxVoigtArgs {
   int32_t n_slots;                  // slots over all jobs (0: no moments in this launch)
   int32_t n_items;                  // items (spans over all jobs); the last n_items - n_whole split
   int32_t n_whole;
-  int32_t n_queue;                  // queue entries: n_whole + (n_items - n_whole) * ROX_PARTS
+  int32_t split_parts;              // queue entries of a split item: the jobs' largest max_parts
+  int32_t n_queue;                  // queue entries: n_whole + (n_items - n_whole) * split_parts
   int32_t item_end[ROX_MAX_JOBS];   // item_end[k] = spans of jobs 0..k
   RoxListDev list[ROX_MAX_LISTS];
   RoxJobDev job[ROX_MAX_JOBS];

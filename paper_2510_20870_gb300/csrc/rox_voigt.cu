@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     int q = 0, k = 0;
     if (lane == 0) {
       q = atomicAdd(&A.hdr->work_counter, 1);
-      const int it = q < A.n_whole ? q : A.n_whole + (q - A.n_whole) / ROX_PARTS;
+      const int it = q < A.n_whole ? q : A.n_whole + (q - A.n_whole) / A.split_parts;
       int lo_k = 0, hi_k = A.n_jobs - 1;           // first job with item_end > it
       while (lo_k < hi_k) {
         const int mid = (lo_k + hi_k) >> 1;
@@ -794,8 +794,8 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     k = __shfl_sync(0xffffffffu, k, 0);
     if (q >= A.n_queue) break;
     // queue entry -> item and part (-1: the whole span, all parts in order)
-    const int item = q < A.n_whole ? q : A.n_whole + (q - A.n_whole) / ROX_PARTS;
-    const int part = q < A.n_whole ? -1 : (q - A.n_whole) % ROX_PARTS;
+    const int item = q < A.n_whole ? q : A.n_whole + (q - A.n_whole) / A.split_parts;
+    const int part = q < A.n_whole ? -1 : (q - A.n_whole) % A.split_parts;
     const RoxJobDev& J = A.job[k];
     const RoxListDev& Lst = A.list[J.list];
     const int local = item - (k > 0 ? A.item_end[k - 1] : 0);
@@ -838,7 +838,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     int cl0 = 0, cl1 = 0, cr0 = 0, cr1 = 0;
     bool runL = false, runR = false;   // the lines beyond the cells on that side run through the edge scan
     int xa = lo, xb = lo, xc = hi, xd = hi;
-    if (!NU && J.n_cells > 0 && hi > lo) {
+    if (!NU && J.n_cells > 0 && hi - lo >= ROX_CELL_LINES * ((2 * Lst.c_steps + ROX_SPAN) >> ROX_CELL_LOG2)) {
       const int c_end = J.c_first + J.n_cells;
       cl0 = max((Bw - Lst.c_steps + ROX_CELL - 1) >> ROX_CELL_LOG2, J.c_first);
       cr1 = min((Aw + Lst.c_steps) >> ROX_CELL_LOG2, c_end);
@@ -902,7 +902,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     const int n_far = (cl1 - cl0) + (cr1 - cr0);
 
     const int nbat = (nn + 31) >> 5;
-    const int np = min(ROX_PARTS, max(1, nbat >> J.part_shift));     // parts of this span
+    const int np = min(J.max_parts, max(1, nbat >> J.part_shift));     // parts of this span
     if (part >= np) continue;
     const int p_first = part < 0 ? 0 : part, p_last = part < 0 ? np - 1 : part;
     for (int p = p_first; p <= p_last; p++) {
