@@ -166,7 +166,8 @@ struct WsLayout {
   float* S32;
   float* tail_part;
   int32_t* tail_cnt;
-  long long tail_cap;
+  long long tail_cap;  // split items, and the part slots they share
+  long long tail_slots;
   size_t clear_bytes;  // header and tail counters
   float2* node_d;      // user-provided nodes only: [n_tiles * ROX_SPAN] offsets, [n_tiles] bases
   float2* span_base;
@@ -196,7 +197,10 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
   w.hdr = (RoxWsHeader*)(base + off);
   off += ROX_WS_HEADER_BYTES;
   long long nt = n_tiles_of(n_grid);
-  w.tail_cap = nt < tail_max ? nt : tail_max;
+  w.tail_cap = tail_max;                       // split items
+  w.tail_slots = ROX_PARTS * (nt < tail_max ? nt : tail_max);
+  const long long least = tail_max < ROX_TAIL_ITEMS_MAX ? ROX_PARTS * tail_max : ROX_TAIL_ITEMS_MAX;   // short grids: many parts
+  if (w.tail_slots < least) w.tail_slots = least;
   w.tail_cnt = (int32_t*)(base + off);         // next to the header: one memset clears both
   off += rox_align256((size_t)w.tail_cap * 4);
   w.clear_bytes = off;
@@ -211,7 +215,7 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
   w.S32 = (float*)(base + off);
   off += rox_align256((size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 4);
   w.tail_part = (float*)(base + off);
-  off += rox_tail_part_bytes(w.tail_cap);
+  off += rox_tail_part_bytes(w.tail_slots);
   w.node_d = nullptr;
   w.span_base = nullptr;
   if (nodes) {
@@ -386,21 +390,22 @@ long long job_cells(RoxJobDev* J, int32_t c_steps) {
 // not depend on what it is launched with.
 void set_parts(RoxJobDev* J, int32_t c_steps) {
   J->part_shift = rox_part_shift(J->n_spans);
-  J->max_parts = ROX_PARTS;
+  J->max_parts = (int32_t)rox_parts_cap(J->n_spans);
   if (c_steps <= 0) return;      // nodes: a span's share of the lines is not known beforehand
   // lines that an average span visits one by one: those within about 700 points where cells take the
   // rest, else all within the cutoff
   const double pts = (double)J->n_spans * ROX_SPAN + 2.0 * c_steps, reach = 2.0 * c_steps + ROX_SPAN;
   const double lines = (double)(J->l1 - J->l0) * (c_steps >= 2 * ROX_SPAN && reach > 1400.0 ? 1400.0 : reach) / pts;
   const double parts = std::ceil(2.0 * lines / 32.0) / (1 << J->part_shift);
-  J->max_parts = parts >= ROX_PARTS ? ROX_PARTS : (parts < 1.0 ? 1 : (int32_t)parts);
+  const double cap = (double)rox_parts_cap(J->n_spans);
+  J->max_parts = (int32_t)(parts >= cap ? cap : (parts < 1.0 ? 1.0 : parts));
 }
 
 // Voigt launches over the jobs, at most ROX_MAX_JOBS per launch; the work counter is reset
 // before each launch (the evaluation count keeps adding up). The last items of each launch,
 // up to tail_cap and half a round of the launch's warps, are split into their parts.
 int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* jobs, int n_jobs, RoxWsHeader* hdr,
-                      float* tail_part, int32_t* tail_cnt, long long tail_cap, const RoxMoments& mom, int nblocks,
+                      float* tail_part, int32_t* tail_cnt, long long tail_cap, long long tail_slots, const RoxMoments& mom, int nblocks,
                       cudaStream_t s, const rox_launch_config& cfg, bool nodes = false, int extras = 0, bool cleared = true) {
   static thread_local RoxVoigtArgs A;   // ~30 KB of per-job parameters, passed by value
   A.hdr = hdr;
@@ -423,8 +428,6 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
       items += J.n_spans;
       A.item_end[nj] = items;
     }
-    A.split_parts = 1;
-    for (int k = 0; k < nj; k++) A.split_parts = std::max(A.split_parts, A.job[k].max_parts);
     A.n_slots = (int32_t)slots;
     A.cells_task = slots < 152 * 64 ? 1 : 4;
     // whole items in complete rounds of the launch's warps, then at least one round of items in
@@ -433,10 +436,30 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
     long long split = items <= warps ? items : items % warps + (long long)cfg.split_rounds * warps;
     if (split > items) split = items;
     if (split > tail_cap) split = tail_cap;
+    // from the last job backwards, as many of them as the part slots hold
+    long long n_split = 0, used = 0;
+    for (int k = nj - 1; k >= 0; k--) {
+      const long long room = std::min<long long>(split - n_split, (tail_slots - used) / A.job[k].max_parts);
+      const long long n = std::min<long long>(A.job[k].n_spans, room);
+      A.slot0[k] = (int32_t)used;
+      n_split += n;
+      used += n * A.job[k].max_parts;
+      if (n < A.job[k].n_spans) {
+        for (int j = k - 1; j >= 0; j--) A.slot0[j] = 0;
+        break;
+      }
+    }
     A.n_jobs = nj;
     A.n_items = items;
-    A.n_whole = items - (int)split;
-    A.n_queue = A.n_whole + (int)split * A.split_parts;
+    A.n_whole = items - (int)n_split;
+    A.n_queue = 0;
+    for (int k = 0; k < nj; k++) {
+      const int item0 = k > 0 ? A.item_end[k - 1] : 0;
+      const int whole = std::min(std::max(A.n_whole - item0, 0), (int)A.job[k].n_spans);
+      A.n_queue += whole + (A.job[k].n_spans - whole) * A.job[k].max_parts;
+      A.q_end[k] = A.n_queue;
+    }
+    split = n_split;
     const long long need = ((long long)A.n_queue + cfg.warps_per_cta - 1) / cfg.warps_per_cta;
     const int blocks = need < nblocks ? (int)need : nblocks;
     int rc;
@@ -710,7 +733,7 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
           jg.push_back(jobs[k]);
           jg.back().list = tidx[k] - g0;
         }
-      if ((rc = launch_voigt_jobs(Ls, ng, jg.data(), (int)jg.size(), w.hdr, w.tail_part, w.tail_cnt, w.tail_cap,
+      if ((rc = launch_voigt_jobs(Ls, ng, jg.data(), (int)jg.size(), w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, w.tail_slots,
                                   w.mom, nblocks, s, cfg, false, ROX_VX_INDEX, g0 == 0)))
         return rc;
     }
@@ -721,7 +744,7 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
                        "scaling and span ranges kernel")))
     return rc;
   const int extras = br ? ROX_VX_BROAD : (pre ? ROX_VX_PRE : 0);
-  if ((rc = launch_voigt_jobs(&L0, 1, jobs.data(), n_pt, w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, w.mom, nblocks, s,
+  if ((rc = launch_voigt_jobs(&L0, 1, jobs.data(), n_pt, w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, w.tail_slots, w.mom, nblocks, s,
                               cfg, on_nodes, extras)))
     return rc;
   return ok();
@@ -949,20 +972,22 @@ namespace {
 struct JobsTail {
   float* part;
   int32_t* cnt;
-  long long cap;
+  long long cap, slots;    // split items, part slots
   size_t clear_bytes;      // header and counters
   RoxMoments mom;
 };
 size_t jobs_layout(const rox_job* jobs, int n_jobs, void* ws, double** S64, float** S32, JobsTail* tail) {
-  long long spans = 0, slots = 0;
+  long long spans = 0, slots = 0, parts = 0;
   for (int k = 0; k < n_jobs; k++) {
     if (jobs[k].n > 0 && jobs[k].first >= 0) {
       const long long ns = (jobs[k].first + jobs[k].n - 1) / ROX_SPAN - jobs[k].first / ROX_SPAN + 1;
       spans += ns;
       slots += rox_job_slots(ns);
+      parts += ns * rox_parts_cap(ns);
     }
   }
   const long long cap = spans < ROX_TAIL_ITEMS_MAX ? spans : ROX_TAIL_ITEMS_MAX;
+  if (parts > ROX_PARTS * ROX_TAIL_ITEMS_MAX) parts = ROX_PARTS * ROX_TAIL_ITEMS_MAX;
   size_t off = ROX_WS_HEADER_BYTES + rox_align256((size_t)cap * 4);     // counters next to the header
   if (tail) tail->clear_bytes = off;
   for (int k = 0; k < n_jobs; k++) {
@@ -974,10 +999,11 @@ size_t jobs_layout(const rox_job* jobs, int n_jobs, void* ws, double** S64, floa
   }
   if (tail) {
     tail->cap = cap;
+    tail->slots = parts;
     tail->part = (float*)((char*)ws + off);
     tail->cnt = (int32_t*)((char*)ws + ROX_WS_HEADER_BYTES);
   }
-  off += rox_tail_part_bytes(cap);
+  off += rox_tail_part_bytes(parts);
   if (tail) tail->mom = moments_at((char*)ws + off, slots);
   off += rox_mom_bytes(slots);
   return off;
@@ -1103,7 +1129,7 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     d.t_row = 0;
     set_parts(&d, L[j.list].c_steps);
   }
-  if ((rc = launch_voigt_jobs(L, n_lists, J.data(), n_jobs, hdr, tail.part, tail.cnt, tail.cap, tail.mom, nblocks, s,
+  if ((rc = launch_voigt_jobs(L, n_lists, J.data(), n_jobs, hdr, tail.part, tail.cnt, tail.cap, tail.slots, tail.mom, nblocks, s,
                               cfg)))
     return rc;
   return ok();

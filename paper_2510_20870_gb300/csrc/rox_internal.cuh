@@ -44,7 +44,7 @@ struct RoxWsHeader {
 
 // Voigt launch: up to ROX_MAX_LISTS prepared line lists and ROX_MAX_JOBS jobs, each job one
 // output window on its list's lattice at one (P,T) point; work items are (job, span) pairs.
-#define ROX_MAX_JOBS 256
+#define ROX_MAX_JOBS 224
 #define ROX_MAX_LISTS 8
 
 struct RoxListDev {
@@ -134,23 +134,31 @@ struct RoxJobDev {
   int32_t mom_off;  // the job's first slot in RoxVoigtArgs::mom and cstart (a multiple of 4)
   int32_t c_first;  // the cell of that slot
   int32_t part_shift;  // a span's parts: its batches of lines >> part_shift, 1 .. max_parts
-  int32_t max_parts;   // 1 .. ROX_PARTS
+  int32_t max_parts;   // 1 .. rox_parts_cap(n_spans)
   int32_t n_cells;  // cells with moments (slot n_cells holds only the first line beyond them); 0: none
 };
 
-// Every span's lines are summed as up to ROX_PARTS consecutive parts (batch-aligned), each from
+// Every span's lines are summed as up to rox_parts_cap consecutive parts (batch-aligned), each from
 // zero, and the part sums are added in part order. How many is fixed by the job and the span: a job of
 // many spans (three rounds of the GPU's warps or more) fills it with whole items and takes a part per 16
 // batches (a part's fixed work, some 400 instructions and the wait for its first batch, is not worth
 // less), a shorter one a part per 4 or per batch, at most about twice what its spans have on average (a
-// split item has a queue entry per possible part). A work item is normally a whole span; the
+// split item has a queue entry per possible part). Jobs of few spans may take more parts than 16, so
+// that a narrow window on a dense list still fills the GPU (12 spans of 4e6 lines: 192 warps with 16
+// parts, 1,536 with 128). A work item is normally a whole span; the
 // last items of a launch are split into their parts, taken by different warps: each part stores
 // its sum in the tail scratch and the last of them to finish adds the parts in the same order.
 // The result is the same either way, so it depends neither on the split nor on the launch grid.
 // How many items are split is chosen per launch so that the whole items fill complete rounds of
-// the launch's warps and the split ones end the launch in pieces of 1/ROX_PARTS of an item
-// (at most ROX_TAIL_ITEMS_MAX items, the size of the workspace's tail scratch).
+// the launch's warps and the split ones end the launch in pieces of a part (at most
+// ROX_TAIL_ITEMS_MAX items and the part slots of the workspace's tail scratch).
 #define ROX_PARTS 16
+#define ROX_PARTS_MAX 128
+#define ROX_JOB_PART_SLOTS 2048    // part slots that a job of few spans may use
+static inline long long rox_parts_cap(long long n_spans) {
+  const long long c = n_spans > 0 ? ROX_JOB_PART_SLOTS / n_spans : ROX_PARTS_MAX;
+  return c > ROX_PARTS_MAX ? ROX_PARTS_MAX : (c < ROX_PARTS ? ROX_PARTS : c);
+}
 static inline int32_t rox_part_shift(long long n_spans) { return n_spans >= 8192 ? 4 : (n_spans >= 2048 ? 2 : 0); }
 #define ROX_TAIL_ITEMS_MAX 8192
 // A part's sum: its ROX_SPAN points, then its values at the span's ROX_NODES Chebyshev points
@@ -160,7 +168,7 @@ static inline int32_t rox_part_shift(long long n_spans) { return n_spans >= 8192
 
 struct RoxVoigtArgs {
   RoxWsHeader* hdr;
-  float* tail_part;                 // [n_items - n_whole][ROX_PARTS][ROX_PART_FLOATS] part sums
+  float* tail_part;                 // [part slots][ROX_PART_FLOATS] part sums
   int32_t* tail_cnt;                // [n_items - n_whole] parts finished (zeroed per launch)
   float4* mom;                      // [slots][4] moments of the jobs' cells
   int32_t* cstart;                  // [slots] first line (position) of each cell
@@ -169,9 +177,10 @@ struct RoxVoigtArgs {
   int32_t n_slots;                  // slots over all jobs (0: no moments in this launch)
   int32_t n_items;                  // items (spans over all jobs); the last n_items - n_whole split
   int32_t n_whole;
-  int32_t split_parts;              // queue entries of a split item: the jobs' largest max_parts
-  int32_t n_queue;                  // queue entries: n_whole + (n_items - n_whole) * split_parts
+  int32_t n_queue;                  // queue entries: one per whole item, max_parts of its job per split item
   int32_t item_end[ROX_MAX_JOBS];   // item_end[k] = spans of jobs 0..k
+  int32_t q_end[ROX_MAX_JOBS];      // queue entries of jobs 0..k
+  int32_t slot0[ROX_MAX_JOBS];      // part slot of job k's first split item
   RoxListDev list[ROX_MAX_LISTS];
   RoxJobDev job[ROX_MAX_JOBS];
 };
@@ -211,8 +220,8 @@ static inline long long rox_job_slots(long long n_spans) {
 static inline size_t rox_mom_bytes(long long slots) {
   return rox_align256((size_t)slots * 64) + rox_align256((size_t)slots * 4);
 }
-// tail scratch of a workspace: `cap` items x ROX_PARTS x ROX_PART_FLOATS floats (the items' counters
-// lie next to the header)
-static inline size_t rox_tail_part_bytes(long long cap) {
-  return rox_align256((size_t)cap * ROX_PARTS * ROX_PART_FLOATS * sizeof(float));
+// tail scratch of a workspace: part slots of ROX_PART_FLOATS floats (the items' counters lie next to the
+// header)
+static inline size_t rox_tail_part_bytes(long long slots) {
+  return rox_align256((size_t)slots * ROX_PART_FLOATS * sizeof(float));
 }

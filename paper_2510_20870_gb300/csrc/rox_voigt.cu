@@ -112,6 +112,13 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
   return d;
 }
 
+// v += x with the running compensation c (Kahan) weighted by kw: 1 keeps it, 0 leaves the plain sum
+__device__ __forceinline__ void sum_add(float& v, float& c, float x, float kw) {
+  const float y = x - c, t = v + y;
+  c = ((t - v) - y) * kw;
+  v = t;
+}
+
 // Far-form constants of pair k, packed for the paired instructions.
 struct PairC {
   f32x2 A, B, P, Q;
@@ -748,7 +755,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   __shared__ __align__(16) float s_carry[W][2][12];   // moments of the edge lines so far, per side
   __shared__ __align__(8) float s_zacc[W][ROX_SPAN];
   __shared__ float s_tot[W][ROX_SPAN];    // the span's sum over its parts
-  __shared__ float s_part[W][2][ROX_SPAN];  // a part's sum and its compensation
+  __shared__ float s_part[W][3][ROX_SPAN];  // a part's sum and its compensation; the compensation of s_tot
   __shared__ __align__(16) f32x2 s_cf[W][16];   // a zoned line's form coefficients
   __shared__ int s_status;
 
@@ -767,7 +774,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   const float cheb = rox_cheb_x[lane];
   float* zacc = s_zacc[w];
   float* stot = s_tot[w];
-  float *part_tot = s_part[w][0] + lane, *part_cmp = s_part[w][1] + lane;   // [32 m]: this lane's points
+  float *part_tot = s_part[w][0] + lane, *part_cmp = s_part[w][1] + lane, *tot_cmp = s_part[w][2] + lane;   // [32 m]: this lane's points
   f32x2* cbuf = s_cf[w];
   float* carry = s_carry[w][0];
   const float* cr = rox_core_r[lane & 15];
@@ -782,23 +789,25 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     int q = 0, k = 0;
     if (lane == 0) {
       q = atomicAdd(&A.hdr->work_counter, 1);
-      const int it = q < A.n_whole ? q : A.n_whole + (q - A.n_whole) / A.split_parts;
-      int lo_k = 0, hi_k = A.n_jobs - 1;           // first job with item_end > it
+      int lo_k = 0, hi_k = A.n_jobs - 1;           // first job with q_end > q
       while (lo_k < hi_k) {
         const int mid = (lo_k + hi_k) >> 1;
-        if (A.item_end[mid] > it) hi_k = mid; else lo_k = mid + 1;
+        if (A.q_end[mid] > q) hi_k = mid; else lo_k = mid + 1;
       }
       k = lo_k;
     }
     q = __shfl_sync(0xffffffffu, q, 0);
     k = __shfl_sync(0xffffffffu, k, 0);
     if (q >= A.n_queue) break;
-    // queue entry -> item and part (-1: the whole span, all parts in order)
-    const int item = q < A.n_whole ? q : A.n_whole + (q - A.n_whole) / A.split_parts;
-    const int part = q < A.n_whole ? -1 : (q - A.n_whole) % A.split_parts;
+    // queue entry -> the job's item and part (-1: the whole span, all parts in order)
     const RoxJobDev& J = A.job[k];
     const RoxListDev& Lst = A.list[J.list];
-    const int local = item - (k > 0 ? A.item_end[k - 1] : 0);
+    const int item0 = k > 0 ? A.item_end[k - 1] : 0;
+    const int whole = min(max(A.n_whole - item0, 0), J.n_spans);     // the job's whole items come first
+    const int lq = q - (k > 0 ? A.q_end[k - 1] : 0), sq = lq - whole;
+    const int local = sq < 0 ? lq : whole + sq / J.max_parts, part = sq < 0 ? -1 : sq % J.max_parts;
+    const int cnt_i = item0 + local - A.n_whole;                     // split items: counter, first part slot
+    const int slot0 = A.slot0[k] + (local - whole) * J.max_parts;
     const int span = J.span_first + J.n_spans - 1 - local;       // wide-line (high nu) spans first
     const int f16 = Lst.width_f16;
     // compensation weight of the part sums: 1 (ROX_KAHAN) keeps the Kahan correction term, 0
@@ -824,7 +833,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     const float half = NU ? 0.5f * Ws : 0.5f * (ROX_SPAN - 1) * dnu_f;
     const float tau = NU ? fmaf(cheb, half, half) : fmaf(cheb, 0.5f * (ROX_SPAN - 1), 0.5f * (ROX_SPAN - 1));
     const float inv_cut = rox_rcp(Lst.cutoff_f);
-    float ntot = 0.f;   // whole items: this lane's Chebyshev point, over the parts
+    float ntot = 0.f, ncmt = 0.f;   // whole items: this lane's Chebyshev point, over the parts
     const int lo = (int)max(Lst.span_lo[span], J.l0), hi = (int)min(Lst.span_hi[span], J.l1);   // at most 2e9 lines
     const int wlo = (int)max(J.first, (long long)Aw);              // evaluated points of this span
     const int whi = (int)min(J.first + J.n - 1, (long long)Bw);
@@ -906,8 +915,8 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     if (part >= np) continue;
     const int p_first = part < 0 ? 0 : part, p_last = part < 0 ? np - 1 : part;
     for (int p = p_first; p <= p_last; p++) {
-      const int plo = 32 * ((nbat * p) / np);
-      const int phi = min(nn, 32 * ((nbat * (p + 1)) / np));
+      const int plo = 32 * (int)((long long)nbat * p / np);
+      const int phi = min(nn, 32 * (int)((long long)nbat * (p + 1) / np));
       // the part's total and its compensation: in shared memory (touched once in four batches),
       // Chebyshev point in nsum, ncmp
       int ekL = 0, ekR = 0;             // edge lines: first point without its final sum, per side
@@ -1173,16 +1182,13 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         if ((nb & 3) == 3 || b0 + 32 >= mhi) {
 #pragma unroll
           for (int m = 0; m < ROX_K; m++) {
-            const float t0 = part_tot[32 * m], yk = acc[m] - part_cmp[32 * m];
-            const float tk = t0 + yk;
-            part_cmp[32 * m] = ((tk - t0) - yk) * kw;
-            part_tot[32 * m] = tk;
+            float v = part_tot[32 * m], c = part_cmp[32 * m];
+            sum_add(v, c, acc[m], kw);
+            part_tot[32 * m] = v;
+            part_cmp[32 * m] = c;
             acc[m] = 0.f;
           }
-          const float yn = nacc - ncmp;
-          const float tn = nsum + yn;
-          ncmp = ((tn - nsum) - yn) * kw;
-          nsum = tn;
+          sum_add(nsum, ncmp, nacc, kw);
           nacc = 0.f;
         }
       }
@@ -1213,14 +1219,19 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         part_tot[32 * m] += zacc[32 * m + lane] - part_cmp[32 * m];
       }
       if (part >= 0) {           // a split item: this part's sum goes to the tail scratch
-        float* dst = A.tail_part + ((size_t)(item - A.n_whole) * ROX_PARTS + p) * ROX_PART_FLOATS;
+        float* dst = A.tail_part + (size_t)(slot0 + p) * ROX_PART_FLOATS;
 #pragma unroll
         for (int m = 0; m < ROX_K; m++) __stcg(&dst[32 * m + lane], part_tot[32 * m]);
         __stcg(&dst[ROX_SPAN + lane], nsum);
       } else {
-        ntot = p == 0 ? nsum : ntot + nsum;
+        sum_add(ntot, ncmt, nsum, kw);
 #pragma unroll
-        for (int m = 0; m < ROX_K; m++) stot[32 * m + lane] = p == 0 ? part_tot[32 * m] : stot[32 * m + lane] + part_tot[32 * m];
+        for (int m = 0; m < ROX_K; m++) {
+          float v = p == 0 ? 0.f : stot[32 * m + lane], c = p == 0 ? 0.f : tot_cmp[32 * m];
+          sum_add(v, c, part_tot[32 * m], kw);
+          stot[32 * m + lane] = v;
+          tot_cmp[32 * m] = c;
+        }
       }
       __syncwarp();
     }   // parts
@@ -1230,21 +1241,22 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
       __threadfence();
       __syncwarp();
       int done = 0;
-      if (lane == 0) done = atomicAdd(&A.tail_cnt[item - A.n_whole], 1);
+      if (lane == 0) done = atomicAdd(&A.tail_cnt[cnt_i], 1);
       done = __shfl_sync(0xffffffffu, done, 0);
       if (done != np - 1) continue;
       __threadfence();
-      const float* src = A.tail_part + (size_t)(item - A.n_whole) * ROX_PARTS * ROX_PART_FLOATS;
+      const float* src = A.tail_part + (size_t)slot0 * ROX_PART_FLOATS + lane;
+      float v[ROX_K], c[ROX_K];
 #pragma unroll
-      for (int m = 0; m < ROX_K; m++) {
-        float v = __ldcg(&src[32 * m + lane]);
-#pragma unroll 4
-        for (int pp = 1; pp < np; pp++) v = v + __ldcg(&src[pp * ROX_PART_FLOATS + 32 * m + lane]);
-        stot[32 * m + lane] = v;
+      for (int m = 0; m < ROX_K; m++) v[m] = c[m] = 0.f;
+#pragma unroll 2
+      for (int pp = 0; pp < np; pp++) {
+#pragma unroll
+        for (int m = 0; m < ROX_K; m++) sum_add(v[m], c[m], __ldcg(&src[pp * ROX_PART_FLOATS + 32 * m]), kw);
+        sum_add(ntot, ncmt, __ldcg(&src[pp * ROX_PART_FLOATS + ROX_SPAN]), kw);
       }
-      ntot = __ldcg(&src[ROX_SPAN + lane]);
-#pragma unroll 4
-      for (int pp = 1; pp < np; pp++) ntot = ntot + __ldcg(&src[pp * ROX_PART_FLOATS + ROX_SPAN + lane]);
+#pragma unroll
+      for (int m = 0; m < ROX_K; m++) stot[32 * m + lane] = v[m];
     }
     // ---- the smooth lines' sum at the Chebyshev points, interpolated to the span's points
     if (__any_sync(0xffffffffu, ntot != 0.f)) interp_span<NU>(ntot, lane, D, half, stot);
