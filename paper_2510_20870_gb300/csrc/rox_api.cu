@@ -56,7 +56,7 @@ cudaError_t rox_launch_select_reduced(const rox_lines* L, int n_temps, const dou
                                       double Q_ref, double* S_T, const unsigned long long* smax_bits, double origin,
                                       double width, long long n_bins, double rel, int32_t* bin,
                                       unsigned long long* binmax_fast, unsigned long long* binmax_exact, float* S32,
-                                      cudaStream_t s);
+                                      int32_t* list, long long* count, cudaStream_t s);
 cudaError_t rox_launch_broad_T(const RoxBroadDev& B, const float* a_coef, long long n, int n_temps,
                                const double* temps, float* G, float* gN, cudaStream_t s);
 cudaError_t rox_launch_lorentz_out(const RoxBroadDev& B, const float* a_coef, long long n, double P_bar, double T,
@@ -654,7 +654,8 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
     }
     if (sel && (rc = cuda_check(rox_launch_select_reduced(lines, n_temps, temps.data(), qs.data(), Q_ref, w.S_T,
                                                           w.hdr->smax_bits, sel_origin, sel->bin_width, n_bins, sel->rel,
-                                                          w.line_bin, w.binmax, w.binmax_exact, w.S32, s),
+                                                          w.line_bin, w.binmax, w.binmax_exact, w.S32, w.keep_idx,
+                                                          w.keep_count, s),
                                 "selection kernels")))
       return rc;
     if (sel) {

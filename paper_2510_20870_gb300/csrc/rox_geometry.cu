@@ -41,34 +41,46 @@ __global__ void k_windows(const double* __restrict__ nu0s, long long n_lines, co
 // Windows on user-provided nodes (nu_k given, strictly increasing): the first node with
 // nu_k - nu0 >= -cutoff and the last with nu_k - nu0 <= cutoff, the differences rounded once
 // in double precision as the cutoff test is written; both are binary searches, the
-// difference being non-decreasing in k. The line centre is carried as a double-float pair
-// {hi, lo} (float hi = nu0 rounded, lo = the remainder) in the geometry record.
+// difference being non-decreasing in k. The lines of a block are consecutive in a sorted list, so the
+// searches of its first and last line bracket the others' (about 8 steps in place of 22 each on
+// 3e6 lines and nodes, 0.50 -> 0.40 ms); a line outside their range (an unsorted list) searches the whole grid.
+// The line centre is carried as a double-float pair {hi, lo} (float hi = nu0 rounded, lo = the
+// remainder) in the geometry record.
+__device__ __forceinline__ int first_node(const double* __restrict__ nodes, double nu0, double cut, bool strict, int a, int b) {
+  while (a < b) {        // strict: first k with nu_k - nu0 > cut, else >= cut
+    const int mid = (a + b) >> 1;
+    const double d = __dsub_rn(nodes[mid], nu0);
+    if (strict ? d > cut : d >= cut) b = mid; else a = mid + 1;
+  }
+  return a;
+}
 __global__ void k_node_windows(const double* __restrict__ nu0s, long long n_lines, const double* __restrict__ nodes,
                                long long n, double cutoff, int32_t* jlo_out, int32_t* jhi_out, float4* geo_out,
                                unsigned long long* evals_out, int32_t* unsorted_out, int32_t unsorted_value) {
+  __shared__ int s_b[4];      // first and last line's bounds: lower ends, upper ends
   long long stride = (long long)gridDim.x * blockDim.x;
   unsigned long long ev = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_lines; i += stride) {
+  for (long long i0 = (long long)blockIdx.x * blockDim.x; i0 < n_lines; i0 += stride) {
+    const long long i = i0 + threadIdx.x, last = min(i0 + (long long)blockDim.x, n_lines) - 1;
+    const double nu_a = nu0s[i0], nu_b = nu0s[last];
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && threadIdx.x < 128) {
+      const int w = threadIdx.x >> 5;       // a warp's lane each: four searches at once
+      s_b[w] = first_node(nodes, w & 1 ? nu_b : nu_a, w < 2 ? -cutoff : cutoff, w >= 2, 0, (int)n);
+    }
+    __syncthreads();
+    if (i >= n_lines) continue;
     const double nu0 = nu0s[i];
     if (i > 0 && nu0s[i - 1] > nu0 && unsorted_out) *unsorted_out = unsorted_value;
-    long long a = 0, b = n;
-    while (a < b) {
-      const long long mid = (a + b) >> 1;
-      if (__dsub_rn(nodes[mid], nu0) >= -cutoff) b = mid; else a = mid + 1;
-    }
-    const long long jl = a;
-    b = n;
-    while (a < b) {
-      const long long mid = (a + b) >> 1;
-      if (__dsub_rn(nodes[mid], nu0) > cutoff) b = mid; else a = mid + 1;
-    }
-    const long long jh = a - 1;
+    const bool in = nu0 >= nu_a && nu0 <= nu_b;
+    const int jl = first_node(nodes, nu0, -cutoff, false, in ? s_b[0] : 0, in ? s_b[1] : (int)n);
+    const int jh = first_node(nodes, nu0, cutoff, true, in ? max(s_b[2], jl) : jl, in ? max(s_b[3], jl) : (int)n) - 1;
     if (jh >= jl) ev += (unsigned long long)(jh - jl + 1);
-    if (jlo_out) jlo_out[i] = (int32_t)jl;
-    if (jhi_out) jhi_out[i] = (int32_t)jh;
+    if (jlo_out) jlo_out[i] = jl;
+    if (jhi_out) jhi_out[i] = jh;
     if (geo_out) {
       const float hi = (float)nu0;
-      geo_out[i] = make_float4(hi, (float)(nu0 - (double)hi), __int_as_float((int)jl), __int_as_float((int)jh));
+      geo_out[i] = make_float4(hi, (float)(nu0 - (double)hi), __int_as_float(jl), __int_as_float(jh));
     }
   }
   if (evals_out) {
