@@ -2,6 +2,7 @@
 // can be measured against scipy.special.wofz without a GPU.
 #include <stdint.h>
 #include "rox_faddeeva.cuh"
+#include "rox_strength_df.h"
 
 extern "C" void rox_host_re_w(const float* x, const float* y, float* out, int64_t n) {
   for (int64_t i = 0; i < n; i++) out[i] = rox_re_w(&rox_daw_taylor[0][0], x[i], y[i]);
@@ -41,5 +42,24 @@ extern "C" void rox_host_core_zone(const float* x, const float* y, float* out, i
     } else {
       out[i] = r;
     }
+  }
+}
+
+// the pair form of the line strength: hi, lo, exponent (e = INT32_MIN where it declines), and the
+// rounded value with a flag for "certain"
+extern "C" void rox_host_strength_df(int hitran, double c2_dT, double q_fac, double c2_T, double c2_Tref, const double* nu0,
+                                     const float* s_or_a, const float* g_up, const float* e_lower, float* hi, float* lo,
+                                     int32_t* ex, float* rounded, uint8_t* certain, int64_t n) {
+  const rox_df_consts k = rox_df_make_consts(hitran, c2_dT, q_fac, c2_T, c2_Tref);
+  rox_df tab[32];
+  for (int j = 0; j < 32; j++) tab[j] = rox_df_split(exp2(j / 32.0));
+  for (int64_t i = 0; i < n; i++) {
+    rox_df s;
+    int e;
+    const bool ok = rox_df_strength(k, tab, nu0[i], s_or_a[i], hitran ? 1.0f : g_up[i], e_lower[i], &s, &e);
+    hi[i] = ok ? s.h : 0.0f;
+    lo[i] = ok ? s.l : 0.0f;
+    ex[i] = ok ? e : INT32_MIN;
+    certain[i] = ok && rox_df_round(s, e, &rounded[i]);
   }
 }
