@@ -47,8 +47,8 @@ cudaError_t rox_launch_prep_lines(const rox_lines* L, const rox_grid* g, double 
                                   const double* q_of_temp, double Q_ref, double* S_T, RoxWsHeader* hdr, float4* geo,
                                   cudaStream_t s);
 cudaError_t rox_launch_prep_scaled(const RoxListDev& L, const RoxJobDev& J, long long n, int n_temps, const double* S_T,
-                                   const RoxWsHeader* hdr, float* S32, const float4* geo, long long n_spans,
-                                   long long* lo, long long* hi, float4* rec, cudaStream_t s);
+                                   const unsigned long long* smax_bits, float* S32, const float4* geo,
+                                   long long n_spans, long long* lo, long long* hi, float4* rec, cudaStream_t s);
 cudaError_t rox_launch_select(const double* nu0, const double* S_T, long long n, int n_temps,
                               const unsigned long long* smax_bits, double origin, double width, long long n_bins,
                               double rel, int32_t* bin, unsigned long long* binmax_bits, float* S32, cudaStream_t s);
@@ -184,7 +184,7 @@ struct WsLayout {
   float* broad_G;      // broadening descriptions only: [n_temps][n_lines] broadeners' sums, [n_lines]
   float* broad_N;      //   natural widths
   RoxMoments mom;      // uniform grids: moments of ROX_MOM_JOBS jobs' cells
-  float4* rec;         // one temperature on a uniform grid: per line 3 float4 of per-line constants
+  float4* rec;         // one temperature (nodes: up to ROX_PRE_POINTS): per line 3 float4 of per-line constants
   size_t bytes;
 };
 
@@ -271,9 +271,9 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
     off += rox_mom_bytes(slots);
   }
   w.rec = nullptr;
-  if (pre && n_temps == 1 && !nodes && n_bins == 0 && !broad) {
+  if (pre && n_temps <= (nodes ? ROX_PRE_POINTS : 1) && n_bins == 0 && !broad) {
     w.rec = (float4*)(base + off);
-    off += rox_align256((size_t)(n_lines > 0 ? n_lines : 1) * 3 * sizeof(float4));
+    off += rox_align256((size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 3 * sizeof(float4));
   }
   w.bytes = off;
   return w;
@@ -341,18 +341,18 @@ rox_launch_config launch_config() {
   return g_cfg;
 }
 
-// resident CTAs per SM of each instantiation (uniform grid, nodes, precomputed per-line
-// constants) and warps per CTA (4, 8) on the current device
-int g_voigt_per_sm[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-int g_voigt_sms[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-int g_voigt_device[3][2] = {{-1, -1}, {-1, -1}, {-1, -1}};
+// resident CTAs per SM of each instantiation (uniform grid, nodes, and either with precomputed
+// per-line constants) and warps per CTA (4, 8) on the current device
+int g_voigt_per_sm[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+int g_voigt_sms[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+int g_voigt_device[4][2] = {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}};
 
 // persistent grid of the Voigt kernel on the current device for the launch configuration cfg
 int voigt_grid(int* out, const rox_launch_config& cfg, bool nodes = false, bool pre = false) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_check(e, "cudaGetDevice");
-  const int v = pre ? 2 : (nodes ? 1 : 0), wi = cfg.warps_per_cta == 4 ? 0 : 1;
+  const int v = (pre ? 2 : 0) + (nodes ? 1 : 0), wi = cfg.warps_per_cta == 4 ? 0 : 1;
   if (dev != g_voigt_device[v][wi]) {
     int sms = 0, per = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -620,8 +620,8 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
   const int n_temps = (int)temps.size();
   if (!ws || ((uintptr_t)ws & 255)) return fail(ROX_EINVAL, "workspace NULL or not 256-byte aligned");
   WsLayout w = ws_layout(ws, lines->n, n_grid, n_temps, on_nodes, n_bins, br != nullptr, tail_max, allow_pre);
-  // one (P,T) point on a uniform grid: the per-line constants once per line (k_line_params)
-  const bool pre = w.rec != nullptr && n_pt == 1 && lines->n > 0;
+  // one (P,T) point per temperature: the per-line constants once per line
+  const bool pre = w.rec != nullptr && n_pt == n_temps && lines->n > 0;
   if (ws_bytes < w.bytes) return fail(ROX_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, w.bytes);
 
   cudaStream_t s = (cudaStream_t)stream;
@@ -694,13 +694,13 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
   L0.width_f16 = lines->width_dtype == ROX_WIDTH_F16;
   L0.idx = nullptr;
   L0.inv_dnu_f = on_nodes ? 0.0f : (float)(1.0 / grid->dnu);
-  L0.rec = pre ? w.rec : nullptr;
   L0.cutoff_f = (float)cutoff;
   L0.c_steps = on_nodes ? 0 : cutoff_steps(cutoff, grid->dnu);
   std::vector<RoxJobDev> jobs(n_pt);
   for (int k = 0; k < n_pt; k++) {
     RoxJobDev& J = jobs[k];
-    J.S32 = w.S32 + (size_t)tidx[k] * (size_t)(nl > 0 ? nl : 1);
+    J.S32 = pre ? reinterpret_cast<const float*>(w.rec + (size_t)k * (size_t)nl * 3)
+                : w.S32 + (size_t)tidx[k] * (size_t)(nl > 0 ? nl : 1);
     J.sigma = sigma_out + (size_t)k * (size_t)n_grid;
     J.smax_bits = &w.hdr->smax_bits[tidx[k]];
     J.l0 = 0;
@@ -740,10 +740,13 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
     }
     return ok();
   }
-  if ((rc = cuda_check(rox_launch_prep_scaled(L0, jobs[0], nl, nl > 0 ? n_temps : 1, w.S_T, w.hdr, w.S32, w.geo, nt, w.tlo,
-                                              w.thi, pre ? w.rec : nullptr, s),
-                       "scaling and span ranges kernel")))
-    return rc;
+  // with constants, one launch per point (point k is the only one of temperature k)
+  for (int k = 0; k < (pre ? n_pt : 1); k++)
+    if ((rc = cuda_check(rox_launch_prep_scaled(L0, jobs[k], nl, pre || nl == 0 ? 1 : n_temps, w.S_T + (size_t)k * (size_t)nl,
+                                                &w.hdr->smax_bits[k], w.S32, w.geo, nt, k == 0 ? w.tlo : nullptr,
+                                                k == 0 ? w.thi : nullptr, pre ? w.rec + (size_t)k * (size_t)nl * 3 : nullptr, s),
+                         "scaling and span ranges kernel")))
+      return rc;
   const int extras = br ? ROX_VX_BROAD : (pre ? ROX_VX_PRE : 0);
   if ((rc = launch_voigt_jobs(&L0, 1, jobs.data(), n_pt, w.hdr, w.tail_part, w.tail_cnt, w.tail_cap, w.tail_slots, w.mom, nblocks, s,
                               cfg, on_nodes, extras)))
@@ -1105,7 +1108,6 @@ int rox_xsec_jobs(const rox_prepared* lists, int n_lists, const rox_job* jobs, i
     L[l].nu_min_f = (float)P.lattice.nu_min;
     L[l].width_f16 = P.lines.width_dtype == ROX_WIDTH_F16;
     L[l].inv_dnu_f = (float)(1.0 / P.lattice.dnu);
-    L[l].rec = nullptr;
     L[l].cutoff_f = (float)P.cutoff;
     L[l].c_steps = cutoff_steps(P.cutoff, P.lattice.dnu);
   }

@@ -42,15 +42,42 @@ __global__ void k_windows(const double* __restrict__ nu0s, long long n_lines, co
 // nu_k - nu0 >= -cutoff and the last with nu_k - nu0 <= cutoff, the differences rounded once
 // in double precision as the cutoff test is written; both are binary searches, the
 // difference being non-decreasing in k. The lines of a block are consecutive in a sorted list, so the
-// searches of its first and last line bracket the others' (about 8 steps in place of 22 each on
-// 3e6 lines and nodes, 0.50 -> 0.40 ms); a line outside their range (an unsorted list) searches the whole grid.
-// The line centre is carried as a double-float pair {hi, lo} (float hi = nu0 rounded, lo = the
-// remainder) in the geometry record.
+// searches of its first and last line bracket the others' (about 8 steps in place of 22 each); a line
+// outside their range (an unsorted list) searches the whole grid. 3e6 lines, 3e6 nodes: 0.50 -> 0.40 ms
+// so, 0.146 ms with the comparisons as integers. The line centre is carried as a double-float pair
+// {hi, lo} (float hi = nu0 rounded, lo = the remainder) in the geometry record.
+// Nodes are compared with nu0 -+ cutoff as integers that order like them (FP64 comparisons
+// issue at two per clock per SM); the rounded sum may be a few units off, so the exact test moves the result
+// to the boundary from there.
+__device__ __forceinline__ long long node_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b >= 0 ? b : (long long)(0x8000000000000000ULL - (unsigned long long)b);
+}
 __device__ __forceinline__ int first_node(const double* __restrict__ nodes, double nu0, double cut, bool strict, int a, int b) {
-  while (a < b) {        // strict: first k with nu_k - nu0 > cut, else >= cut
+  // strict: first k in [a, b) with nu_k - nu0 > cut, else >= cut; b if none (a NaN centre: none)
+  const auto past = [&](int k) {
+    const double d = __dsub_rn(nodes[k], nu0);
+    return strict ? d > cut : d >= cut;
+  };
+  if (!(nu0 == nu0)) return b;
+  const int first = a, end = b;
+  const long long key = node_key(nu0 + cut);
+  while (a < b) {
     const int mid = (a + b) >> 1;
-    const double d = __dsub_rn(nodes[mid], nu0);
-    if (strict ? d > cut : d >= cut) b = mid; else a = mid + 1;
+    if (node_key(nodes[mid]) >= key) b = mid; else a = mid + 1;
+  }
+#pragma unroll 1
+  for (int step = 0; step < 8; step++) {
+    if (a > first && past(a - 1)) a--;
+    else if (a < end && !past(a)) a++;
+    else return a;
+  }
+  // many nodes within the rounding (or nodes that do not increase: an error the call reports)
+  a = first;
+  b = end;
+  while (a < b) {
+    const int mid = (a + b) >> 1;
+    if (past(mid)) b = mid; else a = mid + 1;
   }
   return a;
 }

@@ -68,10 +68,6 @@ struct RoxListDev {
   // {nu0 hi, nu0 lo, jlo, jhi}
   const float2* node_d;
   const float2* span_base;
-  // precomputed per-line constants of the launch's one (P,T) point (ROX_VX_PRE lists, else NULL):
-  // per line 3 float4, {A, B, P, Q}, {t_z, 1/gamma_G, y, S/(gamma_G
-  // sqrt(pi))}, {X^2 of the end of its own zone (LineTab::z), zlo, zhi (int bits), smooth_dmin}
-  const float4* rec;
   long long n_lattice;
   float dnu_f;
   float nu_min_f;
@@ -113,10 +109,18 @@ struct RoxBroadDev {
 // extras of a Voigt launch (kernel instantiations)
 #define ROX_VX_INDEX 1    // lists are subsets of the sorted lines given by an index (RoxListDev::idx)
 #define ROX_VX_BROAD 2    // widths from the broadening pass (RoxListDev::gLT, gN)
-#define ROX_VX_PRE 4      // per-line constants precomputed for the launch's one (P,T) point (RoxListDev::rec)
+#define ROX_VX_PRE 4      // per-line constants precomputed for each (P,T) point (RoxJobDev::S32)
+// (P,T) points up to which a call on user-provided nodes keeps them, 48 bytes of workspace per line and
+// point (on a uniform grid: one, where most pairs need only the cells' moments). 3e6 lines, 3e6 nodes, two
+// points: constants per span 4.85 ms, kept 4.57 ms.
+#define ROX_PRE_POINTS 4
 
 struct RoxJobDev {
-  const float* S32;                      // S * 2^-e of lines l0, l0+1, ... at this job's T
+  // S * 2^-e of lines l0, l0+1, ... at this job's T. In a ROX_VX_PRE launch the job's per-line
+  // constants instead, 3 float4 for each line of the list: {A, B, P, Q}, {t_z, 1/gamma_G, y,
+  // S/(gamma_G sqrt(pi))}, {X^2 of the end of its own zone (LineTab::z), zlo, zhi (int bits),
+  // smooth_dmin}; on user-provided nodes the last is {X^2, zone half-width, 0, smooth_dmin at width 0}
+  const float* S32;
   float* sigma;                          // sigma[j - first] for lattice points j in [first, first + n)
   const unsigned long long* smax_bits;   // this job's largest strength (double bits)
   long long l0;

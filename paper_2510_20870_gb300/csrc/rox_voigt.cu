@@ -673,12 +673,13 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
         if (in) {
           float a, b, p, q, hz;
           if constexpr (PRE) {
-            const float4 r0 = L.rec[3 * li];
+            const float4* rec = reinterpret_cast<const float4*>(J.S32);
+            const float4 r0 = rec[3 * li];
             a = r0.x;
             b = r0.y;
             p = r0.z;
             q = r0.w;
-            const float z2 = fmaxf(L.rec[3 * li + 1].x - a, 0.f) + 1e-30f;   // t_z = hz^2 + A
+            const float z2 = fmaxf(rec[3 * li + 1].x - a, 0.f) + 1e-30f;   // t_z = hz^2 + A
             hz = z2 * rox_rsqrt(z2) * 1.001f;
           } else {
             float gref, nt;
@@ -781,7 +782,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   const float4 core_r = make_float4(cr[0], cr[1], cr[2], cr[3]);
   float2* Drow = NU ? s_nodes + w * ROX_SPAN : nullptr;   // this span's node offsets
   // PRE: per warp 32 lines x 3 float4 of per-line constants
-  float4(*rec_st)[3] = PRE ? reinterpret_cast<float4(*)[3]>(s_nodes) + 32 * w : nullptr;
+  float4(*rec_st)[3] = PRE ? reinterpret_cast<float4(*)[3]>(s_nodes + (NU ? W * ROX_SPAN : 0)) + 32 * w : nullptr;
   const float2* D = NU ? Drow + lane : nullptr;
   unsigned long long evals = 0;   // (line, point) pairs inside the cutoff and the job's window
 
@@ -840,6 +841,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     const double smax = __longlong_as_double((long long)*J.smax_bits);
     const int e = smax > 0.0 ? ilogb(smax) : 0;     // S32 holds S * 2^-e (FP32)
     const float* S_row = J.S32 - J.l0;              // indexed by line number
+    const float4* rec = reinterpret_cast<const float4*>(J.S32);   // PRE: the job's constants of every line
 
     // Cells taken through their moments: left of the span [cl0, cl1), right of it [cr0, cr1), all of
     // whose lines cover the span, far enough for the expansion and for the lines' slow zones. Their
@@ -950,7 +952,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
             const int li = IDX ? Lst.idx[line_at(q)] : line_at(q);
             g_n = Lst.geo[li];
             if constexpr (PRE) {
-              const float4 r0 = Lst.rec[3 * (long long)li];
+              const float4 r0 = rec[3 * (long long)li];
               k_n.A = r0.x;
               k_n.B = r0.y;
               k_n.P = r0.z;
@@ -992,7 +994,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
           cp_async16(&geo_st[lane], &Lst.geo[li]);
           if constexpr (PRE) {
 #pragma unroll
-            for (int c = 0; c < 3; c++) cp_async16(&rec_st[lane][c], &Lst.rec[3 * (long long)li + c]);
+            for (int c = 0; c < 3; c++) cp_async16(&rec_st[lane][c], &rec[3 * (long long)li + c]);
           } else {
             cp_async4(&S_st[lane], &S_row[li]);
             load_widths<BRD>(J, Lst, f16, li, gref, nt);
@@ -1035,12 +1037,21 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
             kc.y = r1.z;
             kc.pc = r1.w;
             kc.zc = r2.x;
-            zlo = __float_as_int(r2.y);
-            zhi = __float_as_int(r2.z);
-            ax = (float)Aw - g.x;     // exact: both are integers below 2^24
-            ay = -g.y;
-            zoned = !(Bw < zlo || Aw > zhi);
-            dmin = r2.w;
+            if constexpr (NU) {
+              // c = nu0 - (span's first node) as a double-float pair (the hi parts cancel exactly)
+              const float ch = g.x - bh, cl = g.y - bl;
+              ax = ch + cl;
+              ay = cl - (ax - ch);
+              kc.hz = r2.y;
+              dmin = fmaf(ROX_SMOOTH_R, half, r2.w);
+            } else {
+              zlo = __float_as_int(r2.y);
+              zhi = __float_as_int(r2.z);
+              ax = (float)Aw - g.x;     // exact: both are integers below 2^24
+              ay = -g.y;
+              zoned = !(Bw < zlo || Aw > zhi);
+              dmin = r2.w;
+            }
           } else {
             const float Sp = S_st[lane];
             float nu0f;   // line centre; its offset state {E, F} (uniform grid) or {c hi, c lo} (nodes)
@@ -1056,19 +1067,17 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
               ay = -g.y;
             }
             kc = line_consts<BRD>(nu0f, Sp, gref, nt, J, margin_cm);
-            if constexpr (NU) {
-              // the span's offsets run from -c to Ws - c; pass 2 then scans the window itself
-              const float hzp = kc.hz * 1.001f + 1e-6f * (fabsf(ax) + Ws);
-              zoned = -ax < hzp && Ws - ax > -hzp;
-            } else {
+            if constexpr (!NU) {
               zone_bounds(g, kc.hz, Lst.inv_dnu_f, zlo, zhi);
               zoned = !(Bw < zlo || Aw > zhi);
             }
             dmin = smooth_dmin(kc.A, kc.B, half);
           }
           if constexpr (NU) {
+            // the span's offsets run from -c to Ws - c
+            const float hb = kc.hz * 1.001f + 1e-6f * (fabsf(ax) + Ws);
+            zoned = -ax < hb && Ws - ax > -hb;
             if (zoned) {   // the span's nodes within the zone, by bisection on their offsets (widened a little)
-              const float hb = kc.hz * 1.001f + 1e-6f * (fabsf(ax) + Ws);
               int q0 = 0, q1 = 0;
 #pragma unroll
               for (int st = ROX_SPAN / 2; st > 0; st >>= 1) {
@@ -1323,12 +1332,12 @@ __global__ void k_faddeeva(const float* x, const float* y, float* out, long long
 }  // namespace
 
 namespace {
-// dynamic shared memory of an instantiation with W warps per CTA: the node rows (NU) or the
+// dynamic shared memory of an instantiation with W warps per CTA: the node rows (NU), then the
 // staged per-line constants (ROX_VX_PRE)
 template <bool NU, int X, int W>
 constexpr size_t voigt_dyn_smem() {
-  return NU ? (size_t)W * ROX_SPAN * sizeof(float2)
-            : ((X & ROX_VX_PRE) ? (size_t)W * 32 * 3 * sizeof(float4) : (size_t)0);
+  return (NU ? (size_t)W * ROX_SPAN * sizeof(float2) : (size_t)0) +
+         ((X & ROX_VX_PRE) ? (size_t)W * 32 * 3 * sizeof(float4) : (size_t)0);
 }
 }  // namespace
 
@@ -1358,6 +1367,7 @@ cudaError_t blocks_k(int* nb) {
 template <int W>
 cudaError_t launch_w(const RoxVoigtArgs& A, int n_blocks, bool nodes, int extras, cudaStream_t s) {
   if (nodes) {
+    if (extras == ROX_VX_PRE) return launch_k<true, ROX_VX_PRE, W>(A, n_blocks, s);
     if (extras) return cudaErrorNotSupported;   // no caller combines nodes with a selection or broadening
     return launch_k<true, 0, W>(A, n_blocks, s);
   }
@@ -1372,7 +1382,7 @@ cudaError_t launch_w(const RoxVoigtArgs& A, int n_blocks, bool nodes, int extras
 
 template <int W>
 cudaError_t blocks_w(int* nb, bool nodes, bool pre) {
-  if (pre) return blocks_k<false, ROX_VX_PRE, W>(nb);
+  if (pre) return nodes ? blocks_k<true, ROX_VX_PRE, W>(nb) : blocks_k<false, ROX_VX_PRE, W>(nb);
   if (nodes) return blocks_k<true, 0, W>(nb);
   return blocks_k<false, 0, W>(nb);
 }

@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 import rox_synth as rs
-from rox_testutil import q_pair, to_device
+from rox_testutil import check_sigma, q_pair, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -66,16 +66,54 @@ def test_equal_strengths(rel):
 
 
 def test_unsorted_blocks_of_node_windows():
-    nodes = rs.fixed_resolution_grid(1000.0, 5000.0, 100_000)
-    rng = np.random.default_rng(8)
-    nu0 = np.sort(rng.uniform(900.0, 5100.0, 4000))
-    nu0[256:512] = rng.permutation(nu0[256:512])     # one block in disorder
-    nu0[700], nu0[900] = nu0[3900], nu0[3]           # single lines out of their block's range
-    nu0[1024:1280] = nu0[1024]                       # a block of equal centres
-    nu0[1300] = nodes[5000] + CUT                    # cutoff on a node
+    _check_node_windows(rs.fixed_resolution_grid(1000.0, 5000.0, 100_000))
+
+
+def test_node_windows_with_nodes_within_the_rounding():
+    """Hundreds of nodes closer to zero than the rounding of their distance from a line."""
+    nodes = np.concatenate([np.arange(1, 400) * 1e-18, np.geomspace(1e-10, 40.0, 500)])
+    c = np.concatenate([CUT + np.arange(-3, 4) * np.spacing(CUT), [1e-18, 24.0, 65.0]])
+    _compare(np.sort(c), nodes)
+
+
+def _compare(nu0, nodes):
     nd, d = torch.from_numpy(nodes).cuda(), torch.from_numpy(nu0).cuda()
     jlo = torch.empty(nu0.size, dtype=torch.int32, device="cuda")
     jhi = torch.empty_like(jlo)
     rox.rox_node_windows(d, nd, CUT, jlo, jhi)
     ol, oh = oracle.node_windows(nu0, nodes, CUT)
     assert np.array_equal(jlo.cpu().numpy(), ol) and np.array_equal(jhi.cpu().numpy(), oh)
+
+
+def _check_node_windows(nodes):
+    rng = np.random.default_rng(8)
+    nu0 = np.sort(rng.uniform(900.0, 5100.0, 4000))
+    nu0[256:512] = rng.permutation(nu0[256:512])     # one block in disorder
+    nu0[700], nu0[900] = nu0[3900], nu0[3]           # single lines out of their block's range
+    nu0[1024:1280] = nu0[1024]                       # a block of equal centres
+    nu0[1300] = nodes[5000] + CUT                    # cutoff on a node
+    _compare(nu0, nodes)
+
+
+@pytest.mark.parametrize("pts", [[(1.0, 400.0)], [(0.1, 300.0), (10.0, 1000.0), (1e-4, 2000.0), (1.0, 3000.0)],
+                                 [(1e-4, 300.0), (1.0, 600.0), (1.0, 900.0), (10.0, 1200.0), (0.01, 2500.0)],
+                                 [(1e-3, 700.0), (20.0, 700.0)]])
+def test_nodes_points_on_both_sides_of_the_record_limit(pts):
+    """Constants kept per line and point (each point its own temperature, at most four) or computed per
+    span (more temperatures, or two pressures at one), both against the oracle; its usual tolerance."""
+    w = rs.CONFIGS[1]
+    L = oracle.sort_lines(rs.make_lines(w, 0, 4000))
+    L = {key: v[(L["nu0"] > 1980.0) & (L["nu0"] < 2320.0)] if isinstance(v, np.ndarray) else v for key, v in L.items()}
+    nodes = rs.fixed_resolution_grid(2000.0, 2300.0, 60_000)
+    nd, dl = torch.from_numpy(nodes).cuda(), to_device(L, torch)
+    qs = [q_pair(w, T) for _, T in pts]
+    n_temps = len(set(T for _, T in pts))
+    ws = torch.empty(rox.rox_xsec_nodes_workspace_size(L["nu0"].size, nodes.size, n_temps), dtype=torch.uint8, device="cuda")
+    sigma = torch.empty((len(pts), nodes.size), dtype=torch.float32, device="cuda")
+    rox.rox_xsec_nodes_batch(dl, nd, [p for p, _ in pts], [t for _, t in pts], [q for q, _ in qs], qs[0][1], w.mass_amu,
+                             CUT, sigma, ws)
+    assert rox.rox_ws_status(ws)[0] == 0
+    got = sigma.double().cpu().numpy()
+    for k, (P, T) in enumerate(pts):
+        ref = oracle.xsec_nodes(L, nodes, P, T, qs[k][0], qs[k][1], w.mass_amu, CUT)
+        check_sigma(got[k], ref, label="nodes point %d of %d" % (k, len(pts)))
