@@ -34,17 +34,15 @@ import numpy as np  # noqa: E402
 
 import rox_synth as rs  # noqa: E402
 
-FLOPS_PER_EVAL = 11.0   # far-wing pair formula: 10 FFMA + 2 FMUL per 2 evaluations (+ 1 MUFU rcp)
-# DRAM bytes per Voigt launch on the full exomol workload: ncu dram__bytes_read + write of the
-# 2e6-line case (151.3 MB + 43.4 MB, profiles/k_voigt_exomol_2e6lines.md), scaled by evaluations
-# (x5.0); most of the writes are L2 write-backs of the per-line constants k_line_params wrote
-VOIGT_TRAFFIC_BYTES = 9.737e8
+# Warp instructions of k_voigt per evaluation (a (line, point) pair inside the cutoff), and DRAM bytes per
+# evaluation: ncu counters of one launch (profiles/k_voigt_counters.md). An evaluation is the definition's
+# unit of work; the kernel forms most of them from per-cell moments and interpolation, so flops per
+# evaluation mean nothing and the kernel is measured against the warp schedulers' issue rate, its bound.
+VOIGT_INST = {"exomol": None, "large": None}
+VOIGT_DRAM = {"exomol": None, "large": None}
 # DRAM bytes of one k_cia_grid launch on the CIA workload (ncu dram__bytes_read + write,
 # profiles/k_cia_grid_40T_2970001pts.md; part of the 950 MB output is still in L2 at the end)
 CIA_TRAFFIC_BYTES = 8.955e8
-# DRAM bytes per evaluation of k_voigt on the large list: ncu dram__bytes_read + write on one
-# 1e7-line chunk of it (4.170 GB for 1.989e11 evaluations, profiles/k_voigt_large_1e7_chunk.md)
-VOIGT_TRAFFIC_LARGE = 4.1697e9 / 1.98948e11
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
 METRIC = "Voigt line-profile evals/s"
@@ -556,17 +554,9 @@ def run_gpu(args):
 
     csum = clocks.summary()
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak = sms * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
-    v_ms = statistics.mean(voigt_ms)
-    achieved = evals * FLOPS_PER_EVAL / (v_ms * 1e-3) / 1e12
-    roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": VOIGT_TRAFFIC_BYTES if (args.config == 2 and args.lines is None and not args.nodes) else None,
-            "traffic_note": "ncu capture of the 2e6-line case scaled by evaluations", "kernel": "k_voigt",
-            "kernel_ms": v_ms,
-            "peak_basis": "%d SMs x 128 FP32 lanes x 2 flop x %.0f MHz (max SM clock)" % (sms, SM_MAX_MHZ),
-            "flops_per_eval": FLOPS_PER_EVAL}
-    if csum.get("sm_mhz"):
-        roof["frac_at_median_clock"] = achieved / (sms * FP32_LANES_PER_SM * 2 * csum["sm_mhz"] * 1e6 / 1e12)
+    kind = "exomol" if (args.config == 2 and args.lines is None and not args.nodes and args.select is None
+                        and not args.broadening) else None
+    roof = voigt_roofline(evals, statistics.mean(voigt_ms), kind, sms, csum)
 
     ws_mb = ws.numel() / 1e6
     sigma_bytes = sigma.numel() * 4
@@ -619,14 +609,15 @@ def run_gpu(args):
                             " and the nodes" if args.nodes else "", "rox_xsec_nodes_batch" if args.nodes else "rox_xsec",
                             "; two list buffers, step k+1's upload and sort overlap step k's cross-section"
                             if pipelined else "")},
-                "gpu_launches": args.steps * 6 if args.select is None else args.steps * 9,
+                "gpu_launches": args.steps * (11 if args.select is not None else 5 if args.nodes or args.broadening else 4),
                 "gpu_launches_note": (
-                    "per step: windows, strengths, line bins, bin maxima, FP64 fix-up of the bin maxima, "
-                    "selection and scaling, kept flags, span ranges over the kept lines, Voigt kernel (+ CUB's "
-                    "two select kernels and memsets)" if args.select is not None else
-                    "per step: %swindows, strengths, strength scaling, %stile ranges, %sVoigt kernel "
-                    "(+ memsets)" % ("node offsets, " if args.nodes else "", "broadening, " if args.broadening else "",
-                                     "" if args.nodes or args.broadening else "per-line constants, ")),
+                    "per step: windows and strengths, line bins, bin maxima, candidates, their FP64 maxima, "
+                    "thresholds, selection and scaling, kept flags, span ranges over the kept lines, moments, Voigt "
+                    "kernel (+ CUB's two select kernels and memsets)" if args.select is not None else
+                    "per step: node offsets, node windows, strengths, per-line constants and span ranges, Voigt "
+                    "kernel (+ memset)" if args.nodes else
+                    "per step: windows and strengths, %sscaling and span ranges, moments, Voigt kernel (+ memset)" % (
+                        "broadening, " if args.broadening else "")),
                 "clocks": csum}
         print(json.dumps(line))
     if dist is not None:
@@ -690,19 +681,23 @@ def loop_ceilings(dev_index, sms, out):
     return res
 
 
-def voigt_roofline(evals, kernel_ms, peaks, traffic, traffic_note, clocks):
-    achieved = evals * FLOPS_PER_EVAL / (kernel_ms * 1e-3) / 1e12
-    peak = peaks["formula_tflops"]
-    roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": traffic, "traffic_note": traffic_note, "kernel": "k_voigt", "kernel_ms": kernel_ms,
-            "peak_basis": peaks["formula_basis"], "flops_per_eval": FLOPS_PER_EVAL,
-            "peak_measured": peaks["measured_tflops"], "frac_of_measured": achieved / peaks["measured_tflops"],
-            "peak_measured_basis": peaks["measured_basis"], "peak_measured_sm_mhz": peaks.get("measured_sm_mhz")}
-    if peaks.get("pair_loop_evals_s"):
-        roof["pair_loop_ceiling_evals_s"] = peaks["pair_loop_evals_s"]
-        roof["frac_of_pair_loop"] = evals / (kernel_ms * 1e-3) / peaks["pair_loop_evals_s"]
-        roof["pair_loop_basis"] = peaks["pair_loop_basis"]
-    if clocks.get("sm_mhz"):
+def voigt_roofline(evals, kernel_ms, kind, sms, clocks, peaks=None):
+    """The Voigt kernel (with the moments pass ahead of it) against the issue rate of the warp schedulers,
+    one instruction per clock each. kind: the workload whose instruction and byte counts apply, or None."""
+    peak = sms * 4 * SM_MAX_MHZ * 1e6 / 1e12
+    inst, dram = VOIGT_INST.get(kind), VOIGT_DRAM.get(kind)
+    achieved = evals * inst / (kernel_ms * 1e-3) / 1e12 if inst else None
+    roof = {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "T warp instructions/s",
+            "frac": achieved / peak if inst else None, "kernel": "k_voigt", "kernel_ms": kernel_ms,
+            "peak_basis": "%d SMs x 4 schedulers x %.0f MHz (max SM clock)" % (sms, SM_MAX_MHZ),
+            "traffic": dram * evals if dram else None, "warp_inst_per_eval": inst,
+            "note": "instructions and DRAM bytes per evaluation from ncu on one launch of this list, times the "
+                    "evaluations; most evaluations come from moments and interpolation, not one by one"}
+    if peaks and peaks.get("pair_loop_evals_s"):
+        roof["pair_loop_evals_s"] = peaks["pair_loop_evals_s"]
+        roof["vs_pair_loop"] = evals / (kernel_ms * 1e-3) / peaks["pair_loop_evals_s"]
+        roof["pair_loop_basis"] = "every evaluation one by one: " + peaks["pair_loop_basis"]
+    if achieved and clocks.get("sm_mhz"):
         roof["frac_at_median_clock"] = achieved / (peak * clocks["sm_mhz"] / SM_MAX_MHZ)
     return roof
 
@@ -890,11 +885,7 @@ def run_large(args):
     torch.cuda.empty_cache()
 
     peaks = fp32_peaks(local, sms)
-    roof = voigt_roofline(evals, statistics.mean(voigt_ms), peaks,
-                          VOIGT_TRAFFIC_LARGE * evals if VOIGT_TRAFFIC_LARGE else None,
-                          "ncu dram__bytes_read + write of k_voigt on one 1e7-line chunk of this workload, per "
-                          "evaluation, times this step's evaluations (the kernel reads each line once per span it "
-                          "reaches; the traffic grows with the evaluations)", csum)
+    roof = voigt_roofline(evals, statistics.mean(voigt_ms), "large" if n == 1_000_000_000 else None, sms, csum, peaks)
     roof["kernel_ms_note"] = "sum over the %d chunk launches of one step (CUDA events around each launch)" % len(starts)
 
     extra2 = None
@@ -920,16 +911,16 @@ def run_large(args):
                                                                  w.cutoff, P, T),
                            "evals_per_step": evals, "xsecs_per_s": world * args.steps / (ms * 1e-3),
                            "step": "rox_xsec_batch per chunk (strengths, windows, span ranges, per-line constants, "
-                                   "Voigt accumulate), flags ROX_KAHAN, chunks after the first also ROX_ACCUMULATE",
+                                   "moments, Voigt accumulate), flags ROX_KAHAN, chunks after the first also ROX_ACCUMULATE",
                            "l2": "inputs larger than L2 (line list %.1f GB)" % (line_bytes / 1e9),
                            "sigma_max": sig_max, "parallelism": "replicas" if world > 1 else "single GPU",
                            "launch_config": launch_cfg,
                            "launch_config_source": "autotuner cache (paper_2510_20870_gb300/tuning.json)" if tuned
                                                    else "library default (no cache entry for this GPU)"},
                 "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "config2": extra2, "serving": serving,
-                "gpu_launches": args.steps * 6 * len(starts),
-                "gpu_launches_note": "per chunk: windows, strengths, strength scaling, span ranges, per-line "
-                                     "constants, Voigt kernel (+ memsets)",
+                "gpu_launches": args.steps * 4 * len(starts),
+                "gpu_launches_note": "per chunk: windows and strengths; per-line constants and span ranges; moments; "
+                                     "Voigt kernel (+ memset)",
                 "clocks": csum}
         print(json.dumps(line))
     if dist is not None:
@@ -987,7 +978,8 @@ def config2_summary(args, peaks):
             "value": evals / (ms * 1e-3), "unit": UNIT, "ms_per_step": ms, "steps": steps, "status": rc,
             "kernel_ms": kms, "xsecs_per_s": 1e3 / ms, "summation": "compensated (ROX_KAHAN)",
             "ms_per_step_plain_sum": ms_plain, "launch_config": launch_cfg, "launch_config_tuned": tuned,
-            "roofline_frac": evals * FLOPS_PER_EVAL / (kms * 1e-3) / 1e12 / peaks["formula_tflops"]}
+            "roofline": voigt_roofline(evals, kms, "exomol", torch.cuda.get_device_properties(0).multi_processor_count,
+                                       {}, peaks)}
 
 
 # ------------------------------------------------------------------ other workloads (documentation runs)
@@ -1076,7 +1068,7 @@ def run_batch_config(args):
     del raw, lines, ws, sigma, sort_ws
     torch.cuda.empty_cache()
     peaks = fp32_peaks(0, torch.cuda.get_device_properties(0).multi_processor_count)
-    roof = voigt_roofline(evals, kms, peaks, None, "not captured for this workload", csum)
+    roof = voigt_roofline(evals, kms, None, torch.cuda.get_device_properties(0).multi_processor_count, csum, peaks)
     cpu = None
     if not args.no_cpu_baseline:
         import multiprocessing as mp
@@ -1097,14 +1089,14 @@ def run_batch_config(args):
                       "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
                       "vs_baseline": None, "dtype": "f32", "data": "synthetic",
                       "config": {"workload": "batch: %d lines (ExoMol-style), %d (P,T) points (15 P x 20 T) in one "
-                                             "persistent launch, grid %d points, cutoff %g" % (n, len(pts), grid[2],
+                                             "call, grid %d points, cutoff %g" % (n, len(pts), grid[2],
                                                                                               w.cutoff),
                                  "evals_per_step": evals, "xsecs_per_s": len(pts) / (ms * 1e-3), "status": rc,
                                  "launch_config": launch_cfg, "launch_config_tuned": tuned,
                                  "l2": "inputs larger than L2 (line list %.1f GB, output 3.56 GB)" % (n * 28 / 1e9)},
-                      "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": args.steps * 5,
-                      "gpu_launches_note": "per step: windows, strengths (20 temperatures), strength scaling, span "
-                                           "ranges, Voigt kernel over 300 (P,T) (+ memsets)",
+                      "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": args.steps * (2 + 2 * ((len(pts) + 15) // 16)),
+                      "gpu_launches_note": "per step: windows and strengths (20 temperatures); strength scaling and "
+                                           "span ranges; per 16 (P,T) points moments and Voigt kernel (+ memsets)",
                       "clocks": csum}))
 
 

@@ -123,8 +123,8 @@ const char* rox_last_error(void);
 /* Library version string. */
 const char* rox_version(void);
 
-/* a1 -- line strengths S(T) (cm/molecule) of all lines, FP32 output, FP64 arithmetic
- * for the Boltzmann and stimulated-emission factors and the partition-function ratio.
+/* a1 -- line strengths S(T) (cm/molecule) of all lines, FP32 output: the formula in FP64 rounded
+ * once (in pairs of floats where their error bound leaves one rounding, in FP64 elsewhere).
  * Paper: "Compute line-strengths and -widths".
  * T > 0 (K); Q_T = Q(T) > 0 and Q_ref = Q(296 K) > 0 are computed by the caller (host).
  * S_out [n] float (device). Strengths below the FP32 range round to 0 or a subnormal. */
@@ -133,11 +133,11 @@ int rox_line_strengths(const rox_lines* lines, double T, double Q_T, double Q_re
 
 /* a1 -- the strengths exactly as the cross-section launches compute them (rox_xsec_batch and the
  * calls built on it), in double: the Boltzmann exponent a = -c2 E''(1/T - 1/296) (HITRAN) or
- * -c2 E''/T (ExoMol) in FP64, reduced as a = k ln2 + r (ln 2 in two parts, Cody and Waite);
- * exp(r), the stimulated-emission factor(s) and the prefactor in FP32 on a 2^64 pre-scale, put
- * back by the exact powers 2^-64 and 2^k. Exponents with |a| >= 700 and FP32 products outside
+ * -c2 E''/T (ExoMol) over ln 2 as an FP32 product and its remainder, split into an integer k and a
+ * fraction; 2^fraction, the stimulated-emission factor(s) and the prefactor in FP32 on a 2^64
+ * pre-scale, put back by the exact power 2^(k-64). Exponents with |a| >= 700 and FP32 products outside
  * [2^-100, 2^100] take the full FP64 form of rox_line_strengths. Relative error below 1e-6 (the
- * sum of the FP32 roundings, the expf and expm1f errors included). Paper: "Compute
+ * sum of the FP32 roundings, the exp2f and expm1f errors included). Paper: "Compute
  * line-strengths and -widths". Arguments as rox_line_strengths; S_out [n] double (device). */
 int rox_line_strengths_reduced(const rox_lines* lines, double T, double Q_T, double Q_ref,
                                double* S_out, void* stream);
@@ -176,7 +176,8 @@ int rox_line_windows(const double* nu0_sorted, int64_t n_lines, const rox_grid* 
 int rox_tile_ranges(const int32_t* jlo, const int32_t* jhi, int64_t n_lines, int64_t n_grid,
                     int32_t tile_pts, int64_t* lo_out, int64_t* hi_out, void* stream);
 
-/* FP32 Faddeeva real part used by the Voigt kernel: out[i] = Re w(x[i] + i y[i]), y >= 0.
+/* FP32 Faddeeva real part: out[i] = Re w(x[i] + i y[i]), y >= 0 (the Voigt kernel evaluates forms
+ * of its own, per line).
  * All device arrays of n floats. Max relative error against an FP64 reference about 1.1e-5
  * (values below 1e-15 excepted). */
 int rox_faddeeva_re(const float* x, const float* y, float* out, int64_t n, void* stream);
@@ -193,10 +194,9 @@ int rox_faddeeva_re(const float* x, const float* y, float* out, int64_t n, void*
  * ws        device workspace of rox_xsec_workspace_size(lines->n, grid, n_temps) bytes, where
  *           n_temps is the number of distinct temperatures among T[0..n_pt-1] (S(T) is
  *           computed once per distinct temperature and kept in the workspace as a double).
- * Voigt profile and tile sums in FP32 (compensated across line chunks). S(T): the Boltzmann
- * exponent and its reduction k ln2 + r in FP64, exp(r), the stimulated-emission factor and the
- * prefactor in FP32 (relative error below 1e-6, against 1e-16 for rox_line_strengths).
- * Line-centre offsets: exact index decomposition in FP64. */
+ * Voigt profile and tile sums in FP32 (compensated across line chunks). S(T): the reduced form of
+ * rox_line_strengths_reduced (relative error below 1e-6). Line-centre offsets: exact index
+ * decomposition in 64-bit fixed point. */
 size_t rox_xsec_workspace_size(int64_t n_lines, const rox_grid* grid, int n_temps);
 int rox_xsec_batch(const rox_lines* lines, const rox_grid* grid, int n_pt,
                    const double* P_bar, const double* T, const double* Q_T, double Q_ref,

@@ -16,9 +16,10 @@
 //                      node x_c (step 1/8, nodes to 7.25). This form keeps relative accuracy
 //                      in the Gaussian tail near the real axis, where Re w is tiny next to
 //                      Im w.
-// The two core forms (rox_re_w_core) hold 1.1e-5 out to |z| = 7.1 for y < 0.5 and 2e-6 for
-// 0.5 <= y <= 1.01; the Voigt kernel uses them directly in the |z| < 6.5 zones of lines with the
-// Pade far form (boundary 6.5^2 for y < 1.006).
+// The Voigt kernel's slow zones use other forms of their own (rox_core_*, rox_core_tables.h): per
+// line one rational in U = x^2 / (y^2 + 3/2), N(U)/D(U) of degrees (7, 8) down to (2, 3) as y grows,
+// its coefficients polynomials in y, plus for y < 0.1 the Gaussian part e^{y^2-x^2} cos(2xy) (there
+// the rational gives Re w minus that part, over y).
 // The continued fraction truncations miss the exponentially small e^{-z^2} part of w,
 // which can matter just outside |z| = 6 when y is essentially zero; it is added there.
 //

@@ -5,29 +5,33 @@
 //
 // Persistent kernel; the unit of work is one warp and one span of ROX_SPAN consecutive grid
 // points at one (P,T) point, taken from an atomic counter by the warp itself, so warps never
-// wait for one another. Each lane owns ROX_K points of the span, strided by 32, in registers.
-// The lines that reach the span form a contiguous range of the nu0-sorted list (precomputed
-// per span); they pass through the warp in batches of 32: each lane stages one line's
-// geometry and strength with cp.async one batch ahead, turns it into per-line constants in
-// the warp's shared-memory slots, and then all lanes walk the batch's lines in order. The
-// span is written once at the end, so the summation order is fixed.
+// wait for one another. Each lane owns ROX_K points of the span, strided by 32. The lines that reach
+// the span form a contiguous range of the nu0-sorted list (precomputed per span). The span is
+// written once at the end and every sum has a fixed order, so results are reproducible bit for bit.
 //
-// Work per (line, point) pair, in physical units X = nu_j - nu0, Y = gamma_L: outside a
-// per-line slow zone the far-zone form of rox_faddeeva.cuh (rox_re_w_far: per-line
-// coefficients alpha, beta, kappa of y = gamma_L/gamma_G), scaled by gamma_G, gives
-// S V = (S Y / pi)(t + K) / (t^2 + B) with t = X^2 + A, A = alpha gamma_G^2,
-// B = beta gamma_G^4, K = kappa gamma_G^2, i.e. 4 FMAs and one reciprocal; two lines share
-// one reciprocal (n1/d1 + n2/d2 = (n1 d2 + n2 d1)/(d1 d2)), so a pair costs 12 FP32
-// operations and one MUFU per point, three of them as paired (f32x2) instructions. The slow
-// zone is x^2 + y^2 < r^2(y) for the lines with the per-line Pade form (y < 11.5 except next to
-// its coefficients' pole at y = 0.866; r^2 from 6.5^2 to below 22^2, rox_far_coefs) and < 22^2
-// for the others (2-level continued fraction), at least the precision margin.
-// Lines are evaluated in two passes per batch. Pass 1 applies the far formula to every line at
-// every point of its window, in pairs; a line whose slow zone meets the span has t clamped to
-// the zone boundary, t = max(t, t_z), so inside the zone it adds the far form's (finite) value
-// at the boundary. Pass 2 visits exactly those points (t < t_z, decided on the same rounded t)
-// and adds the full FP32 Faddeeva forms (rox_faddeeva.cuh) minus that boundary value, one form
-// per 32-point sub-span where possible, accumulated in warp-private shared memory.
+// A line's profile outside its slow zone is a rational in X = nu - nu0 (rox_re_w_far: per-line
+// coefficients of y = gamma_L/gamma_G): S V = (P t + Q)/(t^2 + B), t = X^2 + A; two lines share one
+// reciprocal. Far from its poles that function is smooth, so a line is evaluated at every point of
+// a span only where it has to be:
+//  1. Cells (uniform grids). Lines whose window covers the span, at least four times their cell's
+//     half-width plus pole modulus away: k_moments has summed the lines of each cell of 64 grid points
+//     into 14 moments of a multipole expansion, evaluated once per cell at the span's 32 Chebyshev
+//     points.
+//  2. Edge runs. Lines beyond the cells, cut by the window's end inside the span: running sums of 8
+//     moments per line, one evaluation per point (edge_batch).
+//  3. The rest, in batches of 32, a lane setting up a line. Lines smooth on the span are evaluated
+//     at the 32 Chebyshev points (one step a pair in place of ROX_K); lines covering it, with their
+//     poles near, at every point, t clamped to the slow zone's boundary; window-edge lines near
+//     the span under masks; then, inside the slow zones, the Faddeeva forms minus the boundary
+//     value added before (zone_batch, a lane a line; zone_line where zones lie apart).
+// The sums at the Chebyshev points go to the span's points by one interpolation per span (error
+// 1e-7 of a line's value at the distances admitted: smooth_dmin).
+//
+// Every form but the slow zones' works per line and span, not per line and point: on the 1e7-line
+// ExoMol list the kernel took 16.0 ms with each line at each of its 5,001 points, 3.24 ms so. It is bound
+// by instruction issue and, as the code is long, by instruction fetch (4.2 of 9.2 stalled warps
+// per issue before the loops were kept short): a form that saves a few instructions with a second
+// copy of a loop costs more than it gives.
 #include <cuda_fp16.h>
 #include "rox_internal.cuh"
 #include "rox_lines.cuh"
@@ -278,8 +282,8 @@ __device__ __forceinline__ void edge_pair(const PairTab& P, const LineTab& L, in
 
 // Pass 2 for the line in slot s, whose slow zone meets the span: at exactly the points where
 // pass 1 clamped t (t < t_z on the same rounded t, inside the window), the FP32 Faddeeva form of
-// the line's y (rox_faddeeva.cuh) replaces the far form's boundary value cf that pass 1 added there: + S V - cf. In a zone widened to the precision margin the
-// points beyond the form's own zone (X^2 >= zc) take the far form on an offset rounded once.
+// the line's y (rox_faddeeva.cuh) replaces the far form's boundary value cf that pass 1 added there:
+// + S V - cf. In a zone widened to the precision margin the points beyond the form's own zone (X^2 >= zc) take the far form on an offset rounded once.
 // The pass is bound by instruction issue, so a lane takes two points at once in paired FP32
 // instructions (two neighbouring points of the uniform grid: 64 points a warp step, one 8-byte
 // update of the warp's shared-memory row zacc; on nodes two sub-spans), the polynomials' coefficients
@@ -608,8 +612,9 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
 // t = (Y - d)^2 + A, a rational function whose expansion f = sum_l m_l / Y^(l+2) follows from
 // f (Y^4 + d3 Y^3 + d2 Y^2 + d1 Y + d0) = P Y^2 - 2 P d Y + P (d^2 + A) + Q by a four-term
 // recurrence, exact for every order. One warp takes four consecutive cells of one job (one where
-// there are too few to fill the GPU: 9.8 us with four against 5.2 on a list of 1e4 lines), finds the first by a 32-way search of the sorted centres and walks its lines 32 at a time; lanes' sums
-// are added by a fixed tree. Truncated after ROX_MOMENTS terms the expansion errs by
+// there are too few to fill the GPU: 9.8 us with four against 5.2 on a list of 1e4 lines),
+// finds the first by a 32-way search of the sorted centres and walks its lines 32 at a time; the lanes'
+// sums are added by a fixed tree. Truncated after ROX_MOMENTS terms the expansion errs by
 // (r^14)(15 - 14 r) of a line's value, r = (half-width + pole modulus)/|Y|: k_voigt takes a cell only
 // where r <= 1/4 (5e-8).
 __device__ __forceinline__ float cell_k0(const RoxListDev& L, long long pos) {
@@ -741,7 +746,8 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
 // NU: the lists are on user-provided nodes (node offsets in dynamic shared memory, one
 // ROX_SPAN row of float2 per warp). X: ROX_VX_INDEX (each list is a subset of the sorted lines,
 // given by RoxListDev::idx, e.g. the kept lines of a main-contributor selection; span ranges
-// then count positions in that index) and ROX_VX_BROAD (widths from the broadening pass). Each
+// then count positions in that index), ROX_VX_BROAD (widths from the broadening pass) and
+// ROX_VX_PRE (per-line constants from the preparation kernel). Each
 // extra is compiled only into the instantiations that use it: in this kernel even a few added
 // instructions per line batch cost several percent of the plain launch.
 template <bool NU, int X, int W>
@@ -1026,7 +1032,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
           LineK kc;
           float dmin;
           if constexpr (PRE) {
-            // uniform grid, constants from k_line_params
+            // uniform grid, constants from k_prep_scaled
             const float4 r0 = rec_st[lane][0], r1 = rec_st[lane][1], r2 = rec_st[lane][2];
             kc.A = r0.x;
             kc.B = r0.y;
@@ -1291,8 +1297,8 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   if (lane == 0 && evals) atomicAdd(&A.hdr->evals_total, evals);
 }
 
-// Probe of the attainable rate of pass 1's inner loop: cover_pair for clean pairs (the code
-// k_voigt runs for most pairs), alone, with W warps per CTA as k_voigt's launch, on synthetic
+// Probe of the rate of evaluating lines point by point: cover_pair without the clamp (what k_voigt
+// would run if every line were evaluated at every point), alone, with W warps per CTA as k_voigt's launch, on synthetic
 // far-wing constants held in each warp's pair table (offsets of 3-8 cm^-1, so no clamp or mask
 // applies). Each warp walks its 16 pairs `reps` times; no line set-up, staging, edges or slow
 // zones. Not part of the cross-section method.
