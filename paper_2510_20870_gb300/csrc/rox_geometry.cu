@@ -317,7 +317,7 @@ cudaError_t rox_launch_tile_ranges_idx(const float4* geo, const int32_t* idx, co
 }
 
 size_t rox_sort_ws_bytes(long long n) {
-  return rox_align256(cub_temp_bytes(n)) + rox_align256((size_t)n * 8) + 2 * rox_align256((size_t)n * 4) + 256;
+  return rox_align256(cub_temp_bytes(n)) + 2 * rox_align256((size_t)n * 4) + 256;
 }
 
 cudaError_t rox_launch_sort(const rox_lines* in, const rox_lines_buf* out, int64_t* perm_out, void* ws,
@@ -326,16 +326,15 @@ cudaError_t rox_launch_sort(const rox_lines* in, const rox_lines_buf* out, int64
   char* p = (char*)ws;
   size_t tb = cub_temp_bytes(n);
   void* temp = p; p += rox_align256(tb);
-  unsigned long long* keys_out = (unsigned long long*)p; p += rox_align256((size_t)n * 8);
   int32_t* idx_in = (int32_t*)p; p += rox_align256((size_t)n * 4);
   int32_t* idx_out = (int32_t*)p;
   k_iota<<<grid_for(n), 256, 0, s>>>(idx_in, n);
-  // positive doubles order like their bit patterns; bit 63 (sign) is zero for nu0 > 0
-  cudaError_t e = cub::DeviceRadixSort::SortPairs(temp, tb, (const unsigned long long*)in->nu0, keys_out,
+  // positive doubles order like their bit patterns; bit 63 (sign) is zero for nu0 > 0. The sorted keys are
+  // the sorted centres: they go straight to the output (their gather took 0.079 ms of 1.60 for 1e7 lines)
+  cudaError_t e = cub::DeviceRadixSort::SortPairs(temp, tb, (const unsigned long long*)in->nu0, (unsigned long long*)out->nu0,
                                                   idx_in, idx_out, (int64_t)n, 0, 63, s);
   if (e != cudaSuccess) return e;
   int gb = grid_for(n);
-  k_gather<double><<<gb, 256, 0, s>>>(in->nu0, idx_out, out->nu0, n);
   k_gather<float><<<gb, 256, 0, s>>>(in->s_or_a, idx_out, out->s_or_a, n);
   if (in->convention == ROX_EXOMOL) k_gather<float><<<gb, 256, 0, s>>>(in->g_up, idx_out, out->g_up, n);
   k_gather<float><<<gb, 256, 0, s>>>(in->e_lower, idx_out, out->e_lower, n);
