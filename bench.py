@@ -38,8 +38,8 @@ import rox_synth as rs  # noqa: E402
 # evaluation: ncu counters of one launch (profiles/k_voigt_counters.md). An evaluation is the definition's
 # unit of work; the kernel forms most of them from per-cell moments and interpolation, so flops per
 # evaluation mean nothing and the kernel is measured against the warp schedulers' issue rate, its bound.
-VOIGT_INST = {"exomol": None, "large": None}
-VOIGT_DRAM = {"exomol": None, "large": None}
+VOIGT_INST = {"exomol": 2.3804e9 / 4.998e10, "large": 2.5837e10 / 1.98948e12}
+VOIGT_DRAM = {"exomol": 1.573e9 / 4.998e10}
 # DRAM bytes of one k_cia_grid launch on the CIA workload (ncu dram__bytes_read + write,
 # profiles/k_cia_grid_40T_2970001pts.md; part of the 950 MB output is still in L2 at the end)
 CIA_TRAFFIC_BYTES = 8.955e8
