@@ -64,8 +64,10 @@ extern "C" {
 
 /* flags of rox_xsec_batch (and of the rox_job of rox_xsec_jobs) */
 #define ROX_ACCUMULATE 1u /* add into sigma_out instead of overwriting it (chunked line lists) */
-#define ROX_KAHAN 2u      /* compensated (Kahan) summation of the FP32 partial sums of each span part and of
-                             the parts; without it they are added plainly (rox_xsec always sets it) */
+#define ROX_KAHAN 2u      /* compensated (Kahan) summation of the FP32 partial sums (at most 128 lines) of
+                             each span part and of the parts; without it they are added plainly. The sums
+                             of a cell's lines, of a span's cells and of its window edges are always
+                             compensated. rox_xsec always sets the flag */
 
 /* limits */
 #define ROX_MAX_PT 512            /* (P,T) points per rox_xsec_batch call */

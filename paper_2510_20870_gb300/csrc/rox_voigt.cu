@@ -524,7 +524,10 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
 // count points from the side the lines come from: key = Bw - jhi or jlo - Aw, non-decreasing.
 // Centre distances are one cutoff give or take the span's half-width; with (half-width + pole
 // modulus) / (cutoff - half-width) at most ROX_EDGE_R, eight terms err by 9 r^8 = 1e-7.
+// The sums carried from batch to batch are compensated: a part may have 1e5 and more lines of a side, and
+// 3e5 lines of 1e-9 beside one of 1 were dropped whole by a plain sum (2.6e-4 of the value).
 #define ROX_EDGE_R 0.1f
+#define ROX_CARRY (2 * ROX_EDGE_TERMS)   // floats of a side's running sums and their compensations
 // points [k0, k1) of one side: their line's sum from the records rec[0 .. n_rec - 1] (n_rec 33, or 1 to take rec[0])
 template <bool NU>
 __device__ __forceinline__ void edge_points(const EdgeRec* rec, int n_rec, bool left, int k0, int k1, int lane,
@@ -566,21 +569,6 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
   for (int l = 4; l < ROX_EDGE_TERMS; l++) m[l] = fmaf(d3, m[l - 1], fmaf(d2, m[l - 2], fmaf(d1, m[l - 3], d0 * m[l - 4])));
   int kk = mine ? key : -1;
   __syncwarp();                      // the tables of the batch before are no longer read
-  {
-    const float4 ca = reinterpret_cast<const float4*>(carry)[0], cb = reinterpret_cast<const float4*>(carry)[1];
-    if (lane == 0) {
-      reinterpret_cast<float4*>(rec[0].m)[0] = ca;
-      reinterpret_cast<float4*>(rec[0].m)[1] = cb;
-      m[0] += ca.x;
-      m[1] += ca.y;
-      m[2] += ca.z;
-      m[3] += ca.w;
-      m[4] += cb.x;
-      m[5] += cb.y;
-      m[6] += cb.z;
-      m[7] += cb.w;
-    }
-  }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int ko = __shfl_up_sync(0xffffffffu, kk, o);
@@ -591,16 +579,26 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
       if (lane >= o) m[l] += t;
     }
   }
-  const float4 ma = make_float4(m[0], m[1], m[2], m[3]), mb = make_float4(m[4], m[5], m[6], m[7]);
-  float4* r = reinterpret_cast<float4*>(rec[lane + 1].m);
-  r[0] = ma;
-  r[1] = mb;
-  rec[lane + 1].key = kk;
-  if (lane == 31) {
-    reinterpret_cast<float4*>(carry)[0] = ma;
-    reinterpret_cast<float4*>(carry)[1] = mb;
+  const float4 ca = reinterpret_cast<const float4*>(carry)[0], cb = reinterpret_cast<const float4*>(carry)[1];
+  const float c[ROX_EDGE_TERMS] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+  if (lane == 0) {
+    reinterpret_cast<float4*>(rec[0].m)[0] = ca;
+    reinterpret_cast<float4*>(rec[0].m)[1] = cb;
   }
+  float4* r = reinterpret_cast<float4*>(rec[lane + 1].m);
+  r[0] = make_float4(c[0] + m[0], c[1] + m[1], c[2] + m[2], c[3] + m[3]);
+  r[1] = make_float4(c[4] + m[4], c[5] + m[5], c[6] + m[6], c[7] + m[7]);
+  rec[lane + 1].key = kk;
   __syncwarp();
+  if (lane == 31) {                  // the batch's sum into the carried one, read by all lanes above
+#pragma unroll
+    for (int l = 0; l < ROX_EDGE_TERMS; l++) {
+      float v = c[l], e = carry[ROX_EDGE_TERMS + l];
+      sum_add(v, e, m[l], 1.0f);
+      carry[l] = v;
+      carry[ROX_EDGE_TERMS + l] = e;
+    }
+  }
   const int klast = min(__shfl_sync(0xffffffffu, kk, 31), ROX_SPAN);
   edge_points<NU>(rec, 33, left, kcur, klast, lane, centre, inv_cut, dnu_f, Drow, zacc);
   kcur = max(kcur, klast);
@@ -614,9 +612,11 @@ __device__ __forceinline__ void edge_batch(EdgeRec* rec, float* carry, bool left
 // recurrence, exact for every order. One warp takes four consecutive cells of one job (one where
 // there are too few to fill the GPU: 9.8 us with four against 5.2 on a list of 1e4 lines),
 // finds the first by a 32-way search of the sorted centres and walks its lines 32 at a time; the lanes'
-// sums are added by a fixed tree. Truncated after ROX_MOMENTS terms the expansion errs by
-// (r^14)(15 - 14 r) of a line's value, r = (half-width + pole modulus)/|Y|: k_voigt takes a cell only
-// where r <= 1/4 (5e-8).
+// sums are added by a fixed tree, every ROX_CELL_FOLD rounds of 32 lines into a compensated total (a cell
+// of 2.4e5 lines, one of them 4e7 times the others', was 1.7e-4 off with one plain sum per lane).
+// Truncated after ROX_MOMENTS terms the expansion errs by (r^14)(15 - 14 r) of a line's value,
+// r = (half-width + pole modulus)/|Y|: k_voigt takes a cell only where r <= 1/4 (5e-8).
+#define ROX_CELL_FOLD 16
 __device__ __forceinline__ float cell_k0(const RoxListDev& L, long long pos) {
   return L.geo[L.idx ? (long long)L.idx[pos] : pos].x;
 }
@@ -662,6 +662,8 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
       if (lane == 0) A.cstart[J.mom_off + s] = (int32_t)lo;
       if (s == J.n_cells) break;               // the end of the last cell
       float M[ROX_MOMENTS], pm = 0.f, zm = 0.f;
+      float sum = 0.f, cmp = 0.f;              // lane l: moment l of the rounds folded so far
+      int rounds = 0;
 #pragma unroll
       for (int l = 0; l < ROX_MOMENTS; l++) M[l] = 0.f;
       for (;;) {
@@ -722,14 +724,18 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
           }
         }
         lo += nb;
+        if (nb == 32 && ++rounds < ROX_CELL_FOLD) continue;
+        rounds = 0;
+        float v = 0.f;
+#pragma unroll
+        for (int l = 0; l < ROX_MOMENTS; l++) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) M[l] += __shfl_xor_sync(0xffffffffu, M[l], o);
+          v = lane == l ? M[l] : v;
+          M[l] = 0.f;
+        }
+        sum_add(sum, cmp, v, 1.0f);
         if (nb < 32) break;
-      }
-      float v = 0.f;
-#pragma unroll
-      for (int l = 0; l < ROX_MOMENTS; l++) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) M[l] += __shfl_xor_sync(0xffffffffu, M[l], o);
-        v = lane == l ? M[l] : v;
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -737,7 +743,7 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
         zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
       }
       if (!(pm <= 64.0f * half)) pm = 1e30f;   // powers of the poles beyond FP32's range: not to be used
-      v = lane == ROX_MOMENTS ? pm : (lane == ROX_MOMENTS + 1 ? zm : v);
+      const float v = lane == ROX_MOMENTS ? pm : (lane == ROX_MOMENTS + 1 ? zm : sum);
       if (lane < 16) reinterpret_cast<float*>(A.mom + 4 * (size_t)(J.mom_off + s))[lane] = v;
     }
   }
@@ -759,7 +765,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   __shared__ float4 s_geo[W][32];
   __shared__ float s_S[PRE ? 1 : W][32];
   __shared__ __align__(16) unsigned char s_tab[W][sizeof(BatchTab)];
-  __shared__ __align__(16) float s_carry[W][2][12];   // moments of the edge lines so far, per side
+  __shared__ __align__(16) float s_carry[W][2][ROX_CARRY];   // moments of the edge lines so far, per side
   __shared__ __align__(8) float s_zacc[W][ROX_SPAN];
   __shared__ float s_tot[W][ROX_SPAN];    // the span's sum over its parts
   __shared__ float s_part[W][3][ROX_SPAN];  // a part's sum and its compensation; the compensation of s_tot
@@ -929,7 +935,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
       // Chebyshev point in nsum, ncmp
       int ekL = 0, ekR = 0;             // edge lines: first point without its final sum, per side
       bool edgeL = false, edgeR = false;
-      if (lane < 24) carry[lane] = 0.f;
+      carry[lane] = 0.f;                // both sides' 2 x ROX_CARRY floats
       float acc[ROX_K], nacc = 0.f, nsum = 0.f, ncmp = 0.f;
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
@@ -980,7 +986,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
             if (mine && ov > 0) evals += (unsigned)ov;
             const int key = left ? (jhi < Bg ? Bw - jhi : 0) : max(jlo - Aw, 0);
             const float v = -fmaf((float)Aw - g.x, dnu_f, -g.y);
-            edge_batch<NU>(BT.scan, carry + 12 * side, left, mine, key, (v - centre) * inv_cut, k, kcur, lane, centre, inv_cut,
+            edge_batch<NU>(BT.scan, carry + ROX_CARRY * side, left, mine, key, (v - centre) * inv_cut, k, kcur, lane, centre, inv_cut,
                            dnu_f, Drow, zacc);
           }
           if (left) ekL = kcur; else ekR = kcur;
@@ -1134,7 +1140,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
             }
             if (__any_sync(0xffffffffu, mR)) {
               edgeR = true;
-              edge_batch<NU>(BT.scan, carry + 12, false, mR, jlo - Aw, dR * inv_cut, kk, ekR, lane, cR, inv_cut, dnu_f, Drow, zacc);
+              edge_batch<NU>(BT.scan, carry + ROX_CARRY, false, mR, jlo - Aw, dR * inv_cut, kk, ekR, lane, cR, inv_cut, dnu_f, Drow, zacc);
             }
             scanned = mL || mR;
           }
@@ -1192,16 +1198,17 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         for (unsigned z = zslots; z; z &= z - 1)
           zone_line<NU>(PT, LT, __ffs(z) - 1, Aw, lane, dnu_f, core_r, D, cbuf, zacc);
         __syncwarp();
-        // the partial sums into the part's total every 4 batches: compensated (Kahan) with
-        // ROX_KAHAN, else plainly (kw = 0: the correction term stays 0)
+        // the partial sums (acc, and zacc's masked pairs and zones) into the part's total every 4
+        // batches: compensated (Kahan) with ROX_KAHAN, else plainly (kw = 0: the correction term stays 0)
         if ((nb & 3) == 3 || b0 + 32 >= mhi) {
 #pragma unroll
           for (int m = 0; m < ROX_K; m++) {
             float v = part_tot[32 * m], c = part_cmp[32 * m];
-            sum_add(v, c, acc[m], kw);
+            sum_add(v, c, acc[m] + zacc[32 * m + lane], kw);
             part_tot[32 * m] = v;
             part_cmp[32 * m] = c;
             acc[m] = 0.f;
+            zacc[32 * m + lane] = 0.f;
           }
           sum_add(nsum, ncmp, nacc, kw);
           nacc = 0.f;
@@ -1212,11 +1219,13 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
 #pragma unroll 1
       for (int side = 0; side < 2; side++)
         if (side ? edgeR : edgeL)
-          edge_points<NU>(reinterpret_cast<const EdgeRec*>(carry + 12 * side), 1, side == 0, side ? ekR : ekL, ROX_SPAN, lane,
+          edge_points<NU>(reinterpret_cast<const EdgeRec*>(carry + ROX_CARRY * side), 1, side == 0, side ? ekR : ekL, ROX_SPAN, lane,
                           side ? half + Lst.cutoff_f : half - Lst.cutoff_f, inv_cut, dnu_f, Drow, zacc);
       __syncwarp();
-      // this part's share of the far cells, at this lane's Chebyshev point
-      for (int c = n_far * p / np; c < n_far * (p + 1) / np; c++) {
+      // this part's share of the far cells, at this lane's Chebyshev point, 16 of them to a compensated
+      // addition (4e3 cells of 3e-8 each beside one of 1 lost 1.1e-4 in a plain sum)
+      float ncell = 0.f;
+      for (int c = n_far * p / np, c1 = n_far * (p + 1) / np; c < c1; c++) {
         const int cell = c < cl1 - cl0 ? cl0 + c : cr0 + (c - (cl1 - cl0));
         const float4* mo = A.mom + 4 * (size_t)(J.mom_off + cell - J.c_first);
         const float4 v0 = mo[0], v1 = mo[1], v2 = mo[2], v3 = mo[3];
@@ -1226,9 +1235,14 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         f = fmaf(z, fmaf(z, fmaf(z, fmaf(z, f, v2.w), v2.z), v2.y), v2.x);
         f = fmaf(z, fmaf(z, fmaf(z, fmaf(z, f, v1.w), v1.z), v1.y), v1.x);
         f = fmaf(z, fmaf(z, fmaf(z, fmaf(z, f, v0.w), v0.z), v0.y), v0.x);
-        nsum = fmaf(z * z, f, nsum);
+        ncell = fmaf(z * z, f, ncell);
+        if ((c & 15) == 15 || c + 1 == c1) {
+          sum_add(nsum, ncmp, ncell, 1.0f);
+          ncell = 0.f;
+        }
       }
-      // fold in the pass-2 (near-centre) sums
+      nsum -= ncmp;
+      // fold in what the last batches and the edges left in zacc
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
         part_tot[32 * m] += zacc[32 * m + lane] - part_cmp[32 * m];
