@@ -387,18 +387,32 @@ long long job_cells(RoxJobDev* J, int32_t c_steps) {
 }
 
 // Parts of a job's spans (see ROX_PARTS): from the job's lines and spans alone, so that its result does
-// not depend on what it is launched with.
+// not depend on what it is launched with. Twice what an average span has use for; but on few spans
+// the lines may be gathered in some of them, which an average does not see, so that a short grid may
+// take 10, 8 or 4 all the same (3,000 lines on 2 spans at a reach of 100 cm^-1: 0.59 ms in 3 parts a span,
+// 0.22 in 10; in a band of 1,172 spans 0.146 and 0.075 ms with 1 and 4). Many more would use up the part
+// slots in calls of many points (200 points of 2 spans: 0.67 ms with 3 parts, 3.0 with 94). Where the
+// average is below half a batch the parts are of four batches, as lists spread out would take more
+// (3,000 lines over 1,172 spans: 55 us so, 66 with a part per batch).
 void set_parts(RoxJobDev* J, int32_t c_steps) {
-  J->part_shift = rox_part_shift(J->n_spans);
-  J->max_parts = (int32_t)rox_parts_cap(J->n_spans);
-  if (c_steps <= 0) return;      // nodes: a span's share of the lines is not known beforehand
-  // lines that an average span visits one by one: those within about 700 points where cells take the
-  // rest, else all within the cutoff
-  const double pts = (double)J->n_spans * ROX_SPAN + 2.0 * c_steps, reach = 2.0 * c_steps + ROX_SPAN;
-  const double lines = (double)(J->l1 - J->l0) * (c_steps >= 2 * ROX_SPAN && reach > 1400.0 ? 1400.0 : reach) / pts;
-  const double parts = std::ceil(2.0 * lines / 32.0) / (1 << J->part_shift);
-  const double cap = (double)rox_parts_cap(J->n_spans);
-  J->max_parts = (int32_t)(parts >= cap ? cap : (parts < 1.0 ? 1.0 : parts));
+  J->part_shift = J->n_spans >= 8192 ? 4 : (J->n_spans >= 2048 ? 2 : 0);
+  const double cap = (double)rox_parts_cap(J->n_spans), n_lines = (double)(J->l1 - J->l0);
+  double parts = cap;
+  if (c_steps > 0) {      // on nodes a span's share of the lines is not known beforehand
+    // lines that an average span visits one by one: those within about 700 points where cells take the
+    // rest, else all within the cutoff
+    const double pts = (double)J->n_spans * ROX_SPAN + 2.0 * c_steps, reach = 2.0 * c_steps + ROX_SPAN;
+    const double lines = n_lines * (c_steps >= 2 * ROX_SPAN && reach > 1400.0 ? 1400.0 : reach) / pts;
+    parts = std::ceil(2.0 * lines / 32.0);
+    if (J->n_spans >= 2048) {
+      parts /= 1 << J->part_shift;
+    } else {
+      if (parts < 2.0) J->part_shift = 2;
+      parts = std::max(parts, J->n_spans <= 16 ? 10.0 : (J->n_spans <= 128 ? 8.0 : 4.0));
+    }
+    parts = std::min(parts, std::floor((n_lines + 31.0) / 32.0 / (1 << J->part_shift)));   // no span has more
+  }
+  J->max_parts = (int32_t)std::max(1.0, std::min(parts, cap));
 }
 
 // Voigt launches over the jobs, at most ROX_MAX_JOBS per launch; the work counter is reset

@@ -84,8 +84,9 @@ struct RoxListDev {
 #define ROX_CELL_LOG2 6
 #define ROX_CELL (1 << ROX_CELL_LOG2)
 #define ROX_MOMENTS 14
-#define ROX_CELL_LINES 2           // lines a cell on average from which a span takes its cells: reading a cell
-                                   // takes 25 instructions, a line that is smooth on the span about 20
+#define ROX_CELL_LINES 2           // lines a cell (of those within reach, at most the job's) from which a span
+                                   // takes its cells: reading a cell takes 25 instructions, a line that
+                                   // is smooth on the span about 20
 #define ROX_CELL_EXT 512           // cells kept on each side of a job's spans (further lines: one by one)
 #define ROX_MOM_JOBS 16            // jobs whose cells the workspace of a cross-section call holds at a time
 #define ROX_CELL_BYTES 68          // 16 floats and the cell's first line (int32)
@@ -146,8 +147,8 @@ struct RoxJobDev {
 // zero, and the part sums are added in part order. How many is fixed by the job and the span: a job of
 // many spans (three rounds of the GPU's warps or more) fills it with whole items and takes a part per 16
 // batches (a part's fixed work, some 400 instructions and the wait for its first batch, is not worth
-// less), a shorter one a part per 4 or per batch, at most about twice what its spans have on average (a
-// split item has a queue entry per possible part). Jobs of few spans may take more parts than 16, so
+// less), a shorter one a part per 1 to 4 batches, in many spans at most about twice what they have on
+// average (a split item has a queue entry per possible part; set_parts in rox_api.cu). Jobs of few spans may take more parts than 16, so
 // that a narrow window on a dense list still fills the GPU (12 spans of 4e6 lines: 192 warps with 16
 // parts, 1,536 with 128). A work item is normally a whole span; the
 // last items of a launch are split into their parts, taken by different warps: each part stores
@@ -163,7 +164,6 @@ static inline long long rox_parts_cap(long long n_spans) {
   const long long c = n_spans > 0 ? ROX_JOB_PART_SLOTS / n_spans : ROX_PARTS_MAX;
   return c > ROX_PARTS_MAX ? ROX_PARTS_MAX : (c < ROX_PARTS ? ROX_PARTS : c);
 }
-static inline int32_t rox_part_shift(long long n_spans) { return n_spans >= 8192 ? 4 : (n_spans >= 2048 ? 2 : 0); }
 #define ROX_TAIL_ITEMS_MAX 8192
 // A part's sum: its ROX_SPAN points, then its values at the span's ROX_NODES Chebyshev points
 // (the lines that are smooth on the span, rox_voigt.cu)

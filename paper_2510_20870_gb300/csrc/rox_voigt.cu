@@ -852,6 +852,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     const int whi = (int)min(J.first + J.n - 1, (long long)Bw);
     const double smax = __longlong_as_double((long long)*J.smax_bits);
     const int e = smax > 0.0 ? ilogb(smax) : 0;     // S32 holds S * 2^-e (FP32)
+    if (part > 0 && part >= (max(hi - lo, 0) + 31) >> (5 + J.part_shift)) continue;   // more parts than batches
     const float* S_row = J.S32 - J.l0;              // indexed by line number
     const float4* rec = reinterpret_cast<const float4*>(J.S32);   // PRE: the job's constants of every line
 
@@ -861,7 +862,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     int cl0 = 0, cl1 = 0, cr0 = 0, cr1 = 0;
     bool runL = false, runR = false;   // the lines beyond the cells on that side run through the edge scan
     int xa = lo, xb = lo, xc = hi, xd = hi;
-    if (!NU && J.n_cells > 0 && hi - lo >= ROX_CELL_LINES * ((2 * Lst.c_steps + ROX_SPAN) >> ROX_CELL_LOG2)) {
+    if (!NU && J.n_cells > 0 && hi - lo >= ROX_CELL_LINES * min((2 * Lst.c_steps + ROX_SPAN) >> ROX_CELL_LOG2, J.n_cells)) {
       const int c_end = J.c_first + J.n_cells;
       cl0 = max((Bw - Lst.c_steps + ROX_CELL - 1) >> ROX_CELL_LOG2, J.c_first);
       cr1 = min((Aw + Lst.c_steps) >> ROX_CELL_LOG2, c_end);
