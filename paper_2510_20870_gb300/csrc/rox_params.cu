@@ -6,6 +6,7 @@
 // cross-section launches a reduced one (line_strength_fast) that keeps only the Boltzmann
 // exponent and its reduction in FP64. This GPU's FP64 rate, not the bytes, bounds these
 // kernels.
+#include <algorithm>
 #include <cuda_fp16.h>
 #include "rox_internal.cuh"
 #include "rox_strength.cuh"
@@ -260,16 +261,15 @@ __global__ void k_bin_candidates(const int32_t* __restrict__ bin, const double* 
 __global__ void k_bin_max_fix(const rox_lines L, const __grid_constant__ TempSet ts, const int32_t* __restrict__ bin,
                               double* S_T, long long n_bins, const int32_t* __restrict__ list,
                               const long long* __restrict__ count, unsigned long long* binmax_exact) {
-  long long stride = (long long)gridDim.x * blockDim.x;
-  for (int t = 0; t < ts.n; t++) {
-    const long long m = count[t];
-    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += stride) {
-      const long long i = list[(long long)t * L.n + j];
-      const double g = (L.convention == ROX_EXOMOL) ? (double)L.g_up[i] : 1.0;
-      const double sx = line_strength(ts.k[t], L.nu0[i], (double)L.s_or_a[i], g, (double)L.e_lower[i]);
-      S_T[(long long)t * L.n + i] = sx;
-      atomicMax(&binmax_exact[(long long)t * n_bins + bin[i]], (unsigned long long)__double_as_longlong(sx));
-    }
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const int t = blockIdx.y;
+  const long long m = count[t];
+  for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += stride) {
+    const long long i = list[(long long)t * L.n + j];
+    const double g = (L.convention == ROX_EXOMOL) ? (double)L.g_up[i] : 1.0;
+    const double sx = line_strength(ts.k[t], L.nu0[i], (double)L.s_or_a[i], g, (double)L.e_lower[i]);
+    S_T[(long long)t * L.n + i] = sx;
+    atomicMax(&binmax_exact[(long long)t * n_bins + bin[i]], (unsigned long long)__double_as_longlong(sx));
   }
 }
 
@@ -448,7 +448,11 @@ cudaError_t rox_launch_select_reduced(const rox_lines* L, int n_temps, const dou
   k_bin_max<<<grid_for((n + ROX_BIN_RUN - 1) / ROX_BIN_RUN), 256, 0, s>>>(bin, S_T, n, n_temps, n_bins, binmax_fast);
   if ((e = cudaMemsetAsync(count, 0, (size_t)n_temps * 8, s)) != cudaSuccess) return e;
   k_bin_candidates<<<grid_for(n), 256, 0, s>>>(bin, S_T, n, n_temps, n_bins, binmax_fast, list, count);
-  k_bin_max_fix<<<grid_for((n + 31) / 32), 256, 0, s>>>(*L, ts, bin, S_T, n_bins, list, count, binmax_exact);
+  // a thread per four lines, two warps a block: a short list's candidates (about two in a bin) spread over
+  // the SMs' FP64 units, each some 2 us a strength (3e4 lines, three temperatures: 39.9 us with a thread
+  // per 32 lines and the temperatures in turn)
+  const dim3 fix((unsigned)std::max(1LL, std::min(152LL * 16, (n / 4 + 63) / 64)), (unsigned)n_temps);
+  k_bin_max_fix<<<fix, 64, 0, s>>>(*L, ts, bin, S_T, n_bins, list, count, binmax_exact);
   double* thr = reinterpret_cast<double*>(binmax_fast);
   k_bin_thresholds<<<grid_for(n_temps * n_bins), 256, 0, s>>>(binmax_exact, (long long)n_temps * n_bins, rel, thr);
   k_select_scale<<<grid_for(n), 256, 0, s>>>(*L, ts, S_T, smax_bits, bin, thr, n_bins, S32);
