@@ -528,6 +528,11 @@ __device__ __forceinline__ void zone_batch(bool on, int q0, int q1, int qa, int 
 // 3e5 lines of 1e-9 beside one of 1 were dropped whole by a plain sum (2.6e-4 of the value).
 #define ROX_EDGE_R 0.1f
 #define ROX_CARRY (2 * ROX_EDGE_TERMS)   // floats of a side's running sums and their compensations
+// Lines of a side in a general batch from which it is scanned: a scan takes some 250 instructions whatever
+// it holds, a masked pair about 100. At cutoffs of two to four spans most batches hold a few such lines
+// only (30,000 lines, 300,001 points, 10 points (P,T), cutoff 5 cm^-1: 0.470 ms with every batch scanned,
+// 0.43 from 16 lines on); with never a scan, long lists lose (the 3e6-line fixed-resolution grid 4.62 -> 5.1 ms).
+#define ROX_EDGE_SCAN 16
 // points [k0, k1) of one side: their line's sum from the records rec[0 .. n_rec - 1] (n_rec 33, or 1 to take rec[0])
 template <bool NU>
 __device__ __forceinline__ void edge_points(const EdgeRec* rec, int n_rec, bool left, int k0, int k1, int lane,
@@ -906,8 +911,10 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
       if (part <= 0 && lane == 0) evals += (unsigned long long)((long long)(xb - xa) + (xd - xc)) * (unsigned)(whi - wlo + 1);
     }
     // without cells on the left the list is cut at the span's centre, so that the lines left of it
-    // can run downwards (their window edges then come in order, see edge_batch)
-    if (cl1 <= cl0 && hi > lo) {
+    // can run downwards (their window edges then come in order, see edge_batch); a few batches
+    // seldom hold enough of them for a scan, and are left as they are
+    const bool ordered = cl1 > cl0 || hi - lo > 4 * 32;
+    if (cl1 <= cl0 && ordered) {
       const float mid = NU ? bh + half : (float)(Aw + ROX_SPAN / 2);
       int a = lo, len = hi - lo;
       while (len > 0) {
@@ -1134,7 +1141,9 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
             const float v = NU ? ax + ay : -fmaf(ax, dnu_f, ay);              // the line, from there
             const float bm = fabsf(kk.B) + 1e-30f, r2 = fabsf(kk.A) + bm * rox_rsqrt(bm) + 1e-30f;
             const float dL = v - cL, dR = v - cR, room = ROX_EDGE_R * (Lst.cutoff_f - half) - r2 * rox_rsqrt(r2);
-            const bool mL = eL && fabsf(dL) <= room, mR = eR && fabsf(dR) <= room;
+            bool mL = eL && ordered && fabsf(dL) <= room, mR = eR && fabsf(dR) <= room;
+            mL = __popc(__ballot_sync(0xffffffffu, mL)) >= ROX_EDGE_SCAN && mL;
+            mR = __popc(__ballot_sync(0xffffffffu, mR)) >= ROX_EDGE_SCAN && mR;
             if (__any_sync(0xffffffffu, mL)) {
               edgeL = true;
               edge_batch<NU>(BT.scan, carry, true, mL, Bw - jhi, dL * inv_cut, kk, ekL, lane, cL, inv_cut, dnu_f, Drow, zacc);
