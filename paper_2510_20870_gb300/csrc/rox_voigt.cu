@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
         }
         const int nb = __popc(__ballot_sync(0xffffffffu, in));
         if (in) {
-          float a, b, p, q, hz;
+          float a, b, p, q, tz;
           if constexpr (PRE) {
             const float4* rec = reinterpret_cast<const float4*>(J.S32);
             const float4 r0 = rec[3 * li];
@@ -696,8 +696,7 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
             b = r0.y;
             p = r0.z;
             q = r0.w;
-            const float z2 = fmaxf(rec[3 * li + 1].x - a, 0.f) + 1e-30f;   // t_z = hz^2 + A
-            hz = z2 * rox_rsqrt(z2) * 1.001f;
+            tz = rec[3 * li + 1].x;
           } else {
             float gref, nt;
             load_widths<BRD>(J, L, L.width_f16, li, gref, nt);
@@ -706,8 +705,12 @@ __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ RoxVoig
             b = kc.B;
             p = kc.P;
             q = kc.Q;
-            hz = kc.hz * 1.001f;
+            tz = kc.tz;
           }
+          // the zone's half-width, t_z = hz^2 + A: from what the records hold too, so that a point has the same
+          // cells alone (with records) and in a call of several
+          const float z2 = fmaxf(tz - a, 0.f) + 1e-30f;
+          const float hz = z2 * rox_rsqrt(z2) * 1.001f;
           const float bm = fabsf(b) + 1e-30f;
           const float r2 = fabsf(a) + bm * rox_rsqrt(bm) + 1e-30f;      // |pole|^2 at most
           pm = fmaxf(pm, r2 * rox_rsqrt(r2) * 1.001f);
