@@ -196,6 +196,9 @@ int rox_faddeeva_re(const float* x, const float* y, float* out, int64_t n, void*
  * ws        device workspace of rox_xsec_workspace_size(lines->n, grid, n_temps) bytes, where
  *           n_temps is the number of distinct temperatures among T[0..n_pt-1] (S(T) is
  *           computed once per distinct temperature and kept in the workspace as a double).
+ *           For n_temps = 1 the size includes 48 bytes per line of constants that a call of one
+ *           point computes once; a workspace without them (such as one sized for more
+ *           temperatures) serves as well, with the same result in a little more time.
  * Voigt profile and tile sums in FP32 (compensated across line chunks). S(T): the reduced form of
  * rox_line_strengths_reduced (relative error below 1e-6). Line-centre offsets: exact index
  * decomposition in 64-bit fixed point. */
@@ -296,7 +299,9 @@ int rox_line_select(const rox_lines* lines, const rox_grid* grid, double cutoff,
  * ROX_EGRID. ws: device workspace of rox_xsec_nodes_workspace_size(lines->n, nodes->n,
  * n_temps) bytes (n_temps as for rox_xsec_batch); it includes each node's offset from the
  * first node of its ROX_SPAN-node span, the kernel's exact stand-in for the index
- * decomposition of a uniform grid. */
+ * decomposition of a uniform grid. For up to 4 temperatures, and while they take at most 16 GiB, it also
+ * includes 48 bytes per line and temperature of per-line constants, used where each temperature
+ * has one point; a workspace without them (such as one sized for 5 temperatures) serves as well. */
 size_t rox_xsec_nodes_workspace_size(int64_t n_lines, int64_t n_nodes, int n_temps);
 int rox_xsec_nodes_batch(const rox_lines* lines, const rox_nodes* nodes, int n_pt,
                          const double* P_bar, const double* T, const double* Q_T, double Q_ref,

@@ -185,6 +185,7 @@ struct WsLayout {
   float* broad_N;      //   natural widths
   RoxMoments mom;      // uniform grids: moments of ROX_MOM_JOBS jobs' cells
   float4* rec;         // one temperature (nodes: up to ROX_PRE_POINTS): per line 3 float4 of per-line constants
+  size_t least;        // bytes without rec (the last part), which a call can do without
   size_t bytes;
 };
 
@@ -270,10 +271,12 @@ WsLayout ws_layout(void* ws, long long n_lines, long long n_grid, int n_temps, b
     w.mom = moments_at(base + off, slots);
     off += rox_mom_bytes(slots);
   }
+  w.least = off;
   w.rec = nullptr;
-  if (pre && n_temps <= (nodes ? ROX_PRE_POINTS : 1) && n_bins == 0 && !broad) {
+  const size_t rec_bytes = (size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 3 * sizeof(float4);
+  if (pre && n_temps <= (nodes ? ROX_PRE_POINTS : 1) && (!nodes || rec_bytes <= ROX_PRE_NODES_BYTES) && n_bins == 0 && !broad) {
     w.rec = (float4*)(base + off);
-    off += rox_align256((size_t)n_temps * (size_t)(n_lines > 0 ? n_lines : 1) * 3 * sizeof(float4));
+    off += rox_align256(rec_bytes);
   }
   w.bytes = off;
   return w;
@@ -639,9 +642,9 @@ int xsec_batch_impl(const rox_lines* lines, const rox_grid* grid, const rox_node
   const int n_temps = (int)temps.size();
   if (!ws || ((uintptr_t)ws & 255)) return fail(ROX_EINVAL, "workspace NULL or not 256-byte aligned");
   WsLayout w = ws_layout(ws, lines->n, n_grid, n_temps, on_nodes, n_bins, br != nullptr, tail_max, allow_pre);
-  // one (P,T) point per temperature: the per-line constants once per line
-  const bool pre = w.rec != nullptr && n_pt == n_temps && lines->n > 0;
-  if (ws_bytes < w.bytes) return fail(ROX_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, w.bytes);
+  // one (P,T) point per temperature: the per-line constants once per line, where the workspace has room
+  const bool pre = w.rec != nullptr && ws_bytes >= w.bytes && n_pt == n_temps && lines->n > 0;
+  if (ws_bytes < w.least) return fail(ROX_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, w.least);
 
   cudaStream_t s = (cudaStream_t)stream;
   const rox_launch_config cfg = launch_config();

@@ -115,6 +115,7 @@ struct RoxBroadDev {
 // point (on a uniform grid: one, where most pairs need only the cells' moments). 3e6 lines, 3e6 nodes, two
 // points: constants per span 4.85 ms, kept 4.57 ms.
 #define ROX_PRE_POINTS 4
+#define ROX_PRE_NODES_BYTES ((size_t)16 << 30)   // and up to 6% of the device's memory
 
 struct RoxJobDev {
   // S * 2^-e of lines l0, l0+1, ... at this job's T. In a ROX_VX_PRE launch the job's per-line
