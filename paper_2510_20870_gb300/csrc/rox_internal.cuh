@@ -112,8 +112,9 @@ struct RoxBroadDev {
 #define ROX_VX_BROAD 2    // widths from the broadening pass (RoxListDev::gLT, gN)
 #define ROX_VX_PRE 4      // per-line constants precomputed for each (P,T) point (RoxJobDev::S32)
 // (P,T) points up to which a call on user-provided nodes keeps them, 48 bytes of workspace per line and
-// point (on a uniform grid: one, where most pairs need only the cells' moments). 3e6 lines, 3e6 nodes, two
-// points: constants per span 4.85 ms, kept 4.57 ms.
+// point (on a uniform grid: one, where most pairs need only the cells' moments). 3e6 lines, 3e6 nodes:
+// kept 2.53, 4.61, 6.72, 8.85 ms for one to four points, per span 2.64, 4.86, 7.09, 9.33; 5% also on 1e6 lines,
+// nothing on 3e4 (0.389 and 0.385 ms). The gain does not fall with the points; the workspace sets the limit.
 #define ROX_PRE_POINTS 4
 #define ROX_PRE_NODES_BYTES ((size_t)16 << 30)   // and up to 6% of the device's memory
 
