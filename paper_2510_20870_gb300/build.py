@@ -3,8 +3,10 @@
 `python -m paper_2510_20870_gb300.build` or `build()` compiles every translation unit
 in parallel with nvcc (one -gencode, no cmake) and links them next to this file. The
 FP32 Faddeeva constant tables are regenerated first and must match the committed
-header (the generator uses only exact arithmetic and numpy's FFT).
+header (the generator uses only exact arithmetic and numpy's FFT). The slow zones' tables
+(rox_core_tables.h), whose generator needs mpmath, must name the generator they came from.
 """
+import hashlib
 import os
 import subprocess
 import sys
@@ -28,12 +30,25 @@ def check_tables():
     with open(os.path.join(CSRC, "rox_faddeeva_tables.h")) as f:
         if f.read().strip() != gen.strip():
             raise RuntimeError("rox_faddeeva_tables.h is stale: rerun gen_faddeeva_tables.py")
+    with open(os.path.join(CSRC, "gen_core_tables.py"), "rb") as f:
+        digest = hashlib.sha256(f.read()).hexdigest()
+    with open(os.path.join(CSRC, "rox_core_tables.h")) as f:
+        if "generator: sha256 " + digest not in f.read(400):
+            raise RuntimeError("rox_core_tables.h is stale: rerun gen_core_tables.py")
 
 
 def make_interp_table():
-    """The span interpolation table (rox_interp_table.h), into the build folder."""
-    with open(os.path.join(BUILD, "rox_interp_table.h"), "w") as f:
-        subprocess.run([sys.executable, os.path.join(CSRC, "gen_interp_table.py")], check=True, stdout=f)
+    """The span interpolation table (rox_interp_table.h), into the build folder; put in place when it is
+    complete, so that a failed or concurrent build leaves no partial header."""
+    path = os.path.join(BUILD, "rox_interp_table.h")
+    part = "%s.%d" % (path, os.getpid())
+    try:
+        with open(part, "w") as f:
+            subprocess.run([sys.executable, os.path.join(CSRC, "gen_interp_table.py")], check=True, stdout=f)
+        os.replace(part, path)
+    finally:
+        if os.path.exists(part):
+            os.remove(part)
 
 
 def _run(cmd):

@@ -13,6 +13,8 @@ solutions of a linear system analytic in y they are smooth in y, and each is sto
 polynomial: of degree 7 in t = a log2(y) + b on [-1, 1], for R of degree 3 in y^2.
 Re w = Re(exp(-z^2) erfc(-iz)) in 50 digits (mpmath); scipy's wofz only places the U_j.
 """
+import hashlib
+
 import mpmath as mp
 import numpy as np
 from scipy.special import wofz
@@ -121,7 +123,9 @@ def row_r():
 
 
 def main():
-    o = ["/* Generated by gen_core_tables.py -- do not edit. */", "#pragma once",
+    with open(__file__, "rb") as f:     # checked by the build, which has no mpmath everywhere
+        digest = hashlib.sha256(f.read()).hexdigest()
+    o = ["/* Generated by gen_core_tables.py -- do not edit. */", "/* generator: sha256 %s */" % digest, "#pragma once",
          "#define ROX_CORE_ROWS %d" % len(ROWS), "#define ROX_CORE_DEG %d" % DEG,
          "#define ROX_CORE_KAPPA %.1ff" % KAPPA,
          "/* lower end of each y interval, and a, b of t = a log2(y) + b */",
