@@ -63,3 +63,12 @@ extern "C" void rox_host_strength_df(int hitran, double c2_dT, double q_fac, dou
     certain[i] = ok && rox_df_round(s, e, &rounded[i]);
   }
 }
+
+// the rounding alone: h + l, scaled by 2^e
+extern "C" void rox_host_df_round(const float* h, const float* l, const int32_t* e, float* rounded, uint8_t* certain,
+                                  int64_t n) {
+  for (int64_t i = 0; i < n; i++) {
+    rounded[i] = 0.0f;
+    certain[i] = rox_df_round({h[i], l[i]}, e[i], &rounded[i]);
+  }
+}
