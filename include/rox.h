@@ -437,9 +437,9 @@ int rox_get_launch_config(rox_launch_config* out);
 size_t rox_fp32_probe_out_size(int n_blocks);
 int rox_fp32_probe(int n_blocks, int reps, float* out, size_t out_bytes, double* fma_out, void* stream);
 
-/* Measurement helper: the attainable rate of the Voigt kernel's inner loop. Runs the pass-1
- * pair loop of the cross-section kernel (two lines per reciprocal, far form, no clamp or mask)
- * alone on synthetic far-wing constants, n_blocks blocks of 256 threads (8 warps, as the
+/* Measurement helper: the attainable rate of evaluating lines point by point. Runs the cross-section
+ * kernel's loop for lines that cover a span near it (two lines per reciprocal, far form clamped to the
+ * zone boundary, no mask) alone on synthetic far-wing constants, n_blocks blocks of 256 threads (8 warps, as the
  * kernel's default launch), each warp walking 16 pairs reps times over its span of ROX_SPAN
  * points; no line set-up, staging, window edges or slow zones. out as rox_fp32_probe
  * (rox_fp32_probe_out_size(n_blocks) bytes, device). *evals_out (host) receives the

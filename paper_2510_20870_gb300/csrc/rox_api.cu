@@ -455,7 +455,7 @@ int launch_voigt_jobs(const RoxListDev* lists, int n_lists, const RoxJobDev* job
     // to 30% (20,001 points)
     A.cells_task = slots < 152 * 64 ? 1 : 4;
     // whole items in complete rounds of the launch's warps, then at least one round of items in
-    // parts, so the launch ends in pieces of 1/ROX_PARTS of an item
+    // their parts, so the launch ends in pieces of a part
     const long long warps = (long long)nblocks * cfg.warps_per_cta;
     long long split = items <= warps ? items : items % warps + (long long)cfg.split_rounds * warps;
     if (split > items) split = items;

@@ -170,8 +170,7 @@ __global__ void k_tile_ranges(const int32_t* __restrict__ jlo, const int32_t* __
   }
 }
 
-// same, reading the window bounds out of the packed geometry records
-// k_tile_ranges_geo for a list given as indices into the sorted list (the kept lines of a
+// k_tile_ranges_geo (below) for a list given as indices into the sorted list (the kept lines of a
 // selection, still in nu0 order): line i of the list is geo[idx[i]], and the list length is
 // read on the device (*count, at most n_max).
 __global__ void k_tile_ranges_idx(const float4* __restrict__ geo, const int32_t* __restrict__ idx,
@@ -203,6 +202,7 @@ __global__ void k_kept_flags(const float* __restrict__ S32, long long total, uin
     flags[i] = __float_as_uint(S32[i]) != 0x80000000u;
 }
 
+// k_tile_ranges, reading the window bounds out of the packed geometry records
 __global__ void k_tile_ranges_geo(const float4* __restrict__ geo, long long n_lines, long long n_tiles,
                                   int32_t W, long long* lo_out, long long* hi_out) {
   long long stride = (long long)gridDim.x * blockDim.x;

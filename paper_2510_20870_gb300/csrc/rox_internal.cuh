@@ -16,18 +16,17 @@
 #define ROX_PI 3.14159265358979323846
 
 // Voigt work geometry: a warp owns one span of ROX_SPAN = 32*ROX_K consecutive grid points
-// (each lane ROX_K points strided by 32) and is its own unit of scheduling; CTAs of
-// ROX_WARPS warps only share the Dawson table. Lines reach a warp in batches of 32.
-#define ROX_WARPS 8
-#define ROX_THREADS (ROX_WARPS * 32)
+// (each lane ROX_K points strided by 32) and is its own unit of scheduling; the warps of a CTA
+// share nothing. Lines reach a warp in batches of 32.
 #define ROX_K (ROX_SPAN / 32)           // ROX_SPAN (include/rox.h) = 256 grid points per span
 #define ROX_TILE ROX_SPAN               // grid points per work item (per-item line ranges)
 
 // The far formula (rox_re_w_far in physical units) is used only outside each line's slow
-// zone, x^2 + y^2 >= 6.5^2 or 22^2 depending on the line's y. Its per-point offset is
+// zone, whose boundary |z|^2 goes with the line's y (rox_far_coefs). Its per-point offset is
 // X_m = X_0 + 32 m dnu with X_0 the offset at the thread's first point, so X_m carries a
-// rounding error of 6e-8 (|X_m| + span); the slow zone around each line is therefore at
-// least ROX_FAST_MARGIN * span wide, which keeps that error below 2e-6 relative.
+// rounding error of 6e-8 (|X_m| + span). What that does to the profile goes with the larger of |X|
+// and gamma_L (the poles lie gamma_L off the axis), so the slow zone around each line reaches at least to
+// X^2 + gamma_L^2 = (ROX_FAST_MARGIN * span)^2 (line_consts), which keeps the error below 2e-6 relative.
 #define ROX_FAST_MARGIN 0.032
 
 // Workspace header at the start of every xsec / prepared-list workspace.

@@ -3,21 +3,16 @@
 // strength and broadening widths of every transition at the user's pressure and
 // temperature. Each thread reads one line's SoA entries (coalesced) and writes its outputs.
 // The strength exists in two forms: the full FP64 one (line_strength), and for the
-// cross-section launches a reduced one (line_strength_fast) that keeps only the Boltzmann
-// exponent and its reduction in FP64. This GPU's FP64 rate, not the bytes, bounds these
-// kernels.
+// cross-section launches a reduced one (line_strength_fast) without FP64 arithmetic, its Boltzmann
+// exponent a pair of floats. This GPU's FP64 rate, not the bytes, bounds the full form.
 #include <algorithm>
 #include <cuda_fp16.h>
 #include "rox_internal.cuh"
+#include "rox_lines.cuh"      // load_width
 #include "rox_strength.cuh"
 #include "rox_strength_df.h"
 
 namespace {
-
-__device__ __forceinline__ float load_width(const void* p, int f16, long long i) {
-  return f16 ? __half2float(reinterpret_cast<const __half*>(p)[i])
-             : reinterpret_cast<const float*>(p)[i];
-}
 
 // S(T) rounded to FP32: by pairs of floats where their rounding is certain (all but one line in a
 // thousand), by the FP64 form otherwise, so the same bits as from the FP64 form alone. That one was
@@ -62,7 +57,7 @@ __global__ void k_widths(rox_lines L, double gG_fac, float l2_ratio, float p_fac
 }
 
 // S(T) for up to ROX_MAX_PT distinct temperatures in one launch, one sweep over the lines
-// per temperature (FAST: the reduced form; either way FP64 issue, not the bytes, sets its
+// per temperature (FAST: the reduced form, bound by its bytes; else FP64 issue sets the
 // cost); the per-temperature maximum (needed to
 // scale S into FP32 range inside the Voigt kernel) is reduced per warp and combined with
 // an atomic max on the (non-negative) double bit pattern, which is order-independent.
@@ -89,11 +84,10 @@ __global__ void k_strengths_multi(rox_lines L, TempSet ts,
 }
 
 // S * 2^-e per temperature, e the exponent of the largest strength at that temperature,
-// so the Voigt kernel works in FP32 well inside its range whatever the line strengths are.
-// S * 2^-e in FP32 (e the exponent of the temperature's largest S). With a selection
-// (bin != NULL): lines outside the bins, or below rel times their bin's largest S at that
-// temperature (the product rounded once in double precision), get -0.0, which the Voigt kernel
-// tells apart from a kept strength that rounds to +0.0 in FP32.
+// so the Voigt kernel works in FP32 well inside its range whatever the line strengths are: lines outside
+// the selection's bins, or below rel times their bin's largest S at that temperature (the product rounded
+// once in double precision), get -0.0, which the Voigt kernel tells apart from a kept strength that rounds
+// to +0.0 in FP32.
 __global__ void k_scale_strengths(const double* __restrict__ S_T, long long n, int n_temps,
                                   const unsigned long long* __restrict__ smax_bits, float* S32,
                                   const int32_t* __restrict__ bin, const unsigned long long* __restrict__ binmax_bits,
@@ -104,21 +98,15 @@ __global__ void k_scale_strengths(const double* __restrict__ S_T, long long n, i
     double sc = ldexp(1.0, smax > 0.0 ? -ilogb(smax) : 0);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
       const double S = S_T[(long long)t * n + i];
-      bool keep = true;
-      if (bin) {
-        const int b = bin[i];
-        keep = b >= 0 &&
-               S >= __dmul_rn(rel, __longlong_as_double((long long)binmax_bits[(long long)t * n_bins + b]));
-      }
+      const int b = bin[i];
+      const bool keep =
+          b >= 0 && S >= __dmul_rn(rel, __longlong_as_double((long long)binmax_bits[(long long)t * n_bins + b]));
       S32[(long long)t * n + i] = keep ? (float)(S * sc) : -0.0f;   // -0: dropped (+0: kept, below FP32)
     }
   }
 }
 
 // ---- a2 broadening descriptions: sum_b vmr_b gamma_b (296/T)^n_b of line i, l2 = log2(296/T)
-__device__ __forceinline__ float broad_col(const void* p, int f16, long long i) {
-  return f16 ? __half2float(reinterpret_cast<const __half*>(p)[i]) : reinterpret_cast<const float*>(p)[i];
-}
 __device__ __forceinline__ float broad_sum(const RoxBroadDev& B, long long i, float l2) {
   long long j = 0;
   if (B.j_lower) {
@@ -132,8 +120,8 @@ __device__ __forceinline__ float broad_sum(const RoxBroadDev& B, long long i, fl
       gb = B.tab_gamma[b][j];
       nb = B.tab_n[b][j];
     } else {
-      gb = broad_col(B.gamma[b], B.f16, i);
-      nb = broad_col(B.n[b], B.f16, i);
+      gb = load_width(B.gamma[b], B.f16, i);
+      nb = load_width(B.n[b], B.f16, i);
     }
     g = fmaf(B.vmr[b] * gb, exp2f(nb * l2), g);
   }

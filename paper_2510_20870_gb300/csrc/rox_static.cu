@@ -23,7 +23,7 @@ int rox_xsec_tail(const rox_lines* lines, const rox_grid* grid, double P_bar, do
                   long long tail_max);
 size_t rox_xsec_workspace_size_tail(int64_t n_lines, const rox_grid* grid, long long tail_max);
 
-// Split work items the static scratch has room for (16 KB each); the launch splits fewer items
+// Split work items the static scratch has room for (16 parts of 1,152 bytes each); the launch splits fewer items
 // than usual, which changes how its warps share the last items, not the result.
 #define ROX_STATIC_TAIL_ITEMS 256
 

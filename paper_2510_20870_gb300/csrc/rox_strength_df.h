@@ -1,5 +1,5 @@
 // The line strength in pairs of floats (an unevaluated sum hi + lo), for results that are rounded to
-// FP32 (rox_line_params). FP64 arithmetic issues at about two operations per clock per SM here and the
+// FP32 (rox_line_strengths). FP64 arithmetic issues at about two operations per clock per SM here and the
 // FP64 form needs some 65 of them per line; FP32 issues at 128. The pair form is good to
 // ROX_DF_ERR; its rounding is taken where it is certain (hi + lo not within ROX_DF_ERR of the middle of
 // two floats), otherwise the caller takes the FP64 form, so the results are those of the FP64 form.

@@ -41,9 +41,8 @@ namespace {
 
 
 // Per-line constants of one (P,T) point for the batch in hand. Each line has a slot; slots are
-// ordered by class -- lines whose window covers the whole span and whose slow zone misses it
-// ("clean") first, then the other covering lines, then the lines cut by a window edge -- and
-// slots 2k, 2k+1 form pair k. The pair tables hold both lines' far-form constants side by side,
+// ordered by class -- lines that are smooth on the span first, then the others whose window covers all
+// of it, then the lines cut by a window edge that are not scanned -- and slots 2k, 2k+1 form pair k. The pair tables hold both lines' far-form constants side by side,
 // so one 16-byte load brings a field of both; the line table holds what window edges and pass 2
 // need per slot. S is scaled by 2^-e (e the exponent of the largest strength at this
 // temperature).
@@ -195,17 +194,17 @@ __device__ __forceinline__ float pos(int m, float X0, float ch, float cl, const 
   }
 }
 
-// Pass 1 for covering pair k: every point of the span (CLAMP unless both lines are clean).
-template <bool NU, bool CLAMP>
+// Pass 1 for covering pair k: every point of the span, t clamped to each line's zone boundary.
+template <bool NU>
 __device__ __forceinline__ void cover_pair(const PairTab& P, int k, float lanef, float dnu_f, const float2* D,
                                            float (&acc)[ROX_K]) {
-  const PairC c = pair_consts<CLAMP>(P, k);
+  const PairC c = pair_consts<true>(P, k);
   float X0, X1;
   pair_x0<NU>(c, lanef, dnu_f, X0, X1);
 #pragma unroll
   for (int m = 0; m < ROX_K; m++)
-    acc[m] = pair_add<CLAMP, false>(pos<NU>(m, X0, c.e0, c.f0, D, dnu_f), pos<NU>(m, X1, c.e1, c.f1, D, dnu_f), c,
-                                    true, true, acc[m]);
+    acc[m] = pair_add<true, false>(pos<NU>(m, X0, c.e0, c.f0, D, dnu_f), pos<NU>(m, X1, c.e1, c.f1, D, dnu_f), c,
+                                   true, true, acc[m]);
 }
 
 // Pass 1 for pair k of lines that are smooth on the span: their sum at this lane's Chebyshev
@@ -1214,7 +1213,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         // reproducible.
         const int ks = nsm >> 1, kz = ncov >> 1, ke = (nslot + 1) >> 1;
         for (int k = 0; k < ks; k++) nacc = smooth_pair<NU>(PT, k, tau, dnu_f, nacc);
-        for (int k = ks; k < kz; k++) cover_pair<NU, true>(PT, k, lanef, dnu_f, D, acc);
+        for (int k = ks; k < kz; k++) cover_pair<NU>(PT, k, lanef, dnu_f, D, acc);
         for (int k = kz; k < ke; k++) edge_pair<NU>(PT, LT, k, Aw, lane, lanef, dnu_f, D, zacc);
         // ---- pass 2 line by line otherwise
         for (unsigned z = zslots; z; z &= z - 1)
@@ -1333,10 +1332,10 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   if (lane == 0 && evals) atomicAdd(&A.hdr->evals_total, evals);
 }
 
-// Probe of the rate of evaluating lines point by point: cover_pair without the clamp (what k_voigt
-// would run if every line were evaluated at every point), alone, with W warps per CTA as k_voigt's launch, on synthetic
-// far-wing constants held in each warp's pair table (offsets of 3-8 cm^-1, so no clamp or mask
-// applies). Each warp walks its 16 pairs `reps` times; no line set-up, staging, edges or slow
+// Probe of the rate of evaluating lines point by point: cover_pair, the loop that k_voigt runs for lines
+// that cover a span and are not smooth on it, alone, with W warps per CTA as k_voigt's launch, on synthetic
+// far-wing constants held in each warp's pair table (offsets of 3-8 cm^-1, so no clamp applies).
+// Each warp walks its 16 pairs `reps` times; no line set-up, staging, edges or slow
 // zones. Not part of the cross-section method.
 template <int W>
 __global__ void __launch_bounds__(W * 32, 24 / W) k_pair_loop_probe(float* out, int reps, float dnu_f) {
@@ -1357,7 +1356,7 @@ __global__ void __launch_bounds__(W * 32, 24 / W) k_pair_loop_probe(float* out, 
   const float lanef = (float)lane;
   for (int r = 0; r < reps; r++) {
 #pragma unroll 1
-    for (int k = 0; k < 16; k++) cover_pair<false, false>(PT, k, lanef, dnu_f, nullptr, acc);
+    for (int k = 0; k < 16; k++) cover_pair<false>(PT, k, lanef, dnu_f, nullptr, acc);
   }
   float t = 0.0f;
 #pragma unroll
