@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 import oracle
-from rox_testutil import q_pair, to_device
+from rox_testutil import check_sigma, q_pair, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +103,29 @@ def _check(name, points, cutoff, L, j0, points_in_call, P):
     err = float((np.abs(got - ref) / ref).max())
     print("PARITY dense lists, %s: max rel err %.3e" % (name, err))
     assert err <= TOL, (name, err)
+
+
+# widest Lorentz half-width in units of 64 half-cells (beyond 1 a cell's moments are not used: the powers of
+# the poles would leave FP32's range)
+@pytest.mark.parametrize("wide", [0.2, 0.9, 0.999, 1.001, 1.5])
+def test_narrow_and_very_wide_lines_in_one_cell(wide):
+    """3,000 lines of 3e-4 to 1e-3 of that width, every 50th of the full width, in cells of 0.128 cm^-1; the
+    tolerance of test_gpu_wings.py."""
+    dnu, points, cutoff = 0.002, 2049, 100.0
+    half = 32 * dnu
+    rng = np.random.default_rng(7)
+    n = 3000
+    nu0 = np.sort(rng.uniform(1000.0 - cutoff, 1004.0 + cutoff, n))
+    gam = (wide * 64 * half) * np.where(np.arange(n) % 50 == 0, 1.0, rng.uniform(3e-4, 1e-3, n))
+    f = lambda v: np.full(n, v, np.float32)  # noqa: E731
+    L = {"convention": 0, "nu0": nu0, "s_or_a": np.exp(rng.uniform(np.log(1e-24), np.log(1e-20), n)).astype(np.float32),
+         "g_up": None, "e_lower": f(0.0), "gamma_ref": gam.astype(np.float32), "n_t": f(0.5)}
+    grid = (1000.0, dnu, points)
+    w = rs.CONFIGS[1]
+    Qt, Qr = q_pair(w, T)
+    ref = oracle.xsec_windowed(L, grid, 1.01325, T, Qt, Qr, MASS, cutoff)
+    ws = torch.empty(rox.rox_xsec_workspace_size(n, grid, 1), dtype=torch.uint8, device="cuda")
+    sigma = torch.empty((1, points), dtype=torch.float32, device="cuda")
+    rox.rox_xsec(to_device(L, torch), grid, 1.01325, T, Qt, Qr, MASS, cutoff, sigma, ws)
+    assert rox.rox_ws_status(ws)[0] == 0
+    check_sigma(sigma[0].double().cpu().numpy(), ref, rel_tol=1.5e-5, label="wide %g" % wide)
