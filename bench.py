@@ -18,6 +18,7 @@ the same workload on the host cores. Under torchrun (N > 1) every rank runs one 
 of the workload on its own GPU (the path has no exchange step).
 """
 import argparse
+import hashlib
 import json
 import math
 import os
@@ -34,12 +35,13 @@ import numpy as np  # noqa: E402
 
 import rox_synth as rs  # noqa: E402
 
-# Warp instructions of k_voigt per evaluation (a (line, point) pair inside the cutoff), and DRAM bytes per
-# evaluation: ncu counters of one launch (profiles/k_voigt_counters.md). An evaluation is the definition's
-# unit of work; the kernel forms most of them from per-cell moments and interpolation, so flops per
-# evaluation mean nothing and the kernel is measured against the warp schedulers' issue rate, its bound.
-VOIGT_INST = {"exomol": 2.3804e9 / 4.998e10, "large": 2.5837e10 / 1.98948e12}
-VOIGT_DRAM = {"exomol": 1.573e9 / 4.998e10}
+# Counters of one k_voigt launch (ncu; profiles/k_voigt_counters.md says how they were taken): warp
+# instructions, executed FP32 operations and DRAM bytes, with the launch's evaluations. An evaluation (a
+# (line, point) pair inside the cutoff) is the definition's unit of work; the kernel forms most of them from
+# per-cell moments and interpolation, so what it executes is counted, not derived from the evaluations. The
+# counters hold for the sources they were taken on, by digest, and are not reported for others.
+VOIGT_COUNTERS = os.path.join(ROOT, "profiles", "k_voigt_counters.json")
+VOIGT_SOURCES = ("rox_voigt.cu", "rox_lines.cuh", "rox_faddeeva.cuh", "rox_core_tables.h", "rox_internal.cuh")
 # DRAM bytes of one k_cia_grid launch on the CIA workload (ncu dram__bytes_read + write,
 # profiles/k_cia_grid_40T_2970001pts.md; part of the 950 MB output is still in L2 at the end)
 CIA_TRAFFIC_BYTES = 8.955e8
@@ -681,18 +683,52 @@ def loop_ceilings(dev_index, sms, out):
     return res
 
 
+def voigt_sources_digest():
+    h = hashlib.sha256()
+    for name in VOIGT_SOURCES:
+        with open(os.path.join(ROOT, "paper_2510_20870_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
+
+
+def voigt_counters(kind):
+    """The counters of workload `kind` per evaluation, or (None, why)."""
+    with open(VOIGT_COUNTERS) as f:
+        d = json.load(f)
+    if kind not in d["launches"]:
+        return None, "no counters taken on this workload"
+    if d["sources_sha256"] != voigt_sources_digest():
+        return None, "the kernel's sources changed since its counters were taken (profiles/k_voigt_counters.json)"
+    c = d["launches"][kind]
+    return {k: v / c["evaluations"] for k, v in c.items() if k != "evaluations"}, None
+
+
 def voigt_roofline(evals, kernel_ms, kind, sms, clocks, peaks=None):
     """The Voigt kernel (with the moments pass ahead of it) against the issue rate of the warp schedulers,
-    one instruction per clock each. kind: the workload whose instruction and byte counts apply, or None."""
+    one instruction per clock each, and (`fp32`) its executed FP32 operations against the FP32 peak. kind:
+    the workload whose counters apply, or None."""
     peak = sms * 4 * SM_MAX_MHZ * 1e6 / 1e12
-    inst, dram = VOIGT_INST.get(kind), VOIGT_DRAM.get(kind)
-    achieved = evals * inst / (kernel_ms * 1e-3) / 1e12 if inst else None
+    c, why = voigt_counters(kind)
+    c = c or {}
+
+    def rate(key):
+        return evals * c[key] / (kernel_ms * 1e-3) / 1e12 if key in c else None
+
+    achieved, flops = rate("warp_instructions"), rate("fp32_flops")
+    f_peak = sms * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
     roof = {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "T warp instructions/s",
-            "frac": achieved / peak if inst else None, "kernel": "k_voigt", "kernel_ms": kernel_ms,
+            "frac": achieved / peak if achieved else None, "kernel": "k_voigt", "kernel_ms": kernel_ms,
             "peak_basis": "%d SMs x 4 schedulers x %.0f MHz (max SM clock)" % (sms, SM_MAX_MHZ),
-            "traffic": dram * evals if dram else None, "warp_inst_per_eval": inst,
-            "note": "instructions and DRAM bytes per evaluation from ncu on one launch of this list, times the "
-                    "evaluations; most evaluations come from moments and interpolation, not one by one"}
+            "traffic": evals * c["dram_bytes"] if "dram_bytes" in c else None,
+            "warp_inst_per_eval": c.get("warp_instructions"),
+            "fp32": {"achieved": flops, "peak": f_peak, "unit": "TFLOP/s", "frac": flops / f_peak if flops else None,
+                     "peak_basis": "%d SMs x 128 FP32 lanes x 2 flop x %.0f MHz (max SM clock)" % (sms, SM_MAX_MHZ),
+                     "note": "executed FP32 operations (FMA 2), not evaluations times the operations of one"},
+            "note": why or "instructions, FP32 operations and DRAM bytes per evaluation from ncu on one launch of this "
+                           "list with these sources, times the evaluations; most evaluations come from moments and "
+                           "interpolation, not one by one"}
+    if peaks and peaks.get("measured_tflops") and flops:
+        roof["fp32"]["frac_of_measured"] = flops / peaks["measured_tflops"]
     if peaks and peaks.get("pair_loop_evals_s"):
         roof["pair_loop_evals_s"] = peaks["pair_loop_evals_s"]
         roof["vs_pair_loop"] = evals / (kernel_ms * 1e-3) / peaks["pair_loop_evals_s"]

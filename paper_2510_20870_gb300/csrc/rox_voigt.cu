@@ -28,7 +28,7 @@
 // 1e-7 of a line's value at the distances admitted: smooth_dmin).
 //
 // Every form but the slow zones' works per line and span, not per line and point: on the 1e7-line
-// ExoMol list the kernel took 16.0 ms with each line at each of its 5,001 points, 3.24 ms so. It is bound
+// ExoMol list the kernel took 16.0 ms with each line at each of its 5,001 points, 3.29 ms so. It is bound
 // by instruction issue and, as the code is long, by instruction fetch (4.2 of 9.2 stalled warps
 // per issue before the loops were kept short): a form that saves a few instructions with a second
 // copy of a loop costs more than it gives.
