@@ -9,7 +9,7 @@ rox_xsec_batch on each chunk in turn, the chunks after the first added into sigm
 (ROX_ACCUMULATE); each call computes strengths and widths, windows and span ranges, and runs the
 Voigt kernel. Metric: Voigt line-profile evaluations per second, one evaluation being a (line,
 grid point) pair inside the cutoff, counted exactly. (The 300-point batch case, 1e8 lines at
-15 P x 20 T, takes about a minute per step; it runs with --config 3.)
+15 P x 20 T, takes 12 s per step; it runs with --config 3.)
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl rox|reference] [--config 1..4]
 
