@@ -28,7 +28,7 @@
 // 1e-7 of a line's value at the distances admitted: smooth_dmin).
 //
 // Every form but the slow zones' works per line and span, not per line and point: on the 1e7-line
-// ExoMol list the kernel took 16.0 ms with each line at each of its 5,001 points, 3.29 ms so. It is bound
+// ExoMol list the kernel took 16.0 ms with each line at each of its 5,001 points, 3.27 ms so. It is bound
 // by instruction issue and, as the code is long, by instruction fetch (4.2 of 9.2 stalled warps
 // per issue before the loops were kept short): a form that saves a few instructions with a second
 // copy of a loop costs more than it gives.
@@ -783,7 +783,10 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   __shared__ __align__(16) float s_carry[W][2][ROX_CARRY];   // moments of the edge lines so far, per side
   __shared__ __align__(8) float s_zacc[W][ROX_SPAN];
   __shared__ float s_tot[W][ROX_SPAN];    // the span's sum over its parts
-  __shared__ float s_part[W][3][ROX_SPAN];  // a part's sum and its compensation; the compensation of s_tot
+  // a part's sum and its compensation, side by side: one 8-byte access each way a point (rows apart, the
+  // exomol list took 0.9% longer)
+  __shared__ __align__(8) float2 s_part[W][ROX_SPAN];
+  __shared__ float s_totc[W][ROX_SPAN];   // the compensation of s_tot
   __shared__ __align__(16) f32x2 s_cf[W][16];   // a zoned line's form coefficients
   __shared__ int s_status;
 
@@ -802,7 +805,8 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
   const float cheb = rox_cheb_x[lane];
   float* zacc = s_zacc[w];
   float* stot = s_tot[w];
-  float *part_tot = s_part[w][0] + lane, *part_cmp = s_part[w][1] + lane, *tot_cmp = s_part[w][2] + lane;   // [32 m]: this lane's points
+  float2* psum = s_part[w] + lane;        // [32 m]: this lane's points
+  float* tot_cmp = s_totc[w] + lane;
   f32x2* cbuf = s_cf[w];
   float* carry = s_carry[w][0];
   const float* cr = rox_core_r[lane & 15];
@@ -950,8 +954,8 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
     for (int p = p_first; p <= p_last; p++) {
       const int plo = 32 * (int)((long long)nbat * p / np);
       const int phi = min(nn, 32 * (int)((long long)nbat * (p + 1) / np));
-      // the part's total and its compensation: in shared memory (touched once in four batches),
-      // Chebyshev point in nsum, ncmp
+      // the part's total and its compensation: psum in shared memory (touched once in four batches), the
+      // Chebyshev point's in nsum, ncmp
       int ekL = 0, ekR = 0;             // edge lines: first point without its final sum, per side
       bool edgeL = false, edgeR = false;
       carry[lane] = 0.f;                // both sides' 2 x ROX_CARRY floats
@@ -959,8 +963,7 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
         acc[m] = 0.f;
-        part_tot[32 * m] = 0.f;
-        part_cmp[32 * m] = 0.f;
+        psum[32 * m] = make_float2(0.f, 0.f);
         zacc[32 * m + lane] = 0.f;
       }
 
@@ -1224,10 +1227,9 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
         if ((nb & 3) == 3 || b0 + 32 >= mhi) {
 #pragma unroll
           for (int m = 0; m < ROX_K; m++) {
-            float v = part_tot[32 * m], c = part_cmp[32 * m];
-            sum_add(v, c, acc[m] + zacc[32 * m + lane], kw);
-            part_tot[32 * m] = v;
-            part_cmp[32 * m] = c;
+            float2 v = psum[32 * m];
+            sum_add(v.x, v.y, acc[m] + zacc[32 * m + lane], kw);
+            psum[32 * m] = v;
             acc[m] = 0.f;
             zacc[32 * m + lane] = 0.f;
           }
@@ -1266,19 +1268,19 @@ __global__ void __launch_bounds__(W * 32, 20 / W) k_voigt(const __grid_constant_
       // fold in what the last batches and the edges left in zacc
 #pragma unroll
       for (int m = 0; m < ROX_K; m++) {
-        part_tot[32 * m] += zacc[32 * m + lane] - part_cmp[32 * m];
+        psum[32 * m].x += zacc[32 * m + lane] - psum[32 * m].y;
       }
       if (part >= 0) {           // a split item: this part's sum goes to the tail scratch
         float* dst = A.tail_part + (size_t)(slot0 + p) * ROX_PART_FLOATS;
 #pragma unroll
-        for (int m = 0; m < ROX_K; m++) __stcg(&dst[32 * m + lane], part_tot[32 * m]);
+        for (int m = 0; m < ROX_K; m++) __stcg(&dst[32 * m + lane], psum[32 * m].x);
         __stcg(&dst[ROX_SPAN + lane], nsum);
       } else {
         sum_add(ntot, ncmt, nsum, kw);
 #pragma unroll
         for (int m = 0; m < ROX_K; m++) {
           float v = p == 0 ? 0.f : stot[32 * m + lane], c = p == 0 ? 0.f : tot_cmp[32 * m];
-          sum_add(v, c, part_tot[32 * m], kw);
+          sum_add(v, c, psum[32 * m].x, kw);
           stot[32 * m + lane] = v;
           tot_cmp[32 * m] = c;
         }
