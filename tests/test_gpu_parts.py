@@ -1,6 +1,6 @@
 """How a short grid's lines are divided among the GPU's warps, where an average over the reach of the
 cutoff says little: 3,000 lines on 301 points. Cutoffs that all reach over the whole grid mean the
-same work, so the longer one may not take much longer (0.08 ms either way; in parts sized by the
+same work, so the longer one may not take much longer (0.20 and 0.24 ms; in parts sized by the
 average it took 2.7 times as long), and the sums agree with the oracle.
 
 Tolerance as in test_gpu_wings.py (1.5e-5); time: a factor of 1.6 between the fastest of 20 calls each."""
